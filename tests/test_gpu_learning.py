@@ -61,6 +61,12 @@ def test_ppo_clip_matches_oracle_and_is_deterministic(N, eps):
     assert abs(outs[0][2] - o_cf) <= (near + 0.5) / N
 
 
+# chunk and lane edges of the GAE kernel: 64-step chunks (a partial one comes first), 32 envs per CTA
+@pytest.mark.parametrize("M,B", [(63, 32), (64, 33), (65, 31), (129, 1), (300, 40)])
+def test_gae_chunk_edges(M, B):
+    test_gae_matches_oracle(M, B, 0.99, 0.95)
+
+
 def test_learning_entry_points_reject_bad_arguments():
     x = torch.zeros(4, device="cuda")
     p = x.data_ptr()
