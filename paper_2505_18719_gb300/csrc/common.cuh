@@ -221,21 +221,31 @@ inline cudaError_t injected_launch_error() {
 extern std::atomic<uint64_t> g_wait_limit_ns;
 constexpr uint64_t kDefaultWaitLimitNs = 1000000000ull;
 
+// `cluster` > 1: thread-block clusters of that many consecutive CTAs along x.
 template <typename... KArgs, typename... Args>
-inline cudaError_t launch_pdl(void (*kern)(KArgs...), dim3 grid, dim3 block, size_t smem,
-                              cudaStream_t stream, Args... args) {
+inline cudaError_t launch_pdl_cluster(void (*kern)(KArgs...), dim3 grid, dim3 block, size_t smem,
+                                      cudaStream_t stream, int cluster, Args... args) {
   if (const cudaError_t inj = injected_launch_error()) return inj;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = grid;
   cfg.blockDim = block;
   cfg.dynamicSmemBytes = smem;
   cfg.stream = stream;
-  cudaLaunchAttribute attr[1];
+  cudaLaunchAttribute attr[2];
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   attr[0].val.programmaticStreamSerializationAllowed = 1;
+  attr[1].id = cudaLaunchAttributeClusterDimension;
+  attr[1].val.clusterDim.x = static_cast<unsigned>(cluster);
+  attr[1].val.clusterDim.y = 1;
+  attr[1].val.clusterDim.z = 1;
   cfg.attrs = attr;
-  cfg.numAttrs = 1;
+  cfg.numAttrs = cluster > 1 ? 2 : 1;
   return cudaLaunchKernelEx(&cfg, kern, static_cast<KArgs>(args)...);
+}
+template <typename... KArgs, typename... Args>
+inline cudaError_t launch_pdl(void (*kern)(KArgs...), dim3 grid, dim3 block, size_t smem,
+                              cudaStream_t stream, Args... args) {
+  return launch_pdl_cluster(kern, grid, block, smem, stream, 1, args...);
 }
 
 // Raises a kernel's dynamic shared-memory limit on the current device.  Function attributes
@@ -243,15 +253,24 @@ inline cudaError_t launch_pdl(void (*kern)(KArgs...), dim3 grid, dim3 block, siz
 // one bit per device index < 64 (beyond that the call is repeated every time).  Host threads
 // racing here at worst both make the call.
 template <typename Kern>
-inline cudaError_t set_smem_limit(Kern kern, int bytes, std::atomic<uint64_t>& done) {
+inline cudaError_t set_attribute_once(Kern kern, cudaFuncAttribute attr, int value, std::atomic<uint64_t>& done) {
   int dev = 0;
   cudaError_t e = cudaGetDevice(&dev);
   if (e != cudaSuccess) return e;
   const uint64_t bit = (dev >= 0 && dev < 64) ? (1ull << dev) : 0ull;
   if (bit && (done.load(std::memory_order_acquire) & bit)) return cudaSuccess;
-  e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+  e = cudaFuncSetAttribute(kern, attr, value);
   if (e == cudaSuccess && bit) done.fetch_or(bit, std::memory_order_release);
   return e;
+}
+template <typename Kern>
+inline cudaError_t set_smem_limit(Kern kern, int bytes, std::atomic<uint64_t>& done) {
+  return set_attribute_once(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes, done);
+}
+// Clusters of up to 16 CTAs (above 8 a kernel has to opt in).
+template <typename Kern>
+inline cudaError_t allow_wide_clusters(Kern kern, std::atomic<uint64_t>& done) {
+  return set_attribute_once(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1, done);
 }
 
 // Makes `dev` current for the scope of one API call and gives the caller's device back on exit

@@ -4,8 +4,9 @@
 //  * GAE (Algorithm 1, "compute advantages"; §3.3): the reverse recursion over M steps,
 //    one lane per env;
 //  * the clipped PPO objective of Eq. 2 with action log-probs as the sum of the 7 token
-//    log-probs (Eq. 1): one CTA, a fixed-order reduction, so the result is deterministic.
+//    log-probs (Eq. 1): one cluster, a fixed-order reduction, so the result is deterministic.
 #include "misc.h"
+#include "ptx.cuh"
 
 namespace vla {
 
@@ -123,45 +124,136 @@ __global__ void __launch_bounds__(32 * kGaeWarps) gae_kernel(const float* r, con
   }
 }
 
-// One CTA of 1024 threads: thread j sums samples j, j + 1024, ... in order; then a fixed tree.
-__global__ void __launch_bounds__(1024) ppo_clip_kernel(const float* lp_new,
-                                                        const float* lp_old,
-                                                        const float* adv, int N, int A,
-                                                        float eps, float* __restrict__ objective,
-                                                        float* __restrict__ ratio,
-                                                        float* __restrict__ clip_frac) {
+// The clipped objective on one thread-block cluster: the samples go round-robin over its CTAs in
+// tiles of 512, each tile's log-probs staged through shared memory (cp.async, all but one stage in
+// flight; A floats per sample are then read at stride A), one sample per thread; the CTAs' sums meet in CTA
+// 0 over distributed shared memory in a fixed order, so no scratch memory is shared between
+// calls and repeated calls give identical results.  One CTA of 1024 threads walked all samples
+// before: 32768 x 7 took 41.3 us with cold caches (21.9 us a call back to back; one SM's share of bandwidth
+// and latency), now 7.6 (about 12, the caller's share included) on 16 CTAs; 1M samples x 7 took 1215 us,
+// now 111, the bandwidth of those 16 SMs.
+constexpr int kPpoTile = 512;   // samples per tile = threads
+constexpr int kPpoMaxA = 16;    // more tokens per sample are read in place (no staging)
+
+__device__ __forceinline__ void ppo_cp16(uint32_t dst, const void* src) {
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst), "l"(src) : "memory");
+}
+
+constexpr int kPpoStageBytes = 2 * kPpoTile * 4;  // per token of a sample
+
+template <int kPpoStages>
+__global__ void __launch_bounds__(kPpoTile) ppo_clip_kernel(const float* lp_new, const float* lp_old,
+                                                            const float* adv, int N, int A, int staged,
+                                                            float eps, float* __restrict__ objective,
+                                                            float* __restrict__ ratio,
+                                                            float* __restrict__ clip_frac) {
+  extern __shared__ __align__(16) float ppo_sm[];  // [stage][new, old][kPpoTile * A]
+  __shared__ float red[2][kPpoTile / 32];
+  __shared__ float2 cta_sum;
   pdl_launch_dependents();
   pdl_wait();
-  __shared__ float red[2][32];
+  const int n_cta = static_cast<int>(gridDim.x), rank = static_cast<int>(blockIdx.x);
+  const int tid = threadIdx.x;
+  const int tiles = (N + kPpoTile - 1) / kPpoTile;
+  const int plane = kPpoTile * A;
+  auto stage_load = [&](int tile, int st) {
+    if (tile < tiles) {
+      const size_t first = static_cast<size_t>(tile) * plane;  // a multiple of 512 floats
+      const int n = min(kPpoTile, N - tile * kPpoTile) * A;
+      float* dn = ppo_sm + static_cast<size_t>(st) * 2 * plane;
+      const uint32_t sn = static_cast<uint32_t>(__cvta_generic_to_shared(dn)), so = sn + plane * 4;
+      const int n4 = n >> 2;
+      for (int i = tid; i < n4; i += kPpoTile) {
+        ppo_cp16(sn + i * 16, lp_new + first + i * 4);
+        ppo_cp16(so + i * 16, lp_old + first + i * 4);
+      }
+      for (int i = (n4 << 2) + tid; i < n; i += kPpoTile) {  // the last 0-3 floats
+        dn[i] = lp_new[first + i];
+        dn[plane + i] = lp_old[first + i];
+      }
+    }
+    asm volatile("cp.async.commit_group;" ::: "memory");
+  };
   float acc = 0.f, clipped = 0.f;
-  for (int n = threadIdx.x; n < N; n += blockDim.x) {
-    float dl = 0.f;
-    for (int i = 0; i < A; ++i)
-      dl += lp_new[static_cast<size_t>(n) * A + i] - lp_old[static_cast<size_t>(n) * A + i];
-    const float rho = expf(dl);
-    const float a = adv[n];
-    const float rc = fminf(fmaxf(rho, 1.f - eps), 1.f + eps);
-    acc += fminf(rho * a, rc * a);
-    clipped += fabsf(rho - 1.f) > eps ? 1.f : 0.f;
-    if (ratio) ratio[n] = rho;
+  auto adv_of = [&](int tile) {
+    const int n = tile * kPpoTile + tid;
+    return tile < tiles && n < N ? adv[n] : 0.f;
+  };
+  float a = adv_of(rank);
+  if (staged)
+    for (int s = 0; s < kPpoStages - 1; ++s) stage_load(rank + s * n_cta, s);
+  int st = 0;
+  for (int tile = rank; tile < tiles; tile += n_cta) {
+    const int n = tile * kPpoTile + tid;
+    const float a_next = adv_of(tile + n_cta);  // in flight during this tile
+    const float *pn, *po;
+    if (staged) {
+      asm volatile("cp.async.wait_group %0;" ::"n"(kPpoStages - 2) : "memory");
+      __syncthreads();
+      stage_load(tile + (kPpoStages - 1) * n_cta, (st + kPpoStages - 1) % kPpoStages);
+      pn = ppo_sm + static_cast<size_t>(st) * 2 * plane + tid * A;
+      po = pn + plane;
+      st = (st + 1) % kPpoStages;
+    } else {
+      pn = lp_new + static_cast<size_t>(n) * A;
+      po = lp_old + static_cast<size_t>(n) * A;
+    }
+    if (n < N) {
+      float dl = 0.f;
+      if (staged && (A & 3) == 0) {  // 16-byte reads: at a stride of 4, 8 or 16 floats scalar ones conflict
+        for (int i = 0; i < A; i += 4) {
+          const float4 x = *reinterpret_cast<const float4*>(pn + i), y = *reinterpret_cast<const float4*>(po + i);
+          dl += x.x - y.x;
+          dl += x.y - y.y;
+          dl += x.z - y.z;
+          dl += x.w - y.w;
+        }
+      } else {
+  #pragma unroll 4
+        for (int i = 0; i < A; ++i) dl += pn[i] - po[i];
+      }
+      const float rho = expf(dl);
+      const float rc = fminf(fmaxf(rho, 1.f - eps), 1.f + eps);
+      acc += fminf(rho * a, rc * a);
+      clipped += fabsf(rho - 1.f) > eps ? 1.f : 0.f;
+      if (ratio) ratio[n] = rho;
+    }
+    a = a_next;
   }
   acc = warp_sum(acc);
   clipped = warp_sum(clipped);
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int warp = tid >> 5, lane = tid & 31;
   if (lane == 0) {
     red[0][warp] = acc;
     red[1][warp] = clipped;
   }
   __syncthreads();
-  if (threadIdx.x == 0) {
+  if (tid == 0) {
     float s = 0.f, c = 0.f;
-    for (int i = 0; i < static_cast<int>(blockDim.x >> 5); ++i) {
+    for (int i = 0; i < kPpoTile / 32; ++i) {
       s += red[0][i];
       c += red[1][i];
     }
-    objective[0] = s / static_cast<float>(N);
-    if (clip_frac) clip_frac[0] = c / static_cast<float>(N);
+    cta_sum = make_float2(s, c);
   }
+  if (n_cta > 1) cluster_sync();
+  if (rank == 0 && tid < 32) {
+    float2 x = make_float2(0.f, 0.f);
+    if (lane < n_cta) {
+      if (lane == 0) {
+        x = cta_sum;
+      } else {
+        const uint32_t at = mapa_shared(smem_u32(&cta_sum), lane);
+        asm volatile("ld.shared::cluster.v2.f32 {%0, %1}, [%2];" : "=f"(x.x), "=f"(x.y) : "r"(at) : "memory");
+      }
+    }
+    const float s = warp_sum(x.x), c = warp_sum(x.y);
+    if (lane == 0) {
+      objective[0] = s / static_cast<float>(N);
+      if (clip_frac) clip_frac[0] = c / static_cast<float>(N);
+    }
+  }
+  if (n_cta > 1) cluster_sync();  // the other CTAs' sums stay readable until CTA 0 has them
 }
 
 }  // namespace
@@ -188,8 +280,22 @@ int gae_launch(const float* r, const float* v, const float* done, int M, int B, 
 int ppo_clip_launch(const float* lp_new, const float* lp_old, const float* adv, int N, int A, float eps,
                     float* objective, float* ratio, float* clip_frac, cudaStream_t s) {
   if (N <= 0) return VLA_ERR_ARG;
-  VLA_CUDA_TRY(launch_pdl(ppo_clip_kernel, dim3(1), dim3(1024), 0, s, lp_new, lp_old, adv, N, A, eps, objective,
-                          ratio, clip_frac));
+  // one tile per CTA up to 16 CTAs (the non-portable cluster maximum); the staging needs 16-byte
+  // aligned log-probs
+  const int tiles = (N + kPpoTile - 1) / kPpoTile;
+  const int n_cta = tiles <= 1 ? 1 : tiles <= 2 ? 2 : tiles <= 4 ? 4 : tiles <= 8 ? 8 : 16;
+  const bool staged = A <= kPpoMaxA && !(reinterpret_cast<uintptr_t>(lp_new) & 15) &&
+                      !(reinterpret_cast<uintptr_t>(lp_old) & 15);
+  static std::atomic<uint64_t> smem_done[2] = {}, cluster_done[2] = {};
+  auto go = [&](auto kern, int stages, int max_a, int which) -> cudaError_t {
+    const int smem = staged ? stages * kPpoStageBytes * A : 0;
+    if (const cudaError_t e = set_smem_limit(kern, stages * kPpoStageBytes * max_a, smem_done[which])) return e;
+    if (const cudaError_t e = allow_wide_clusters(kern, cluster_done[which])) return e;
+    return launch_pdl_cluster(kern, dim3(n_cta), dim3(kPpoTile), smem, s, n_cta, lp_new, lp_old, adv, N, A,
+                              staged ? 1 : 0, eps, objective, ratio, clip_frac);
+  };
+  // as many stages as 192 KB hold
+  VLA_CUDA_TRY(A <= 8 ? go(ppo_clip_kernel<6>, 6, 8, 0) : go(ppo_clip_kernel<3>, 3, kPpoMaxA, 1));
   note_launch();
   VLA_CUDA_TRY(cudaGetLastError());
   return VLA_OK;

@@ -67,6 +67,30 @@ def test_gae_chunk_edges(M, B):
     test_gae_matches_oracle(M, B, 0.99, 0.95)
 
 
+# tile and cluster edges of the PPO kernel (512-sample tiles on 1, 2, 4, 8 or 16 CTAs, then round-robin)
+# and its three ways to read a sample: staged scalars, staged float4 (A % 4 == 0), in place (A > 16 or
+# log-probs off the 16-byte boundary)
+@pytest.mark.parametrize("N,A,offset", [(511, 1, 0), (513, 4, 0), (1024, 16, 0), (1537, 17, 0), (4097, 8, 0),
+                                        (8193, 7, 0), (25000, 6, 0), (2000, 7, 1)])
+def test_ppo_clip_tile_edges(N, A, offset):
+    lp_old = torch.cat([torch.zeros(offset), (-I.uniform_f32((N, A), 300 + N, 1) * 6.0).view(-1)])
+    d = (I.uniform_f32((N, A), 300 + N, 2) - 0.5) * 0.12
+    lp_new = torch.cat([torch.zeros(offset), lp_old[offset:] + d.view(-1)])
+    adv = I.normal_bf16((N,), 300 + N, 3, 1.0).float()
+    gn, go, ga = lp_new.cuda(), lp_old.cuda(), adv.cuda()
+    obj, cf, rho = (torch.full((k,), float("nan"), device="cuda") for k in (1, 1, N))
+    assert V.vla_ppo_clip(gn.data_ptr() + 4 * offset, go.data_ptr() + 4 * offset, ga.data_ptr(), N, A, 0.2,
+                          obj.data_ptr(), rho.data_ptr(), cf.data_ptr(), 0) == 0
+    torch.cuda.synchronize()
+    o_obj, o_rho, o_cf = O.ppo_clip_objective(lp_new[offset:].view(N, A).double(), lp_old[offset:].view(N, A).double(),
+                                              adv.double(), 0.2)
+    # A fp32 differences of values up to 6 (each within 2^-22) under an exponential of magnitude ~1
+    assert float((rho.cpu().double() - o_rho).abs().max()) < A * 2.0 ** -20
+    assert abs(obj.item() - o_obj) < A * 2.0 ** -20
+    near = int(((o_rho - 1.0).abs() - 0.2).abs().lt(1e-5).sum())
+    assert abs(cf.item() - o_cf) <= (near + 0.5) / N
+
+
 def test_learning_entry_points_reject_bad_arguments():
     x = torch.zeros(4, device="cuda")
     p = x.data_ptr()
