@@ -146,7 +146,6 @@ struct vla_handle {
   size_t ws_bytes = 0;
   float* h_last = nullptr;
   float* head_in = nullptr;
-  float* head_z = nullptr;  // action-bin logits [B * A, 256]
   float* head_entropy = nullptr;  // entropy of each action token's distribution [B, A]
   bool entropy_valid = false;     // set by decode / score, cleared by prefill / reset
   float* q_last = nullptr;  // last layer of a prefill: queries of each env's final row [B, d]
@@ -596,7 +595,6 @@ int vla_create(const vla_config* cfg, const vla_weights* w, void* cuda_stream, v
             alloc(reinterpret_cast<void**>(&h->ws), ws) &&
             alloc(reinterpret_cast<void**>(&h->h_last), static_cast<size_t>(B) * d * sizeof(float)) &&
             alloc(reinterpret_cast<void**>(&h->head_in), static_cast<size_t>(B) * A * d * sizeof(float)) &&
-            alloc(reinterpret_cast<void**>(&h->head_z), static_cast<size_t>(B) * A * 256 * sizeof(float)) &&
             alloc(reinterpret_cast<void**>(&h->head_entropy), static_cast<size_t>(B) * A * sizeof(float)) &&
             alloc(reinterpret_cast<void**>(&h->q_last), static_cast<size_t>(B) * d * sizeof(float)) &&
             alloc(reinterpret_cast<void**>(&h->ss_part), static_cast<size_t>(d / 128 + 1) * T * sizeof(float)) &&
@@ -789,7 +787,6 @@ int vla_decode_actions(vla_handle* h, const float* uniforms, float temperature, 
   for (int b = 0; b < B; ++b) max_len_p = std::max(max_len_p, h->len_prefill[b]);
 
   HeadArgs ha;
-  ha.z = h->head_z;
   ha.entropy_out = h->head_entropy;
   ha.B = B;
   ha.n_pos = 1;
@@ -890,7 +887,6 @@ int vla_score_actions(vla_handle* h, const int32_t* tokens, float temperature, f
     return fail(h, rc, t_err);
 
   HeadArgs ha;
-  ha.z = h->head_z;
   ha.entropy_out = h->head_entropy;
   ha.h = h->head_in;
   ha.ldh = d;
@@ -1029,7 +1025,7 @@ void vla_destroy(vla_handle* h) {
   if (!h) return;
   DeviceGuard dev_guard(h->dev);  // best effort: the handle is freed whatever happens
   cudaStreamSynchronize(h->stream);
-  void* bufs[] = {h->kv, h->kv_res, h->h, h->y, h->q, h->ao, h->u, h->ws, h->h_last, h->head_in, h->head_z, h->head_entropy, h->q_last, h->ss_part, h->last_rows, h->rope,
+  void* bufs[] = {h->kv, h->kv_res, h->h, h->y, h->q, h->ao, h->u, h->ws, h->h_last, h->head_in, h->head_entropy, h->q_last, h->ss_part, h->last_rows, h->rope,
                   h->rows, h->tiles, h->sidx, h->didx, h->fed, h->pending, h->status, h->part_o,
                   h->part_ml, h->attn_tickets, h->w16, h->w16_range};
   for (void* p : bufs)
@@ -1215,7 +1211,6 @@ int vla_op_action_head(const float* hs, int ldh, int B, int d, const void* final
       !finite_nonneg(temperature) || (temperature > 0.f && !uniforms))
     return set_err(nullptr, VLA_ERR_ARG, "vla_op_action_head: bad argument");
   HeadArgs ha;
-  ha.z = logits_out;
   ha.h = hs;
   ha.ldh = ldh;
   ha.B = B;
