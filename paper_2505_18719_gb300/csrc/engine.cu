@@ -345,6 +345,28 @@ int run_gemm(vla_handle* h, int cls, const bf16* A, size_t a_plane, int lda, con
   return VLA_OK;
 }
 
+// Keys per decode-attention CTA.  A CTA reads 16 keys at a time and pays about 1.3 us per step, so a
+// call with few (env, head) pairs is bound by the length of that chain, not by bandwidth: its ranges
+// are cut until about kDecodeCtas CTAs share the work, down to 32 keys (two steps; shorter ranges pay
+// more for the merge than they save).  One layer of 32 heads at 290 positions, ranges of 320 keys and
+// of this rule: 1 env 36.2 -> 11.5 us, 4 envs 36.0 -> 13.7, 16 envs 39.8 -> 26.5, 32 envs 48.9 ->
+// 44.2; from 64 envs on one range per 320 keys is as fast as any.
+constexpr int kDecodeCtas = 1536;
+constexpr int kDecodeMinKeys = 32;
+int decode_attn_keys(int n_rows, int H, int max_ctx, int max_keys) {
+  const int pairs = n_rows * H;
+  const int by_len = (max_ctx + max_keys - 1) / max_keys;
+  const int by_fill = std::min((kDecodeCtas + pairs / 2) / pairs, (max_ctx + kDecodeMinKeys - 1) / kDecodeMinKeys);
+  const int S = std::max(1, std::max(by_len, by_fill));
+  return std::max(16, ((max_ctx + S - 1) / S + 15) / 16 * 16);
+}
+// Partial-output slots (rows x heads x ranges) that decode_attn_keys can ask for.
+size_t decode_attn_slots(int max_rows, int H, int capacity, int max_keys) {
+  const size_t pairs = static_cast<size_t>(max_rows) * H;
+  const size_t by_len = pairs * ((capacity + max_keys - 1) / max_keys);
+  return std::max(by_len, static_cast<size_t>(kDecodeCtas) + pairs);
+}
+
 // Rows whose last-layer output is needed (a prefill only feeds the head with each env's
 // final row): idx [n] into the chunk's rows, rows [n] their RowInfo, max_ctx = longest context.
 struct LastRows {
@@ -398,14 +420,14 @@ int forward_layers(vla_handle* h, int M, const RowInfo* rows_dev, bool decode, i
       prof_end(h, ev, VLA_KCLASS_OTHER, 0, 16.0 * last->n * d);
       ev = prof_begin(h, VLA_KCLASS_ATTN_DECODE);
       rc = attn_decode_launch(h->q_last, h->ao, h->ao + pd, last->rows, last->n, last->max_ctx, h->kvl, l, H, hd,
-                              h->attn_chunk, h->part_o, h->part_ml, h->attn_tickets, h->stream, h->fp16);
+                              decode_attn_keys(last->n, H, last->max_ctx, h->attn_chunk), h->part_o, h->part_ml, h->attn_tickets, h->stream, h->fp16);
       prof_end(h, ev, VLA_KCLASS_ATTN_DECODE, 0, 0);
       Mr = last->n;
       resid = h->h_last;
     } else if (decode) {
       ev = prof_begin(h, VLA_KCLASS_ATTN_DECODE);
       rc = attn_decode_launch(h->q, h->ao, h->ao + pd, rows_dev, M, max_ctx, h->kvl, l, H, hd,
-                              h->attn_chunk, h->part_o, h->part_ml, h->attn_tickets, h->stream, h->fp16);
+                              decode_attn_keys(M, H, max_ctx, h->attn_chunk), h->part_o, h->part_ml, h->attn_tickets, h->stream, h->fp16);
       prof_end(h, ev, VLA_KCLASS_ATTN_DECODE, 0, 0);
     } else {
       ev = prof_begin(h, VLA_KCLASS_ATTN_PREFILL);
@@ -577,7 +599,7 @@ int vla_create(const vla_config* cfg, const vla_weights* w, void* cuda_stream, v
     }
   }
   h->ws_bytes = ws;
-  const int max_S = (c.kv_capacity + h->attn_chunk - 1) / h->attn_chunk;
+  const size_t attn_slots = decode_attn_slots(B, c.n_heads, c.kv_capacity, h->attn_chunk);
   h->max_tiles = h->max_tokens / 64 + B + 1;
   const size_t T = h->max_tokens;
 
@@ -607,8 +629,8 @@ int vla_create(const vla_config* cfg, const vla_weights* w, void* cuda_stream, v
             alloc(reinterpret_cast<void**>(&h->fed), static_cast<size_t>(B) * A * sizeof(int)) &&
             alloc(reinterpret_cast<void**>(&h->pending), static_cast<size_t>(B) * sizeof(int)) &&
             alloc(reinterpret_cast<void**>(&h->status), sizeof(uint32_t)) &&
-            alloc(reinterpret_cast<void**>(&h->part_o), static_cast<size_t>(B) * c.n_heads * max_S * c.head_dim * sizeof(float)) &&
-            alloc(reinterpret_cast<void**>(&h->part_ml), static_cast<size_t>(B) * c.n_heads * max_S * sizeof(float2)) &&
+            alloc(reinterpret_cast<void**>(&h->part_o), attn_slots * c.head_dim * sizeof(float)) &&
+            alloc(reinterpret_cast<void**>(&h->part_ml), attn_slots * sizeof(float2)) &&
             alloc(reinterpret_cast<void**>(&h->attn_tickets), static_cast<size_t>(B) * c.n_heads * sizeof(int)) &&
             alloc(reinterpret_cast<void**>(&h->w16), w16_elems(c) * sizeof(f16)) &&
             alloc(reinterpret_cast<void**>(&h->w16_range), sizeof(int)) &&
