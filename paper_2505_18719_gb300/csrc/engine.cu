@@ -261,10 +261,11 @@ struct NextGemm {
   int N, K, epi;
 };
 
-// epi.norm_w set (a residual GEMM followed by an RMSNorm into h->y): when this GEMM and `next`
-// both run as unsplit tile GEMMs, y is written unnormalised with per-tile sums of squares and
-// `next` applies the row scale in its epilogue; otherwise the norm is exact here (fused into
-// the weight-streaming reduction, or its own kernel).
+// epi.norm_w set (a residual GEMM followed by an RMSNorm into h->y): when this GEMM and `next` both
+// run as unsplit tile GEMMs, y is written unnormalised with per-tile sums of squares and `next`
+// applies the row scale in its epilogue; otherwise the norm is exact here: fused into the
+// weight-streaming reduction, or its own kernel (after the cluster GEMM one that has the rows' sums
+// of squares already).
 int run_gemm(vla_handle* h, int cls, const bf16* A, size_t a_plane, int lda, const bf16* W, int ldw,
              int M, int N, int K, EpiArgs epi, const NextGemm* next = nullptr) {
   const Plan pl = plan_gemm(M, N, K, epi.kind, h->cfg.d_model, h->num_sms);
@@ -300,20 +301,15 @@ int run_gemm(vla_handle* h, int cls, const bf16* A, size_t a_plane, int lda, con
                                (epi.kind == EPI_SWIGLU ? (N / 2 + 127) / 128 : (N + 255) / 256);
     g.pair = pair_tiles >= h->num_sms / 2;
   }
-  // A following RMSNorm is fused into the weight-streaming GEMM's reduction; after a tile GEMM
-  // it is deferred to the consuming tile GEMM when both run unsplit, else its own kernel.
   const EpiArgs norm = epi;
   bool defer_norm = false;
   if (!stream_k && norm.norm_w && next && g.splits == 1 && M > 128 && N % 128 == 0) {
     const Plan pn = plan_gemm(M, next->N, next->K, next->epi, h->cfg.d_model, h->num_sms);
     defer_norm = pn.splits == 1;
   }
-  if (!stream_k) {
-    if (defer_norm)
-      g.epi.ss_out = h->ss_part;
-    else
-      g.epi.norm_w = nullptr;
-  }
+  const bool fused_norm = stream_k && gemv_fuses_norm(M);
+  if (defer_norm || (stream_k && norm.norm_w && !fused_norm)) g.epi.ss_out = h->ss_part;
+  if (!defer_norm && !fused_norm) g.epi.norm_w = nullptr;
   // the consumer of a deferred norm: y is unnormalised, scale its rows here
   const bool consume = (A == h->y) && h->y_deferred && (epi.kind == EPI_QKV || epi.kind == EPI_SWIGLU);
   if (consume) {
@@ -335,7 +331,13 @@ int run_gemm(vla_handle* h, int cls, const bf16* A, size_t a_plane, int lda, con
     h->y_deferred = true;
     h->y_ss_tiles = (N + g.block_n - 1) / g.block_n;
   }
-  if (!stream_k && norm.norm_w && !defer_norm) {
+  if (stream_k && norm.norm_w && !fused_norm) {
+    ev = prof_begin(h, VLA_KCLASS_OTHER);
+    rc = norm_scale_launch(norm.resid, norm.ldr, norm.norm_w, h->ss_part, N / 128, M, N, norm.norm_eps, norm.norm_hi,
+                           norm.norm_lo, h->stream, h->fp16, h->status);
+    prof_end(h, ev, VLA_KCLASS_OTHER, 0, 8.0 * M * N);
+    if (rc) return fail(h, rc, t_err);
+  } else if (norm.norm_w && !defer_norm && !fused_norm) {
     ev = prof_begin(h, VLA_KCLASS_OTHER);
     rc = rmsnorm_launch(norm.resid, norm.ldr, norm.norm_w, M, N, norm.norm_eps, norm.norm_hi, norm.norm_lo,
                         h->stream, h->fp16, h->status);
@@ -376,7 +378,12 @@ struct LastRows {
   int max_ctx = 0;
 };
 
-// All decoder layers over M rows already assembled in h->h (Llama-2 layer, §3.1).
+// The RMSNorm of the first layer, applied as the rows are assembled.
+FirstNorm first_norm(const vla_handle* h) {
+  return {h->attn_norm[0], h->cfg.rms_eps, h->y, h->y + static_cast<size_t>(h->max_tokens) * h->cfg.d_model, h->fp16};
+}
+
+// All decoder layers over M rows assembled in h->h, their RMSNorm in h->y (Llama-2 layer, §3.1).
 // decode == true: one query per env row (rows[b] gives env and position), split-K attention.
 // Otherwise n_tiles attention tiles in h->tiles, the largest of tile_rows rows.
 // last != nullptr: the last layer computes q|k|v (the KV cache) for all M rows but attention,
@@ -389,13 +396,9 @@ int forward_layers(vla_handle* h, int M, const RowInfo* rows_dev, bool decode, i
   const size_t pd = static_cast<size_t>(h->max_tokens) * d;   // hi -> lo plane offsets
   const size_t pf = static_cast<size_t>(h->max_tokens) * F;
   int rc;
-  // the first layer's attention RMSNorm; every later RMSNorm follows a residual add
+  // the rows' first RMSNorm came with their assembly; every later one follows a residual add
   h->y_deferred = false;
-  int ev = prof_begin(h, VLA_KCLASS_OTHER);
-  if ((rc = rmsnorm_launch(h->h, d, h->attn_norm[0], M, d, c.rms_eps, h->y, h->y + pd, h->stream, h->fp16,
-                           h->status)))
-    return fail(h, rc, t_err);
-  prof_end(h, ev, VLA_KCLASS_OTHER, 0, 6.0 * M * d);
+  int ev;
   for (int l = 0; l < c.n_layers; ++l) {
 
     EpiArgs e;
@@ -583,7 +586,7 @@ int vla_create(const vla_config* cfg, const vla_weights* w, void* cuda_stream, v
 
   // split-K workspace: worst case over the decode / score projection shapes
   size_t ws = 0;
-  std::vector<int> Ms = {B, (A - 1) * B};
+  std::vector<int> Ms = {B, (A - 1) * B, std::min(128, h->max_tokens)};
   for (int M = 128; M <= h->max_tokens; M += 128) Ms.push_back(M);
   for (int M : Ms) {
     if (M < 1 || M > h->max_tokens) continue;
@@ -760,7 +763,7 @@ int vla_prefill(vla_handle* h, int batch, const void* visual, int n_visual, cons
 
   int ev = prof_begin(h, VLA_KCLASS_OTHER);
   rc = assemble_launch(h->rows, static_cast<int>(total), static_cast<const bf16*>(visual), token_ids,
-                       h->pending, h->embed, c.d_model, c.vocab, h->h, h->status, h->stream);
+                       h->pending, h->embed, c.d_model, c.vocab, h->h, first_norm(h), h->status, h->stream);
   prof_end(h, ev, VLA_KCLASS_OTHER, 0, 6.0 * total * c.d_model);
   if (rc) return fail(h, rc, t_err);
   // the last layer runs past q|k|v only for each env's final row, straight into h_last
@@ -834,7 +837,7 @@ int vla_decode_actions(vla_handle* h, const float* uniforms, float temperature, 
     if (i > 0) {
       const RowInfo* rows_i = h->rows + static_cast<size_t>(i - 1) * B;
       int ev = prof_begin(h, VLA_KCLASS_OTHER);
-      rc = assemble_launch(rows_i, B, nullptr, nullptr, h->fed, h->embed, d, c.vocab, h->h, h->status, h->stream);
+      rc = assemble_launch(rows_i, B, nullptr, nullptr, h->fed, h->embed, d, c.vocab, h->h, first_norm(h), h->status, h->stream);
       prof_end(h, ev, VLA_KCLASS_OTHER, 0, 6.0 * B * d);
       if (rc) return fail(h, rc, t_err);
       if ((rc = forward_layers(h, B, rows_i, true, 0, 0, max_len_p + i))) return rc;
@@ -896,7 +899,7 @@ int vla_score_actions(vla_handle* h, const int32_t* tokens, float temperature, f
 
   if (M > 0) {
     int ev = prof_begin(h, VLA_KCLASS_OTHER);
-    rc = assemble_launch(h->rows, M, nullptr, nullptr, tokens, h->embed, d, c.vocab, h->h, h->status, h->stream);
+    rc = assemble_launch(h->rows, M, nullptr, nullptr, tokens, h->embed, d, c.vocab, h->h, first_norm(h), h->status, h->stream);
     prof_end(h, ev, VLA_KCLASS_OTHER, 0, 6.0 * M * d);
     if (rc) return fail(h, rc, t_err);
     if ((rc = forward_layers(h, M, h->rows, false, n_tiles, n, 0))) return rc;
@@ -1160,6 +1163,8 @@ int op_gemm_decode(const std::string& name, bool fp16, const void* A, const void
                    void* cuda_stream) {
   if (!A || !A_lo || !W || !C || M < 1 || M > 128 || N < 1 || K < 1 || ldc < N || !workspace)
     return set_err(nullptr, VLA_ERR_ARG, name + ": bad argument");
+  if (workspace_bytes < gemv_workspace_bytes(M, N, K, query_num_sms()) || (reinterpret_cast<uintptr_t>(workspace) & 15))
+    return set_err(nullptr, VLA_ERR_ARG, name + ": unsupported arguments or workspace too small");
   GemmArgs g;
   g.A = static_cast<const bf16*>(A);
   g.A_lo = static_cast<const bf16*>(A_lo);

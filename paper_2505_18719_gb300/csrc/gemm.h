@@ -33,9 +33,9 @@ struct EpiArgs {
   int layer = 0;
   const float2* rope = nullptr;   // EPI_QKV: [cap][hd/2] (cos, sin)
   int d = 0, hd = 0;
-  // EPI_RESID of the weight-streaming GEMM only: after the residual add, the row's RMSNorm
-  // with weight norm_w (bf16, N elements) is written as the operand pair norm_hi / norm_lo
-  // [m * ldn + n] in the same kernel.  The tile GEMM rejects it.
+  // EPI_RESID: the RMSNorm that follows, weight norm_w (bf16, N elements), output pair norm_hi /
+  // norm_lo [m * ldn + n].  The weight-streaming GEMM writes it when gemv_fuses_norm(M), the tile
+  // GEMMs take it in the deferred form below.
   const bf16* norm_w = nullptr;
   float norm_eps = 0.f;
   bf16* norm_hi = nullptr;
@@ -44,7 +44,8 @@ struct EpiArgs {
   // EPI_RESID of the tile GEMMs with norm_w set and ss_out != nullptr: the row of the updated
   // residual times norm_w goes to norm_hi / norm_lo NOT normalised, and the sum of squares of
   // the row's columns in each BN-wide tile to ss_out[n_tile * M + m]; the consuming GEMM
-  // applies the normalisation (row_ss).
+  // applies the normalisation (row_ss).  EPI_RESID of the weight-streaming GEMM when
+  // it does not fuse the norm: only the sums of squares, one per 128 columns.
   float* ss_out = nullptr;
   // EPI_QKV / EPI_SWIGLU of the tile GEMMs: row_ss != nullptr scales each output row by
   // rsqrt(sum_{t < row_ss_n} row_ss[t * M + m] / row_d + row_eps) first (the RMSNorm of an
@@ -83,9 +84,11 @@ size_t gemm_workspace_bytes(const GemmArgs& a);
 int gemm_launch(const GemmArgs& a, cudaStream_t stream, int num_sms, GemmCost* cost);
 
 // Weight-streaming (decode) GEMM for M <= 128 rows with a split A (A_lo required; operand
-// format epi.fp16): swap-AB tcgen05 MMAs, stream-K over the weight tiles, partials in
-// `workspace` (gemv_workspace_bytes), then the epilogue of `a.epi` in a fixed-order reduction
-// (EPI_RESID with norm_w set: fused with the following RMSNorm).
+// format epi.fp16): swap-AB tcgen05 MMAs.  Up to 32 rows K is split over a cluster whose partial
+// sums meet in shared memory; above, stream-K over the weight tiles with partials in `workspace`
+// (gemv_workspace_bytes) and the epilogue in a fixed-order reduction, with a following RMSNorm
+// (EPI_RESID, norm_w) in the same kernel.
+bool gemv_fuses_norm(int M);
 size_t gemv_workspace_bytes(int M, int N, int K, int num_sms);
 
 // 2-D tensor map of 2-byte elements (bf16, or fp16 when fp16) over [rows, cols] (row stride ld

@@ -1121,9 +1121,9 @@ __global__ void __maxnreg__(48) stream_reduce_resid_norm_kernel(StreamSrc src, i
   report_saturation(status, sat);
 }
 
-// ----------------------------------------------------------------------------- decode GEMM
-// Weight-streaming GEMM for decode-sized batches (M <= 128 rows of activations), where the
-// projections are bound by reading the weights from HBM once.
+// ----------------------------------------------------------------------------- decode GEMM, stream-K
+// Weight-streaming GEMM for 33 to 128 rows of activations, where the projections are bound by
+// reading the weights from HBM once.  (Up to 32 rows: the cluster kernel below.)
 //  * swap-AB: the 128-row weight tile is the MMA's A operand and the batch (BNX rows, the
 //    activation pair hi / lo) is its N, so no MMA row is wasted on padding and the
 //    activation tiles cost smem fill BNX/128 of the weights';
@@ -1131,7 +1131,7 @@ __global__ void __maxnreg__(48) stream_reduce_resid_norm_kernel(StreamSrc src, i
 //    one per CTA, so all SMs stream the same number of weight bytes; each run of one tile
 //    inside a range accumulates in TMEM and is written as one fp32 partial (StreamSrc);
 //  * weights are loaded evict-first, activations evict-last.
-struct GemvParams {
+struct StreamParams {
   int N, K;
   int tiles, kbt;       // 256-row tiles of W, 64-wide k-blocks per tile
   int per_cta, max_seg; // stream-K range length and partial slots per CTA
@@ -1145,8 +1145,8 @@ struct GemvParams {
 // activation fill per weight byte is BNX/256 * 2 and 4 stages keep 128 KB of weights in flight.
 template <int BNX, int STAGES>
 __global__ void __launch_bounds__(kThreads, 1)
-    gemv_tc_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ CUtensorMap tmX,
-                   const __grid_constant__ CUtensorMap tmX2, const GemvParams p) {
+    gemv_stream_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ CUtensorMap tmX,
+                   const __grid_constant__ CUtensorMap tmX2, const StreamParams p) {
   constexpr int TR = 256, NH = TR / 128;
   constexpr int W_HALF = 128 * BK * 2;
   constexpr int W_BYTES = NH * W_HALF;
@@ -1350,6 +1350,403 @@ __global__ void __launch_bounds__(kThreads, 1)
   }
 }
 
+// ----------------------------------------------------------------------------- decode GEMM, clusters
+// Weight-streaming GEMM for up to 32 rows, bound by reading the weights once and, for small models,
+// by the chain of launches and reductions around that: no partial sum goes through global memory and
+// no reduction kernel follows.  Chained launches of 16 rows, against the stream-K form with its
+// reductions: q|k|v 12288 x 4096 21.2 -> 19.5 us, o 15.3 -> 9.9, gate|up 34.3 -> 33.4, down 23.2 -> 18.4
+// (o and down without the norm that the reduction fused, 4.6 - 7 us in the engine); gate|up of
+// d = 512 7.1 -> 6.8 us.  At 64 rows its exchange costs 5 - 8 us a launch and the stream-K form wins
+// (one 7B decode layer 192 us against 202).
+//  * swap-AB: the weight tile (TR rows) is the MMA's A operand and the batch (BNX rows, the
+//    activation pair hi / lo) is its N, so no MMA row is wasted on padding and the
+//    activation tiles cost smem fill 2 * BNX / TR of the weights';
+//  * a cluster of C CTAs owns one tile and splits K: each CTA sends the others the batch rows that
+//    they finish (bulk copies of its fp32 partial tile into their shared memory), sums its own
+//    rows in rank order and applies the layer's epilogue (RoPE + KV-cache write, SwiGLU, residual
+//    add).  No partial goes through global memory and no reduction kernel follows;
+//  * at most 113 KB of shared memory, so two CTAs share an
+//    SM: the next projection's CTAs become resident while this one's finish (programmatic
+//    dependent launch) and request their first weight stages before they wait;
+//  * weights are loaded evict-first, activations evict-last.
+struct ClusterParams {
+  int M, N, K, kbt;     // kbt: 64-wide k-blocks
+  EpiArgs epi;
+  uint64_t wait_limit;  // ns per bounded mbarrier wait
+};
+
+// Copies `bytes` of this CTA's shared memory to the cluster address dst, completing on the mbarrier
+// bar (cluster address) of the same CTA as dst.
+__device__ __forceinline__ void bulk_copy_cluster(uint32_t dst, uint32_t src, uint32_t bytes, uint32_t bar) {
+  asm volatile("cp.async.bulk.shared::cluster.shared::cta.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(dst),
+               "r"(src), "r"(bytes), "r"(bar)
+               : "memory");
+}
+
+// A CTA's view of the cluster's partial tiles after the exchange: rows m0 .. m0 + mn - 1 of the batch
+// are its own to finish, its own partial in `part` [batch row][TR], the others' in `recv`
+// [other rank][ml rows][TR].
+template <int TR>
+struct TileSums {
+  const float* part;
+  const float* recv;
+  int C, rank, ml, m0, mn;
+  // columns r .. r + 3 of own row i, summed over the ranks in rank order
+  __device__ __forceinline__ float4 sum4(int i, int r) const {
+    float4 a = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll 4
+    for (int s = 0; s < C; ++s) {
+      const float* src = s == rank ? part + (m0 + i) * TR : recv + ((s - (s > rank ? 1 : 0)) * ml + i) * TR;
+      const float4 v = *reinterpret_cast<const float4*>(src + r);
+      a.x += v.x;
+      a.y += v.y;
+      a.z += v.z;
+      a.w += v.w;
+    }
+    return a;
+  }
+};
+
+// Four consecutive cached values: fp16 at dst and, when res is set, their residual codes.
+__device__ __forceinline__ void store_kv4(f16* dst, uint8_t* res, float4 v) {
+  *reinterpret_cast<uint2*>(dst) = make_uint2(pack_f16x2(v.x, v.y), pack_f16x2(v.z, v.w));
+  if (!res) return;
+  const uint32_t c = kv_res_code(v.x, __float2half_rn(v.x)) | (kv_res_code(v.y, __float2half_rn(v.y)) << 4) |
+                     (kv_res_code(v.z, __float2half_rn(v.z)) << 8) | (kv_res_code(v.w, __float2half_rn(v.w)) << 12);
+  *reinterpret_cast<uint16_t*>(res) = static_cast<uint16_t>(c);
+}
+
+// Finishes this CTA's rows of the tile, kFinish items of four columns per thread at a time: what an
+// item reads from global memory is requested before `ready` (the wait for the partial sums).
+constexpr int kFinish = 2;
+template <int TR, class Ready>
+__device__ __forceinline__ void gemv_finish(const ClusterParams& p, const TileSums<TR>& t, int tile, Ready ready,
+                                            uint32_t& sat) {
+  const EpiArgs& e = p.epi;
+  const int tid = threadIdx.x;
+  if (e.kind == EPI_SWIGLU) {
+    constexpr int V = TR / 8;  // float4s of a row's gate half
+    const int F = p.N >> 1;
+    ready();
+    for (int k = tid; k < t.mn * V; k += kThreads) {
+      const int i = k / V, j = (k - i * V) * 4;
+      const float4 g = t.sum4(i, j), u = t.sum4(i, j + TR / 2);
+      const int f = tile * (TR / 2) + j;
+      if (f >= F) continue;  // F % 4 == 0: four features are in or out together
+      uint2 hi, lo;
+      split_pack2(silu_f(g.x) * u.x, silu_f(g.y) * u.y, hi.x, lo.x, e.fp16, sat);
+      split_pack2(silu_f(g.z) * u.z, silu_f(g.w) * u.w, hi.y, lo.y, e.fp16, sat);
+      const size_t off = static_cast<size_t>(t.m0 + i) * e.ldo + f;
+      *reinterpret_cast<uint2*>(e.out_hi + off) = hi;
+      *reinterpret_cast<uint2*>(e.out_lo + off) = lo;
+    }
+  } else if (e.kind == EPI_QKV) {
+    // whole heads lie in a tile (TR % hd == 0, sections are multiples of hd): float4s of rotary
+    // index i and of its partner i + hd / 2
+    constexpr int V = TR / 8;
+    const int d = e.d, hd = e.hd, half = hd >> 1;
+    for (int k0 = tid; k0 < t.mn * V || k0 == tid; k0 += kThreads * kFinish) {
+      int env[kFinish], pos[kFinish];
+      float4 cs[kFinish][2];  // (cos, sin) of i .. i + 3
+#pragma unroll
+      for (int u = 0; u < kFinish; ++u) {
+        const int k = k0 + u * kThreads;
+        env[u] = pos[u] = 0;
+        if (k < t.mn * V) {
+          env[u] = __ldcg(&e.rows[t.m0 + k / V].env);
+          pos[u] = __ldcg(&e.rows[t.m0 + k / V].pos);
+        }
+      }
+#pragma unroll
+      for (int u = 0; u < kFinish; ++u) {
+        const int i = (k0 + u * kThreads) % V * 4 % half;
+        const float4* c4 = reinterpret_cast<const float4*>(e.rope + static_cast<size_t>(pos[u]) * half + i);
+        cs[u][0] = c4[0];
+        cs[u][1] = c4[1];
+      }
+      if (k0 == tid) ready();
+#pragma unroll
+      for (int u = 0; u < kFinish; ++u) {
+        const int k = k0 + u * kThreads;
+        if (k >= t.mn * V) continue;
+        const int row = k / V, j = (k - row * V) * 4;
+        const int lh = j / half, i = j - lh * half;
+        float4 a = t.sum4(row, lh * hd + i), b = t.sum4(row, lh * hd + i + half);
+        const int n = tile * TR + lh * hd;
+        if (n >= p.N) continue;
+        const int sec = n / d, head = (n - sec * d) / hd;
+        if (sec < 2) {
+          const float4 c0 = cs[u][0], c1 = cs[u][1], x = a, y = b;
+          a = make_float4(x.x * c0.x - y.x * c0.y, x.y * c0.z - y.y * c0.w, x.z * c1.x - y.z * c1.y,
+                          x.w * c1.z - y.w * c1.w);
+          b = make_float4(y.x * c0.x + x.x * c0.y, y.y * c0.z + x.y * c0.w, y.z * c1.x + x.z * c1.y,
+                          y.w * c1.z + x.w * c1.w);
+        }
+        if (sec == 0) {
+          float* dst = e.out_q + static_cast<size_t>(t.m0 + row) * d + head * hd + i;
+          *reinterpret_cast<float4*>(dst) = a;
+          *reinterpret_cast<float4*>(dst + half) = b;
+        } else {
+          f16* dst = e.kv.base + static_cast<int64_t>(e.layer) * e.kv.layer_stride +
+                     static_cast<int64_t>(env[u]) * e.kv.env_stride + (sec == 2 ? e.kv.kv_stride : 0) +
+                     static_cast<int64_t>(head) * e.kv.head_stride + static_cast<int64_t>(pos[u]) * hd + i;
+          uint8_t* res = e.kv.res ? e.kv.res + (dst - e.kv.base) / 2 : nullptr;
+          store_kv4(dst, res, a);
+          store_kv4(dst + half, res ? res + half / 2 : nullptr, b);
+        }
+      }
+    }
+  } else {  // F32 / RESID
+    constexpr int V = TR / 4;
+    const bool resid = e.kind == EPI_RESID;
+    float* out = resid ? e.resid : e.out_f32;
+    const int ld = resid ? e.ldr : e.ldo;
+    const bool vec = !(ld & 3) && !(reinterpret_cast<uintptr_t>(out) & 15);
+    for (int k0 = tid; k0 < t.mn * V || k0 == tid; k0 += kThreads * kFinish) {
+      float4 x[kFinish];
+#pragma unroll
+      for (int u = 0; u < kFinish; ++u) {
+        const int k = k0 + u * kThreads, n = tile * TR + k % V * 4;
+        x[u] = make_float4(0.f, 0.f, 0.f, 0.f);
+        if (resid && vec && k < t.mn * V && n + 4 <= p.N)
+          x[u] = __ldcg(reinterpret_cast<const float4*>(out + static_cast<size_t>(t.m0 + k / V) * ld + n));
+      }
+      if (k0 == tid) ready();
+#pragma unroll
+      for (int u = 0; u < kFinish; ++u) {
+        const int k = k0 + u * kThreads;
+        if (k >= t.mn * V) continue;
+        const int i = k / V, r = (k - i * V) * 4;
+        const float4 a = t.sum4(i, r);
+        const int n = tile * TR + r;
+        float* o = out + static_cast<size_t>(t.m0 + i) * ld + n;
+        if (vec && n + 4 <= p.N) {
+          const float4 h = make_float4(x[u].x + a.x, x[u].y + a.y, x[u].z + a.z, x[u].w + a.w);
+          *reinterpret_cast<float4*>(o) = h;
+          if (e.ss_out) {  // a warp holds 128 columns of one row (N % 128 == 0): in or out together
+            const float ss = warp_sum(h.x * h.x + h.y * h.y + h.z * h.z + h.w * h.w);
+            if ((tid & 31) == 0) e.ss_out[static_cast<size_t>(n / 128) * p.M + t.m0 + i] = ss;
+          }
+        } else {
+          const float v[4] = {a.x, a.y, a.z, a.w};
+#pragma unroll
+          for (int q = 0; q < 4; ++q)
+            if (n + q < p.N) o[q] = resid ? __ldcg(o + q) + v[q] : v[q];
+        }
+      }
+    }
+  }
+}
+
+// TR weight rows per tile (SwiGLU: TR / 2 gate rows and the matching up rows), as TR / 128 MMAs of
+// M = 128 sharing each activation tile; grid = tiles * C, clusters of C CTAs.
+template <int BNX, int TR, int STAGES>
+__global__ void __launch_bounds__(kThreads, 2)
+    gemv_cluster_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ CUtensorMap tmW2,
+                   const __grid_constant__ CUtensorMap tmX, const __grid_constant__ CUtensorMap tmX2,
+                   const ClusterParams p) {
+  constexpr int NH = TR / 128;
+  constexpr int W_BYTES = TR * BK * 2;
+  constexpr int X_BYTES = BNX * BK * 2;
+  constexpr int STAGE_BYTES = W_BYTES + 2 * X_BYTES;
+  constexpr uint32_t TMEM_COLS = NH * BNX < 32 ? 32 : NH * BNX;
+  static_assert((TMEM_COLS & (TMEM_COLS - 1)) == 0 && TMEM_COLS <= 256, "TMEM allocation");
+  const uint32_t IDESC = idesc_for((1u << 4) | (1u << 7) | (1u << 10) | (static_cast<uint32_t>(BNX >> 3) << 17) |
+                                       (static_cast<uint32_t>(128 >> 4) << 24),
+                                   p.epi.fp16);
+
+  extern __shared__ uint8_t smem_raw[];
+  uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) &
+                                             ~static_cast<uintptr_t>(1023));
+  uint64_t* bars = reinterpret_cast<uint64_t*>(smem);  // one 1 KB block, then the stages
+  smem += 1024;
+  const uint32_t full0 = smem_u32(bars);
+  const uint32_t empty0 = full0 + 8 * STAGES;
+  const uint32_t done_bar = empty0 + 8 * STAGES;
+  const uint32_t recv_bar = done_bar + 8;
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 2 * STAGES + 2);
+  volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
+
+  const int warp = threadIdx.x >> 5;
+  const int lane = threadIdx.x & 31;
+  uint32_t n_ranks;
+  asm volatile("mov.u32 %0, %%cluster_nctarank;" : "=r"(n_ranks));
+  const int C = static_cast<int>(n_ranks), rank = static_cast<int>(cluster_ctarank());
+  const int tile = blockIdx.x / C;
+  const int kb0 = p.kbt * rank / C, kb1 = p.kbt * (rank + 1) / C;
+  int ok = 1;
+  if (threadIdx.x == 0) {
+    for (int s = 0; s < STAGES; ++s) {
+      mbar_init(full0 + 8 * s, 1);
+      mbar_init(empty0 + 8 * s, 1);
+    }
+    mbar_init(done_bar, 1);
+    mbar_init(recv_bar, 1);
+    *abort_flag = 0;
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&tmW)) : "memory");
+  }
+  if (warp == 1) {
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(
+                     smem_u32(tmem_slot)),
+                 "r"(TMEM_COLS)
+                 : "memory");
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+  }
+  tc_fence_before();
+  __syncthreads();
+  tc_fence_after();
+  pdl_launch_dependents();  // this CTA holds its TMEM: the next kernel's CTAs cannot take it first
+  const uint32_t tmem_base = *tmem_slot;
+  uint32_t* status = p.epi.status;
+  const uint64_t limit = p.wait_limit;
+
+  if (warp == 0) {
+    if (lane == 0) {
+      // ------------------------------------------------------------ TMA producer
+      // The weights do not depend on the previous kernel: the first STAGES weight tiles are
+      // requested before waiting for it, the activations only after.
+      const uint64_t pol_w = policy_evict_first();
+      const uint64_t pol_x = policy_evict_last();
+      const bool swiglu = p.epi.kind == EPI_SWIGLU;
+      const CUtensorMap* second = swiglu ? &tmW2 : &tmW;
+      const int row0 = swiglu ? tile * (TR / 2) : tile * TR;
+      const int row1 = swiglu ? row0 : row0 + TR / 2;
+      const int n = kb1 - kb0;
+      const int pre = n < STAGES ? n : STAGES;
+      uint32_t issued = 0, issued_phase = 0;
+      auto load_w = [&](int stage, int kb) {
+        const uint32_t sw = smem_u32(smem + stage * STAGE_BYTES);
+        mbar_arrive_expect_tx(full0 + 8 * stage, STAGE_BYTES);
+        tma_load_2d_hint(sw, &tmW, full0 + 8 * stage, kb * BK, row0, pol_w);
+        tma_load_2d_hint(sw + W_BYTES / 2, second, full0 + 8 * stage, kb * BK, row1, pol_w);
+      };
+      auto load_x = [&](int stage, int kb) {
+        const uint32_t sx = smem_u32(smem + stage * STAGE_BYTES) + W_BYTES;
+        tma_load_2d_hint(sx, &tmX, full0 + 8 * stage, kb * BK, 0, pol_x);
+        tma_load_2d_hint(sx + X_BYTES, &tmX2, full0 + 8 * stage, kb * BK, 0, pol_x);
+      };
+      for (int i = 0; i < pre; ++i) {
+        load_w(i, kb0 + i);
+        issued |= 1u << i;
+      }
+      pdl_wait_async();
+      for (int i = 0; i < pre; ++i) load_x(i, kb0 + i);
+      int stage = pre % STAGES;
+      uint32_t phase = (pre == STAGES) ? 1u : 0u;
+      for (int i = pre; i < n; ++i) {
+        if (!wait_bounded(empty0 + 8 * stage, phase ^ 1u, abort_flag, status, limit)) break;
+        load_w(stage, kb0 + i);
+        load_x(stage, kb0 + i);
+        issued_phase = (issued_phase & ~(1u << stage)) | (phase << stage);
+        if (++stage == STAGES) {
+          stage = 0;
+          phase ^= 1u;
+        }
+      }
+      for (int s = 0; s < STAGES; ++s)
+        if (issued & (1u << s)) wait_drain(full0 + 8 * s, (issued_phase >> s) & 1u, limit);
+    }
+  } else if (warp == 1) {
+    if (lane == 0) {
+      // ------------------------------------------------------------ MMA issuer
+      int stage = 0;
+      uint32_t phase = 0;
+      for (int kb = kb0; kb < kb1; ++kb) {
+        if (!wait_bounded(full0 + 8 * stage, phase, abort_flag, status, limit)) break;
+        tc_fence_after();
+        const uint32_t sw = smem_u32(smem + stage * STAGE_BYTES);
+        const uint32_t sx = sw + W_BYTES;
+#pragma unroll
+        for (int k = 0; k < BK / 16; ++k) {
+          const uint64_t xh = make_sdesc(sx + k * 32);
+          const uint64_t xl = make_sdesc(sx + X_BYTES + k * 32);
+#pragma unroll
+          for (int h = 0; h < NH; ++h) {
+            const uint64_t adesc = make_sdesc(sw + h * (128 * BK * 2) + k * 32);
+            tc_mma(tmem_base + h * BNX, adesc, xh, IDESC, (kb > kb0 || k > 0) ? 1u : 0u);
+            tc_mma(tmem_base + h * BNX, adesc, xl, IDESC, 1u);
+          }
+        }
+        tc_commit(empty0 + 8 * stage);
+        if (++stage == STAGES) {
+          stage = 0;
+          phase ^= 1u;
+        }
+      }
+      // all MMAs issued by this thread have completed: the sums are in TMEM and the stages are free
+      tc_commit(done_bar);
+      wait_drain(done_bar, 0, limit);
+    }
+  } else {
+    if (lane == 0) ok = wait_bounded(done_bar, 0, abort_flag, status, limit) && !*abort_flag ? 1 : 0;
+    ok = __shfl_sync(0xffffffffu, ok, 0);
+  }
+
+  // Lanes 1..31 of the producer and MMA warps got here long before their lane 0: reconverge first.
+  __syncwarp();
+  cluster_arrive();  // this CTA's stages are free: the others may write their partials there
+  const int ml = (p.M + C - 1) / C;  // batch rows per rank
+  const int pr = (p.M + 15) & ~15;   // rows of the partial tile
+  if (warp >= 2) {
+    // TMEM -> partial tile [batch row][tile row]: for each batch row the 32 lanes of a warp store 32
+    // consecutive floats
+    if (ok) {
+      tc_fence_after();
+      const int q = warp & 3;  // the TMEM lane quarter this warp may read
+      float* part = reinterpret_cast<float*>(smem);
+#pragma unroll
+      for (int h = 0; h < NH; ++h) {
+        float* dst = part + h * 128 + q * 32 + lane;
+        const uint32_t trow = tmem_base + (static_cast<uint32_t>(q * 32) << 16) + h * BNX;
+#pragma unroll 1
+        for (int c = 0; c < pr; c += 16) {
+          float v[16];
+          ld16f(trow + c, v);
+#pragma unroll
+          for (int i = 0; i < 16; ++i) dst[(c + i) * TR] = v[i];
+        }
+      }
+      tc_fence_before();
+    }
+    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+  }
+  __syncthreads();
+  TileSums<TR> t;
+  t.part = reinterpret_cast<const float*>(smem);
+  t.recv = t.part + pr * TR;
+  t.C = C;
+  t.rank = rank;
+  t.ml = ml;
+  t.m0 = rank * ml;
+  t.mn = max(0, min(ml, p.M - t.m0));
+  cluster_wait();
+  if (warp == 0 && lane < C) {
+    // lane s sends rank s its rows (an aborted CTA sends too, so that nobody waits for it)
+    const int s = lane, n_s = min(ml, p.M - s * ml);
+    if (s == rank) {
+      mbar_arrive_expect_tx(recv_bar, static_cast<uint32_t>((C - 1) * t.mn * TR * 4));
+    } else if (n_s > 0) {
+      const int slot = rank - (rank > s ? 1 : 0);
+      bulk_copy_cluster(mapa_shared(smem_u32(t.recv + slot * ml * TR), s), smem_u32(t.part + s * ml * TR),
+                        static_cast<uint32_t>(n_s * TR * 4), mapa_shared(recv_bar, s));
+    }
+  }
+  pdl_wait();  // (long over) the residual and the caches of this step are the previous kernels'
+  uint32_t sat = 0;
+  gemv_finish<TR>(p, t, tile, [&] { wait_drain_reported(recv_bar, 0, status, limit); }, sat);
+  report_saturation(status, sat);
+  __syncwarp();
+  cluster_arrive();
+  if (warp == 1) {
+    tc_fence_after();
+    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_base),
+                 "r"(TMEM_COLS)
+                 : "memory");
+  }
+  cluster_wait();  // no CTA leaves while its partials are still being sent
+}
+
 // ----------------------------------------------------------------------------- host side
 typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*,
                                   const cuuint64_t*, const cuuint64_t*, const cuuint32_t*,
@@ -1513,12 +1910,12 @@ GemmCost gemm_cost(const GemmArgs& a) {
 }
 
 // Stream-K plan of the weight-streaming GEMM.
-struct GemvPlan {
+struct StreamPlan {
   int bnx, grid, tiles, kbt, per_cta, max_seg;
   size_t ws_bytes;
 };
-GemvPlan gemv_plan(int M, int N, int K, int num_sms) {
-  GemvPlan g{};
+StreamPlan stream_plan(int M, int N, int K, int num_sms) {
+  StreamPlan g{};
   g.bnx = M <= 16 ? 16 : M <= 32 ? 32 : M <= 64 ? 64 : 128;
   g.tiles = (N + 255) / 256;
   g.kbt = (K + BK - 1) / BK;
@@ -1532,18 +1929,103 @@ GemvPlan gemv_plan(int M, int N, int K, int num_sms) {
 }
 
 template <int BNX>
-int launch_gemv(const CUtensorMap& w, const CUtensorMap& x, const CUtensorMap& x2,
-                const GemvParams& p, int grid, cudaStream_t stream) {
+int launch_stream(const CUtensorMap& w, const CUtensorMap& x, const CUtensorMap& x2,
+                const StreamParams& p, int grid, cudaStream_t stream) {
   constexpr int STAGE = 256 * BK * 2 + 2 * BNX * BK * 2;
   constexpr int STAGES = (196608 / STAGE) < 8 ? (196608 / STAGE) : 8;
   constexpr int smem = STAGES * STAGE + 1024 + 256;
   static std::atomic<uint64_t> attr_done{0};
-  auto kern = gemv_tc_kernel<BNX, STAGES>;
+  auto kern = gemv_stream_kernel<BNX, STAGES>;
   VLA_CUDA_TRY(set_smem_limit(kern, smem, attr_done));
   VLA_CUDA_TRY(launch_pdl(kern, dim3(grid), dim3(kThreads), smem, stream, w, x, x2, p));
   note_launch();
   VLA_CUDA_TRY(cudaGetLastError());
   return VLA_OK;
+}
+
+// Shared memory of a cluster-kernel CTA for stages, then partial tiles: two CTAs per SM (at most 113 KB
+// each with the 2 KB of alignment and barriers and the runtime's 1 KB).
+constexpr int kClusterData = 112640;
+constexpr int kClusterRows = 32;
+
+// Tile rows, cluster size and grid of the cluster kernel.
+struct ClusterPlan {
+  int bnx, tr, c, tiles, kbt;
+};
+ClusterPlan cluster_plan_for(int M, int N, int K, bool swiglu, int tr, int c) {
+  ClusterPlan g{};
+  g.bnx = M <= 16 ? 16 : 32;
+  g.kbt = (K + BK - 1) / BK;
+  g.tr = tr;
+  g.c = c;
+  g.tiles = swiglu ? (N / 2 + tr / 2 - 1) / (tr / 2) : (N + tr - 1) / tr;
+  return g;
+}
+// The split with the most CTAs that are all resident at once: two per SM,
+// less one cluster per GPC, since clusters are placed whole in one and beside CTAs of the kernel
+// before (a last cluster left to a second wave costs 12 us: 32 clusters of 8 for a 16-row o
+// projection, 31 resident).  Fewer CTAs leave SMs without a second stream of weights.
+ClusterPlan cluster_plan(int M, int N, int K, bool swiglu, int num_sms) {
+  const int slots = 2 * num_sms;
+  ClusterPlan best{};
+  int best_n = -1;
+  for (const int tr : {128, 256})
+    for (int c = 1; c <= 8; ++c) {
+      const ClusterPlan g = cluster_plan_for(M, N, K, swiglu, tr, c);
+      const int n = g.tiles * c, most = slots - 8 * c;
+      if (c > 1 && (c > g.kbt || n > most)) break;
+      // one CTA per tile already exceeds the slots: what its waves fill of them
+      const int score = n <= slots ? n : slots * (n / slots) / (n / slots + 1);
+      if (score > best_n) {
+        best = g;
+        best_n = score;
+      }
+    }
+  return best;
+}
+
+template <int BNX, int TR>
+int launch_cluster(const CUtensorMap& w, const CUtensorMap& w2, const CUtensorMap& x, const CUtensorMap& x2,
+                const ClusterParams& p, const ClusterPlan& pl, cudaStream_t stream) {
+  constexpr int STAGE = TR * BK * 2 + 2 * BNX * BK * 2;
+  constexpr int STAGES = kClusterData / STAGE;
+  // the exchange: the partial tile and the other ranks' rows, (C - 1) * ceil(M / C) < M + C
+  static_assert((2 * BNX + 8) * TR * 4 <= STAGES * STAGE, "the exchange reuses the stages");
+  constexpr int smem = STAGES * STAGE + 2048;
+  static std::atomic<uint64_t> attr_done{0};
+  auto kern = gemv_cluster_kernel<BNX, TR, STAGES>;
+  VLA_CUDA_TRY(set_smem_limit(kern, smem, attr_done));
+  VLA_CUDA_TRY(launch_pdl_cluster(kern, dim3(pl.tiles * pl.c), dim3(kThreads), smem, stream, pl.c, w, w2, x, x2, p));
+  note_launch();
+  VLA_CUDA_TRY(cudaGetLastError());
+  return VLA_OK;
+}
+
+template <int TR>
+int dispatch_cluster(const CUtensorMap& w, const CUtensorMap& w2, const CUtensorMap& x, const CUtensorMap& x2,
+                  const ClusterParams& p, const ClusterPlan& pl, cudaStream_t stream) {
+  return pl.bnx == 16 ? launch_cluster<16, TR>(w, w2, x, x2, p, pl, stream)
+                      : launch_cluster<32, TR>(w, w2, x, x2, p, pl, stream);
+}
+
+int cluster_launch_as(const GemmArgs& a, const ClusterPlan& pl, cudaStream_t stream) {
+  const bool fp16 = a.epi.fp16, swiglu = a.epi.kind == EPI_SWIGLU;
+  CUtensorMap mw, mw2, mx, mx2;
+  const int64_t rows = swiglu ? a.N / 2 : a.N;
+  bool ok = make_map(&mw, a.B, rows, a.K, a.ldb, pl.tr / 2, fp16) && make_map(&mx, a.A, a.M, a.K, a.lda, pl.bnx, fp16) &&
+            make_map(&mx2, a.A_lo, a.M, a.K, a.lda, pl.bnx, fp16);
+  mw2 = mw;
+  if (swiglu) ok = ok && make_map(&mw2, a.B + rows * a.ldb, rows, a.K, a.ldb, pl.tr / 2, fp16);
+  if (!ok) return cuda_fail(cudaErrorInvalidValue, "tensor maps (decode GEMM)");
+  ClusterParams p{};
+  p.M = a.M;
+  p.N = a.N;
+  p.K = a.K;
+  p.kbt = pl.kbt;
+  p.epi = a.epi;
+  p.wait_limit = g_wait_limit_ns.load(std::memory_order_relaxed);
+  return pl.tr == 256 ? dispatch_cluster<256>(mw, mw2, mx, mx2, p, pl, stream)
+                      : dispatch_cluster<128>(mw, mw2, mx, mx2, p, pl, stream);
 }
 
 }  // namespace
@@ -1667,10 +2149,31 @@ int gemm_launch(const GemmArgs& a, cudaStream_t stream, int num_sms, GemmCost* c
 }
 
 
+// The decode-GEMM op asks its callers for the stream-K split's size at every M; up to 32 rows the
+// cluster kernel leaves the workspace alone.
 size_t gemv_workspace_bytes(int M, int N, int K, int num_sms) {
   if (M < 1 || M > 128) return 0;
-  return gemv_plan(M, N, K, num_sms).ws_bytes;
+  return stream_plan(M, N, K, num_sms).ws_bytes;
 }
+
+bool gemv_fuses_norm(int M) { return M > kClusterRows; }
+
+namespace {
+int cluster_launch(const GemmArgs& a, cudaStream_t stream, int num_sms) {
+  const EpiArgs& e = a.epi;
+  // a following RMSNorm is its own kernel: only the sums of squares are written here
+  if (e.norm_w || e.row_ss) return VLA_ERR_ARG;
+  if (e.ss_out && (e.kind != EPI_RESID || a.N % 128 || (e.ldr & 3) || (reinterpret_cast<uintptr_t>(e.resid) & 15)))
+    return VLA_ERR_ARG;
+  if (e.kind == EPI_SWIGLU &&
+      ((a.N & 7) || (e.ldo & 3) || !e.out_hi || !e.out_lo || (reinterpret_cast<uintptr_t>(e.out_hi) & 7) ||
+       (reinterpret_cast<uintptr_t>(e.out_lo) & 7) || (reinterpret_cast<uintptr_t>(a.B + static_cast<int64_t>(a.N / 2) * a.ldb) & 15)))
+    return VLA_ERR_ARG;
+  if (e.kind == EPI_QKV && (a.N != 3 * e.d || (e.hd != 64 && e.hd != 128) || e.d % e.hd)) return VLA_ERR_ARG;
+  if (e.kind == EPI_PARTIAL) return VLA_ERR_ARG;
+  return cluster_launch_as(a, cluster_plan(a.M, a.N, a.K, e.kind == EPI_SWIGLU, num_sms), stream);
+}
+}  // namespace
 
 int gemv_launch(const GemmArgs& a, cudaStream_t stream, int num_sms, GemmCost* cost) {
   if (a.M < 1 || a.M > 128 || a.N < 1 || a.K < 1 || !a.A || !a.A_lo || !a.B) return VLA_ERR_ARG;
@@ -1687,7 +2190,14 @@ int gemv_launch(const GemmArgs& a, cudaStream_t stream, int num_sms, GemmCost* c
         (reinterpret_cast<uintptr_t>(a.epi.norm_lo) & 7))
       return VLA_ERR_ARG;
   }
-  const GemvPlan pl = gemv_plan(a.M, a.N, a.K, num_sms);
+  if (a.epi.row_ss || a.epi.kind == EPI_PARTIAL) return VLA_ERR_ARG;
+  if (a.M <= kClusterRows) {
+    const int rc = cluster_launch(a, stream, num_sms);
+    if (rc == VLA_OK && cost) *cost = gemm_cost(a);
+    return rc;
+  }
+  if (a.epi.ss_out) return VLA_ERR_ARG;
+  const StreamPlan pl = stream_plan(a.M, a.N, a.K, num_sms);
   if (!a.workspace || a.workspace_bytes < pl.ws_bytes || (reinterpret_cast<uintptr_t>(a.workspace) & 15))
     return VLA_ERR_ARG;
   CUtensorMap mw, mx, mx2;
@@ -1695,7 +2205,7 @@ int gemv_launch(const GemmArgs& a, cudaStream_t stream, int num_sms, GemmCost* c
   if (!make_map(&mw, a.B, a.N, a.K, a.ldb, 256, fp16) || !make_map(&mx, a.A, a.M, a.K, a.lda, pl.bnx, fp16) ||
       !make_map(&mx2, a.A_lo, a.M, a.K, a.lda, pl.bnx, fp16))
     return cuda_fail(cudaErrorInvalidValue, "tensor maps (decode GEMM)");
-  GemvParams p{};
+  StreamParams p{};
   p.N = a.N;
   p.K = a.K;
   p.tiles = pl.tiles;
@@ -1708,10 +2218,8 @@ int gemv_launch(const GemmArgs& a, cudaStream_t stream, int num_sms, GemmCost* c
   p.wait_limit = g_wait_limit_ns.load(std::memory_order_relaxed);
   int rc;
   switch (pl.bnx) {
-    case 16: rc = launch_gemv<16>(mw, mx, mx2, p, pl.grid, stream); break;
-    case 32: rc = launch_gemv<32>(mw, mx, mx2, p, pl.grid, stream); break;
-    case 64: rc = launch_gemv<64>(mw, mx, mx2, p, pl.grid, stream); break;
-    default: rc = launch_gemv<128>(mw, mx, mx2, p, pl.grid, stream); break;
+    case 64: rc = launch_stream<64>(mw, mx, mx2, p, pl.grid, stream); break;
+    default: rc = launch_stream<128>(mw, mx, mx2, p, pl.grid, stream); break;
   }
   if (rc != VLA_OK) return rc;
   const StreamSrc src{a.workspace, pl.bnx, pl.kbt, pl.per_cta, pl.max_seg};

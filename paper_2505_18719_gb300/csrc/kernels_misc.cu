@@ -20,7 +20,7 @@ __global__ void __launch_bounds__(256) assemble_kernel(const RowInfo* __restrict
                                                        const int* tokens,
                                                        const bf16* __restrict__ embed, int d,
                                                        int vocab, float* __restrict__ h,
-                                                       uint32_t* status) {
+                                                       const FirstNorm nm, uint32_t* status) {
   pdl_launch_dependents();
   pdl_wait();
   const RowInfo ri = rows[blockIdx.x];
@@ -36,13 +36,65 @@ __global__ void __launch_bounds__(256) assemble_kernel(const RowInfo* __restrict
     src = embed + static_cast<size_t>(id) * d;
   }
   float* dst = h + static_cast<size_t>(blockIdx.x) * d;
-  for (int c = threadIdx.x * 8; c < d; c += blockDim.x * 8) {
-    const uint4 v = *reinterpret_cast<const uint4*>(src + c);
-    const float2 a = unpack_bf16x2(v.x), b = unpack_bf16x2(v.y);
-    const float2 e = unpack_bf16x2(v.z), f = unpack_bf16x2(v.w);
-    reinterpret_cast<float4*>(dst + c)[0] = make_float4(a.x, a.y, b.x, b.y);
-    reinterpret_cast<float4*>(dst + c)[1] = make_float4(e.x, e.y, f.x, f.y);
+  float ss = 0.f;
+  for (int c = threadIdx.x * 4; c < d; c += blockDim.x * 4) {
+    const uint2 x = *reinterpret_cast<const uint2*>(src + c);
+    const float2 a = unpack_bf16x2(x.x), b = unpack_bf16x2(x.y);
+    const float4 v = make_float4(a.x, a.y, b.x, b.y);
+    *reinterpret_cast<float4*>(dst + c) = v;
+    ss += v.x * v.x + v.y * v.y + v.z * v.z + v.w * v.w;
   }
+  // the first layer's RMSNorm of the row, in rmsnorm_kernel's order (the source row again, from L1)
+  __shared__ float red[8];
+  ss = warp_sum(ss);
+  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = ss;
+  __syncthreads();
+  float tot = 0.f;
+  for (int i = 0; i < (blockDim.x >> 5); ++i) tot += red[i];
+  const float r = rsqrtf(tot / static_cast<float>(d) + nm.eps);
+  const size_t off = static_cast<size_t>(blockIdx.x) * d;
+  uint32_t sat = 0;
+  for (int c = threadIdx.x * 4; c < d; c += blockDim.x * 4) {
+    const uint2 x = *reinterpret_cast<const uint2*>(src + c), ww = *reinterpret_cast<const uint2*>(nm.w + c);
+    const float2 a = unpack_bf16x2(x.x), b = unpack_bf16x2(x.y), w0 = unpack_bf16x2(ww.x), w1 = unpack_bf16x2(ww.y);
+    uint2 hi, lo;
+    split_pack2(a.x * r * w0.x, a.y * r * w0.y, hi.x, lo.x, nm.fp16, sat);
+    split_pack2(b.x * r * w1.x, b.y * r * w1.y, hi.y, lo.y, nm.fp16, sat);
+    *reinterpret_cast<uint2*>(nm.y_hi + off + c) = hi;
+    *reinterpret_cast<uint2*>(nm.y_lo + off + c) = lo;
+  }
+  report_saturation(status, sat);
+}
+
+// y = h * rsqrt(mean square + eps) * w of a row whose sums of squares over 128-column blocks are at hand:
+// nothing to reduce, so a row is cut into CTAs of 1024 columns, four per thread, and the kernel is one
+// round trip to L2 (weights and block sums in flight with the row).  A 16-row 7B decode layer spent 6.6 to
+// 9.3 us on each rmsnorm_kernel between its projections.
+__global__ void __launch_bounds__(256) norm_scale_kernel(const float* h, int ldh, const bf16* __restrict__ w,
+                                                         const float* ss, int n_ss, int M, int d, float eps,
+                                                         bf16* __restrict__ y_hi, bf16* __restrict__ y_lo, bool fp16,
+                                                         uint32_t* status) {
+  pdl_launch_dependents();
+  const int m = blockIdx.y, c = (blockIdx.x * 256 + threadIdx.x) * 4, lane = threadIdx.x & 31;
+  uint2 ww = make_uint2(0u, 0u);
+  if (c < d) ww = *reinterpret_cast<const uint2*>(w + c);
+  pdl_wait();
+  float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+  if (c < d) v = __ldcg(reinterpret_cast<const float4*>(h + static_cast<size_t>(m) * ldh + c));
+  float s = 0.f;
+  for (int i = lane; i < n_ss; i += 32) s += __ldcg(ss + static_cast<size_t>(i) * M + m);
+  s = warp_sum(s);
+  if (c >= d) return;
+  const float r = rsqrtf(s / static_cast<float>(d) + eps);
+  const float2 w0 = unpack_bf16x2(ww.x), w1 = unpack_bf16x2(ww.y);
+  uint2 hi, lo;
+  uint32_t sat = 0;
+  split_pack2(v.x * r * w0.x, v.y * r * w0.y, hi.x, lo.x, fp16, sat);
+  split_pack2(v.z * r * w1.x, v.w * r * w1.y, hi.y, lo.y, fp16, sat);
+  const size_t off = static_cast<size_t>(m) * d + c;
+  *reinterpret_cast<uint2*>(y_hi + off) = hi;
+  *reinterpret_cast<uint2*>(y_lo + off) = lo;
+  report_saturation(status, sat);
 }
 
 __global__ void __launch_bounds__(256) rmsnorm_kernel(const float* h, int ldh,
@@ -103,11 +155,11 @@ __global__ void scatter_rows_kernel(const float* src, const int* __restrict__ si
 }  // namespace
 
 int assemble_launch(const RowInfo* rows, int n_rows, const bf16* visual, const int* ids,
-                    const int* tokens, const bf16* embed, int d, int vocab, float* h,
+                    const int* tokens, const bf16* embed, int d, int vocab, float* h, const FirstNorm& norm,
                     uint32_t* status, cudaStream_t s) {
   if (n_rows <= 0) return VLA_OK;
   VLA_CUDA_TRY(launch_pdl(assemble_kernel, dim3(n_rows), dim3(256), 0, s, rows, visual, ids, tokens,
-                          embed, d, vocab, h, status));
+                          embed, d, vocab, h, norm, status));
   note_launch();
   VLA_CUDA_TRY(cudaGetLastError());
   return VLA_OK;
@@ -118,6 +170,16 @@ int rmsnorm_launch(const float* h, int ldh, const bf16* w, int M, int d, float e
   if (M <= 0) return VLA_OK;
   VLA_CUDA_TRY(launch_pdl(rmsnorm_kernel, dim3(M), dim3(256), 0, s, h, ldh, w, d, eps, y_hi, y_lo, fp16,
                           status));
+  note_launch();
+  VLA_CUDA_TRY(cudaGetLastError());
+  return VLA_OK;
+}
+
+int norm_scale_launch(const float* h, int ldh, const bf16* w, const float* ss, int n_ss, int M, int d, float eps,
+                      bf16* y_hi, bf16* y_lo, cudaStream_t s, bool fp16, uint32_t* status) {
+  if (M <= 0) return VLA_OK;
+  VLA_CUDA_TRY(launch_pdl(norm_scale_kernel, dim3((d + 1023) / 1024, M), dim3(256), 0, s, h, ldh, w, ss, n_ss, M, d,
+                          eps, y_hi, y_lo, fp16, status));
   note_launch();
   VLA_CUDA_TRY(cudaGetLastError());
   return VLA_OK;

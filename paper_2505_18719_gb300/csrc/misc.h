@@ -6,9 +6,21 @@ namespace vla {
 
 // h[r] (f32 [rows, d]) = source row of RowInfo r: visual (bf16 row idx), text (embed[ids[idx]])
 // or token (embed[tokens[idx]]).  Ids outside [0, vocab) -> VLA_STATUS_BAD_TOKEN, row 0.
+// The rows' RMSNorm with weight norm.w goes to norm.y_hi / y_lo [rows, d] as the operand pair.
+struct FirstNorm {
+  const bf16* w;
+  float eps;
+  bf16* y_hi;
+  bf16* y_lo;
+  bool fp16;
+};
 int assemble_launch(const RowInfo* rows, int n_rows, const bf16* visual, const int* ids,
-                    const int* tokens, const bf16* embed, int d, int vocab, float* h,
+                    const int* tokens, const bf16* embed, int d, int vocab, float* h, const FirstNorm& norm,
                     uint32_t* status, cudaStream_t s);
+
+// The RMSNorm of rows whose sums of squares are known: sum_i ss[i * M + m], i < n_ss.
+int norm_scale_launch(const float* h, int ldh, const bf16* w, const float* ss, int n_ss, int M, int d, float eps,
+                      bf16* y_hi, bf16* y_lo, cudaStream_t s, bool fp16, uint32_t* status);
 
 // y[m] = h[m] / sqrt(mean(h[m]^2) + eps) * w, h f32 [M, d] (row stride ldh), written as the
 // operand pair (y_hi, y_lo) [M, d] with y_hi + y_lo ~ y, fp16 if `fp16` else bf16; a finite

@@ -204,6 +204,15 @@ __device__ __forceinline__ void wait_drain(uint32_t bar, uint32_t parity, uint64
     if (globaltimer() - t0 > limit_ns) return;
   }
 }
-
+// The same for data that has to arrive: a wait that runs out reports the timeout.
+__device__ __forceinline__ void wait_drain_reported(uint32_t bar, uint32_t parity, uint32_t* status, uint64_t limit_ns) {
+  const uint64_t t0 = globaltimer();
+  while (!mbar_try_wait(bar, parity)) {
+    if (globaltimer() - t0 > limit_ns) {
+      if (status) atomicOr(status, VLA_STATUS_TIMEOUT);
+      return;
+    }
+  }
+}
 
 }  // namespace vla

@@ -87,3 +87,14 @@ def test_forced_edge_bins(weights):
     forced = torch.stack([BASE + edge.roll(b) for b in range(4)]).to(torch.int32)
     rep, _ = _rollout(weights, inp.visual, inp.ids, inp.lengths.tolist(), cap=128, forced=forced)
     assert rep.ok(), rep
+
+
+def test_shape_whose_sections_straddle_weight_tiles(monkeypatch):
+    # d = 640: q, k and v each end inside a 256-row weight tile, and d_ffn is no multiple of one
+    import sys
+    sh = I.ModelShape("tiny", 2, 640, 10, 64, 1712)
+    monkeypatch.setattr(sys.modules[__name__], "SH", sh)
+    w = I.make_weights(sh, WL.weight_seed)
+    ids = I.make_turn_inputs(WL, 0).ids
+    rep, _ = _rollout((w, P.weights_to_device(w)), None, ids, [1, 5, 12], 64)
+    assert rep.ok(), rep

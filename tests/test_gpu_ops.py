@@ -113,6 +113,19 @@ def test_decode_gemm_matches_fp64(M, N, K):
     assert err < 2e-5 * math.sqrt(K) * 8, err
 
 
+@pytest.mark.parametrize("M,N,K", [
+    (1, 1, 8),             # one k-block, one output
+    (15, 130, 72),         # fewer rows than the MMA's 16, a tile of two rows
+    (17, 4099, 4096),      # rows per rank that do not divide M, unaligned output rows
+    (32, 22016, 4096),     # the last size of the cluster kernel, 7B gate|up
+    (33, 512, 448),        # the first of the stream-K kernel
+    (8, 45000, 128),       # more tiles than CTAs resident at once
+    (16, 2560, 640),       # a cluster of 8 over 10 k-blocks
+])
+def test_decode_gemm_dispatch_edges(M, N, K):
+    test_decode_gemm_matches_fp64(M, N, K)
+
+
 def test_gemm_rejects_bad_strides():
     A = torch.zeros(8, 12, dtype=torch.bfloat16, device="cuda")
     C = torch.zeros(8, 8, dtype=torch.float32, device="cuda")
