@@ -9,12 +9,13 @@
 //    fp16 hi/lo pair; the output is written as the operand hi/lo pair the O-projection GEMM
 //    reads (fp16 for the engine, bf16 for the op entry points).
 //  * attn_decode: one query per env (the decode step) with the key range split across CTAs
-//    (flash-decoding); each CTA writes its partial (max, sum, unnormalised output) and the
-//    last CTA of the (env, head) to finish merges the splits in a fixed order.  16 lanes x
-//    16 bytes read one 128-element key row, so each warp streams two rows per instruction.
+//    (flash-decoding); each CTA writes its partial (reference exponent, sum, unnormalised output)
+//    and the last CTA of the (env, head) to finish merges the splits in a fixed order.
 //
 // Keys visible to a query at position p are positions 0..p (all of them are in the cache:
 // chunk rows write their K/V in the QKV epilogue before attention runs).
+#include <algorithm>
+
 #include "attention.h"
 #include "ptx.cuh"
 
@@ -562,180 +563,300 @@ __global__ void __launch_bounds__(128, 4) attn_rows_kernel(const float* q, bf16*
 }
 
 // ---------------------------------------------------------------------------------- decode
-// One query per (env, head, key range): 16 lanes x 16 bytes read one 128-element fp16 key row
-// (with RES, also its 4-bit residual codes, 4 bytes per lane, and use hi + lo as the cached value),
-// each lane group loads 4 key rows (K and V) before using any (memory-level parallelism), the
-// dot products reduce with xor shuffles inside the group, online softmax per lane group; the
-// groups of the CTA merge through shared memory into one partial (max, sum, unnormalised
-// output) per range.  The last CTA of an (env, head) to finish (a ticket on counters[b * H +
-// head], no waiting) merges the S partials in range order and writes the normalised output as
-// the operand pair; with S == 1 the CTA writes it directly.
-// NW = 2 warps per CTA; ptxas allocates 64 registers for both head dims with no spill, so 16
-// CTAs fit on an SM and the 2048 (env, head) CTAs of a 64-env, 32-head step are all resident
-// at once (one wave, no tail).  No minimum-blocks bound is given: capping at 64 forces a small
-// spill in the 64-dim variant.
+// One query per (env, head, key range).  A warp takes 16 keys at a time on mma.sync, with the products
+// arranged so that cached rows go from global memory into MMA operands without a shuffle or a
+// conversion (which of a row's elements an MMA's k index stands for is free as long as both operands
+// agree):
+//   S   keys x 8 columns = K Q^T: lane (g, t) of the A operand reads 16-byte chunks 4 i + t of rows g
+//       and g + 8;
+//   O   dims x 8 columns = V^T P^T: lane (g, t) reads chunks 8 u + g of keys 2t, 2t + 1, 2t + 8, 2t + 9
+//       and pairs two keys' elements with one byte permute.
+// Columns 0 - 2 of the other operand carry three parts, as fp16, of the query or of the weights
+// (together the fp32 value in full, both scaled by a power of two into the middle of fp16's range),
+// columns 3 - 7 zeros; the cached value's low part (RES) multiplies the same columns.  Every MMA chain
+// is at most four long and added up in fp32, since the tensor cores truncate their sums.  Each warp has
+// its own ring of cp.async slots: bytes in flight cost shared memory, not registers.
+// The warps of the CTA merge through shared memory into one partial (reference exponent, sum,
+// unnormalised output) per range.  The last CTA of an (env, head) to finish (a ticket on
+// counters[b * H + head], no waiting) merges the S partials in range order and writes the normalised
+// output as the operand pair; with S == 1 the CTA writes it directly.
+// Bound by the K/V bytes for many pairs and by the chain of one CTA's steps for few.  fp32 FMAs, one key
+// per half warp and 16 keys' loads in registers, took about 1200 instructions per 16 keys and warp; this
+// takes about 700.  Decode of 256 envs at 1100 positions (two 7B layers) 13500 -> 12320 us, 6.1 TB/s of
+// weights and K/V; one layer's attention of 64 envs 83 -> 73 us, of 16 envs 34 -> 25.  (Rows loaded
+// straight into registers, 12 warps per SM: 64 envs 2283 -> 2452 us a decode; two whole 10 KB stages per
+// warp instead of three 5 KB slots: 2320 against 2294.)  Error of the output against 64 bits over 20 to
+// 1100 keys: 1.8e-7 to 2.4e-7 (4.6e-7 for queries eight times as large), before 1.9e-7 to 2.8e-7 (5.8e-7).
 constexpr int kDecodeWarps = 2;
+constexpr int kSmemPerSm = 228 * 1024;
+constexpr int kDecodeStatic = 2304;  // of a CTA's shared memory: the runtime's 1 KB and the static arrays
+
+// Part `n` (0 .. 2) of x, 8 significant bits each: an fp32 value in full, NaN if x is not finite; 0 for
+// n > 2.  Short parts leave the products with 11-bit values room in the tensor cores' sums, which cut
+// terms off at the largest one's last bits.
+__device__ __forceinline__ float part8(float x, int n) {
+  const float p0 = bf2f(f2bf(x));
+  const float r0 = x - p0;
+  const float p1 = bf2f(f2bf(r0));
+  return n == 0 ? p0 : n == 1 ? p1 : n == 2 ? r0 - p1 : 0.f;
+}
+
+// A warp's ring of three slots, each the keys or the values of 16 positions with their codes, in the order
+// K 0, V 0, K 1, V 1 ..: a slot is refilled as soon as its product is done, so two others are in flight or
+// landed.  16-byte chunks are stored xor-swizzled by row so that the operand reads hit distinct banks
+// (value codes: two-way).
+template <int HD, bool RES>
+struct DecodeSlot {
+  static constexpr int ROW = HD * 2, CODE = RES ? HD / 2 : 0;  // bytes of a row, of its codes
+  static constexpr int BYTES = 16 * (ROW + CODE);
+  static constexpr int RING = 3 * BYTES;
+  __device__ static int k(int r, int c) { return r * ROW + ((c ^ ((r & 1) << 2)) << 4); }
+  __device__ static int v(int r, int c) { return r * ROW + ((c ^ (((r >> 1) & 3) << 1)) << 4); }
+  __device__ static int code(int r, int c) {
+    return 16 * ROW + r * CODE + ((HD == 128 ? c ^ ((r >> 1) & 3) : c ^ ((r >> 2) & 1)) << 4);
+  }
+};
+
 template <int HD, bool RES, int NW = kDecodeWarps>
-__global__ void __launch_bounds__(NW * 32, RES ? 14 : 1) attn_decode_kernel(const float* q, const RowInfo* rows,
+__global__ void __launch_bounds__(NW * 32, decode_ctas_per_sm(HD)) attn_decode_kernel(const float* q, const RowInfo* rows,
                                                           KVLayout kv, int layer, int H,
-                                                          int chunk, int S, float scale_log2,
+                                                          int n_whole, int chunk, int S_rest, float scale_log2,
                                                           float* __restrict__ part_o,
                                                           float2* __restrict__ part_ml,
                                                           int* __restrict__ counters,
                                                           bf16* __restrict__ out_hi,
                                                           bf16* __restrict__ out_lo, bool fp16) {
-  constexpr int LPK = HD / 8;     // lanes per key row (8 fp16 = 16 bytes per lane)
-  constexpr int KPI = 32 / LPK;   // key rows per warp instruction
-  constexpr int U = 4;            // key rows per lane group loaded ahead
-  constexpr int NT = NW * 32;      // threads
-  __shared__ float s_m[NW][KPI], s_l[NW][KPI];
-  __shared__ float s_o[NW][KPI][HD];
+  constexpr int KT = HD / 32;  // 16-byte chunks of a key row per lane
+  constexpr int VT = HD / 64;  // 16-byte chunks of a value row per lane
+  constexpr int NT = NW * 32;  // threads
+  using St = DecodeSlot<HD, RES>;
+  extern __shared__ __align__(128) uint8_t sm_dec[];
+  __shared__ float s_m[NW], s_l[NW];
+  __shared__ float s_o[NW][HD];
 
   pdl_launch_dependents();
   pdl_wait();
-  const int split = blockIdx.x, head = blockIdx.y, b = blockIdx.z;
+  // the first n_whole (env, head) pairs take one CTA each, the others S_rest ranges of `chunk` keys
+  const bool whole = static_cast<int>(blockIdx.x) < n_whole;
+  const int rest = static_cast<int>(blockIdx.x) - n_whole;
+  const int S = whole ? 1 : S_rest;
+  const int split = whole ? 0 : rest % S_rest;
+  const int bh = whole ? blockIdx.x : n_whole + rest / S_rest;
+  const int b = bh / H, head = bh - b * H;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int sub = lane / LPK, part = lane - sub * LPK;
+  const int g = lane >> 2, t = lane & 3;
+  uint8_t* ring = sm_dec + warp * St::RING;
   // the queries and row table come from the kernels just before (programmatic dependent
   // launch): read them at L2, never through the non-coherent read-only path
-  RowInfo ri;
-  ri.env = __ldcg(&rows[b].env);
-  ri.pos = __ldcg(&rows[b].pos);
+  const int env = __ldcg(&rows[b].env), pos = __ldcg(&rows[b].pos);
   const int d = H * HD;
   const int k_begin = split * chunk;
-  const int k_end = min(k_begin + chunk, ri.pos + 1);
+  const int k_end = S == 1 ? pos + 1 : min(k_begin + chunk, pos + 1);
 
-  float qv[8];
-  {
-    const float4* qp = reinterpret_cast<const float4*>(q + static_cast<size_t>(b) * d + head * HD + part * 8);
-    const float4 q0 = __ldcg(qp), q1 = __ldcg(qp + 1);
-    qv[0] = q0.x * scale_log2;
-    qv[1] = q0.y * scale_log2;
-    qv[2] = q0.z * scale_log2;
-    qv[3] = q0.w * scale_log2;
-    qv[4] = q1.x * scale_log2;
-    qv[5] = q1.y * scale_log2;
-    qv[6] = q1.z * scale_log2;
-    qv[7] = q1.w * scale_log2;
-  }
   const f16* kbase = kv.base + static_cast<int64_t>(layer) * kv.layer_stride +
-                     static_cast<int64_t>(ri.env) * kv.env_stride +
+                     static_cast<int64_t>(env) * kv.env_stride +
                      static_cast<int64_t>(head) * kv.head_stride;
   const f16* vbase = kbase + kv.kv_stride;
   // RES: the residual codes of the same elements (half a byte each), read with the fp16 parts
   const uint8_t* kres = RES ? kv.res + (kbase - kv.base) / 2 : nullptr;
   const uint8_t* vres = RES ? kres + kv.kv_stride / 2 : nullptr;
 
-  float m = -INFINITY, l = 0.f, o[8];
+  // 16 keys (or values) from key0 on into a slot; past the range's end its last one again (weight zero)
+  auto load = [&](bool value, int key0, int slot) {
+    if (key0 < k_end) {
+      const uint32_t dst = smem_u32(ring + slot * St::BYTES);
+      const f16* base = value ? vbase : kbase;
+      constexpr int RC = HD / 8;  // chunks of a row
 #pragma unroll
-  for (int e = 0; e < 8; ++e) o[e] = 0.f;
-
-  for (int key0 = k_begin + warp * KPI * U; key0 < k_end; key0 += NW * KPI * U) {
-    uint4 kk[U], vv[U];
-    uint32_t kc[U], vc[U];
-#pragma unroll
-    for (int u = 0; u < U; ++u) {
-      const int key = key0 + u * KPI + sub;
-      kk[u] = make_uint4(0, 0, 0, 0);
-      vv[u] = make_uint4(0, 0, 0, 0);
-      kc[u] = vc[u] = 0u;  // fp16 parts of 0: low parts 0 whatever the codes
-      if (key < k_end) {
-        kk[u] = *reinterpret_cast<const uint4*>(kbase + static_cast<int64_t>(key) * HD + part * 8);
-        vv[u] = *reinterpret_cast<const uint4*>(vbase + static_cast<int64_t>(key) * HD + part * 8);
-        if (RES) {
-          kc[u] = *reinterpret_cast<const uint32_t*>(kres + static_cast<int64_t>(key) * (HD / 2) + part * 4);
-          vc[u] = *reinterpret_cast<const uint32_t*>(vres + static_cast<int64_t>(key) * (HD / 2) + part * 4);
-        }
-      }
-    }
-#pragma unroll
-    for (int u = 0; u < U; ++u) {
-      const bool valid = key0 + u * KPI + sub < k_end;
-      const uint32_t w[4] = {kk[u].x, kk[u].y, kk[u].z, kk[u].w};
-      float acc = 0.f;
-#pragma unroll
-      for (int e = 0; e < 4; ++e) {
-        const float2 f = unpack_f16x2(w[e]);
-        acc = fmaf(qv[2 * e], f.x, acc);
-        acc = fmaf(qv[2 * e + 1], f.y, acc);
+      for (int n = 0; n < 16 * RC / 32; ++n) {
+        const int i = lane + 32 * n, r = i / RC, c = i % RC;
+        cp_async16(dst + (value ? St::v(r, c) : St::k(r, c)),
+                   base + static_cast<int64_t>(min(key0 + r, k_end - 1)) * HD + 8 * c, true);
       }
       if (RES) {
-        const uint4 kl = kv_res_lo8(kk[u], kc[u]);
-        const uint32_t wl[4] = {kl.x, kl.y, kl.z, kl.w};
+        const uint8_t* rbase = value ? vres : kres;
+        constexpr int CC = HD / 32;  // chunks of a row's codes
 #pragma unroll
-        for (int e = 0; e < 4; ++e) {
-          const float2 f = unpack_f16x2(wl[e]);
-          acc = fmaf(qv[2 * e], f.x, acc);
-          acc = fmaf(qv[2 * e + 1], f.y, acc);
+        for (int n = 0; n < 16 * CC / 32; ++n) {
+          const int i = lane + 32 * n, r = i / CC, c = i % CC;
+          cp_async16(dst + St::code(r, c), rbase + static_cast<int64_t>(min(key0 + r, k_end - 1)) * (HD / 2) + 16 * c, true);
         }
       }
-      // reduce across the LPK lanes of this key row (a row's lanes share `valid`; the xor
-      // offsets stay inside the group)
+    }
+    cp_async_commit();
+  };
+  const int key_first = k_begin + warp * 16;
+  load(false, key_first, 0);
+  load(true, key_first, 1);
+  load(false, key_first + NW * 16, 2);
+
+  // the query times log2(e) / sqrt(hd), its largest element scaled to [2^9, 2^10): part g of this
+  // lane's dims as the B operand
+  uint32_t qb[KT][4];
+  float q_inv;  // undoes the scaling
+  {
+    float x[KT][8];
+    float amax = 0.f;
 #pragma unroll
-      for (int off = LPK / 2; off > 0; off >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, off);
-      if (valid) {
-        const float m_new = fmaxf(m, acc);
-        const float alpha = exp2f(m - m_new);
-        const float p = exp2f(acc - m_new);
-        l = l * alpha + p;
-        const uint32_t v4[4] = {vv[u].x, vv[u].y, vv[u].z, vv[u].w};
-        uint32_t vl4[4] = {0u, 0u, 0u, 0u};
+    for (int i = 0; i < KT; ++i) {
+      const float4* qp = reinterpret_cast<const float4*>(q + static_cast<size_t>(b) * d + head * HD + 32 * i + 8 * t);
+      const float4 a = __ldcg(qp), c = __ldcg(qp + 1);
+      const float v[8] = {a.x, a.y, a.z, a.w, c.x, c.y, c.z, c.w};
+#pragma unroll
+      for (int e = 0; e < 8; ++e) {
+        x[i][e] = v[e] * scale_log2;
+        amax = fmaxf(amax, fabsf(x[i][e]));
+      }
+    }
+    amax = fmaxf(amax, __shfl_xor_sync(0xffffffffu, amax, 1));
+    amax = fmaxf(amax, __shfl_xor_sync(0xffffffffu, amax, 2));
+    const int ex = static_cast<int>(__float_as_uint(amax) >> 23);  // biased exponent (255: not finite)
+    const int se = min(max(263 - ex, 1), 253);
+    const float q_scale = __uint_as_float(static_cast<uint32_t>(se) << 23);
+    q_inv = __uint_as_float(static_cast<uint32_t>(254 - se) << 23);
+#pragma unroll
+    for (int i = 0; i < KT; ++i)
+#pragma unroll
+      for (int e = 0; e < 4; ++e)
+        qb[i][e] = pack_f16x2(part8(x[i][2 * e] * q_scale, g), part8(x[i][2 * e + 1] * q_scale, g));
+  }
+  // m: the running maximum less 10, so that the weights lie in (0, 2^10]; l: this lane's share of
+  // their sum; o[u][w][h]: dim 64 u + 8 g + 2 w + h, this lane's columns added up
+  float m = -INFINITY, l = 0.f, o[VT][4][2];
+#pragma unroll
+  for (int u = 0; u < VT; ++u)
+#pragma unroll
+    for (int w = 0; w < 4; ++w) o[u][w][0] = o[u][w][1] = 0.f;
+
+  int slot = 0;  // of this step's keys; its values are in the next one
+  for (int key0 = key_first; key0 < k_end; key0 += NW * 16) {
+    cp_async_wait<2>();
+    __syncwarp();
+    const uint8_t* sb = ring + slot * St::BYTES;
+    float s0 = 0.f, s1 = 0.f;  // this lane's columns of keys g and g + 8
+#pragma unroll
+    for (int i = 0; i < KT; ++i) {
+      const uint4 ka = *reinterpret_cast<const uint4*>(sb + St::k(g, 4 * i + t));
+      const uint4 kb = *reinterpret_cast<const uint4*>(sb + St::k(g + 8, 4 * i + t));
+      float c[4] = {0.f, 0.f, 0.f, 0.f};
+      if (RES) {
+        const uint4 la = kv_res_lo8(ka, *reinterpret_cast<const uint32_t*>(sb + St::code(g, i) + 4 * t));
+        const uint4 lb = kv_res_lo8(kb, *reinterpret_cast<const uint32_t*>(sb + St::code(g + 8, i) + 4 * t));
+        mma16816(c, {la.x, lb.x, la.y, lb.y}, qb[i][0], qb[i][1]);
+        mma16816(c, {la.z, lb.z, la.w, lb.w}, qb[i][2], qb[i][3]);
+      }
+      mma16816(c, {ka.x, kb.x, ka.y, kb.y}, qb[i][0], qb[i][1]);
+      mma16816(c, {ka.z, kb.z, ka.w, kb.w}, qb[i][2], qb[i][3]);
+      s0 += c[0] + c[1];
+      s1 += c[2] + c[3];
+    }
+    __syncwarp();  // every lane has read the slot
+    load(true, key0 + NW * 16, slot);
+    slot = slot == 2 ? 0 : slot + 1;
+    // columns 0, 1 are with t = 0 and column 2 with t = 1; then each lane takes keys 2t, 2t + 1,
+    // 2t + 8, 2t + 9
+    s0 += __shfl_xor_sync(0xffffffffu, s0, 1);
+    s1 += __shfl_xor_sync(0xffffffffu, s1, 1);
+    float p[4];
+    p[0] = __shfl_sync(0xffffffffu, s0, 8 * t);
+    p[1] = __shfl_sync(0xffffffffu, s0, 8 * t + 4);
+    p[2] = __shfl_sync(0xffffffffu, s1, 8 * t);
+    p[3] = __shfl_sync(0xffffffffu, s1, 8 * t + 4);
+    float mx = -INFINITY;
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      p[j] = key0 + 2 * t + (j & 1) + 8 * (j >> 1) < k_end ? p[j] * q_inv : -INFINITY;
+      mx = fmaxf(mx, p[j]);
+    }
+    mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 1));
+    mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 2));
+    const float m_new = fmaxf(m, mx - 10.f);
+    const float alpha = exp2f(m - m_new);
+    m = m_new;
+#pragma unroll
+    for (int j = 0; j < 4; ++j) p[j] = exp2f(p[j] - m_new);
+    l = l * alpha + ((p[0] + p[1]) + (p[2] + p[3]));
+    cp_async_wait<2>();
+    __syncwarp();
+    sb = ring + slot * St::BYTES;
+    const uint32_t b0 = pack_f16x2(part8(p[0], g), part8(p[1], g));
+    const uint32_t b1 = pack_f16x2(part8(p[2], g), part8(p[3], g));
+#pragma unroll
+    for (int u = 0; u < VT; ++u) {
+      uint32_t hw[4][4], lw[4][4];
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        const int r = 2 * t + (j & 1) + 8 * (j >> 1);
+        const uint4 hv = *reinterpret_cast<const uint4*>(sb + St::v(r, 8 * u + g));
+        hw[j][0] = hv.x;
+        hw[j][1] = hv.y;
+        hw[j][2] = hv.z;
+        hw[j][3] = hv.w;
         if (RES) {
-          const uint4 vl = kv_res_lo8(vv[u], vc[u]);
-          vl4[0] = vl.x;
-          vl4[1] = vl.y;
-          vl4[2] = vl.z;
-          vl4[3] = vl.w;
+          const uint4 lv = kv_res_lo8(hv, *reinterpret_cast<const uint32_t*>(sb + St::code(r, 2 * u + (g >> 2)) + 4 * (g & 3)));
+          lw[j][0] = lv.x;
+          lw[j][1] = lv.y;
+          lw[j][2] = lv.z;
+          lw[j][3] = lv.w;
         }
+      }
 #pragma unroll
-        for (int e = 0; e < 4; ++e) {
-          const float2 f = unpack_f16x2(v4[e]);
-          const float2 fl = unpack_f16x2(vl4[e]);
-          o[2 * e] = fmaf(p, f.x + fl.x, o[2 * e] * alpha);
-          o[2 * e + 1] = fmaf(p, f.y + fl.y, o[2 * e + 1] * alpha);
-        }
-        m = m_new;
+      for (int w = 0; w < 4; ++w) {
+        // rows g and g + 8 of the product: dims 2w and 2w + 1 of the chunk
+        float c[4] = {0.f, 0.f, 0.f, 0.f};
+        if (RES)
+          mma16816(c, {__byte_perm(lw[0][w], lw[1][w], 0x5410), __byte_perm(lw[0][w], lw[1][w], 0x7632),
+                       __byte_perm(lw[2][w], lw[3][w], 0x5410), __byte_perm(lw[2][w], lw[3][w], 0x7632)}, b0, b1);
+        mma16816(c, {__byte_perm(hw[0][w], hw[1][w], 0x5410), __byte_perm(hw[0][w], hw[1][w], 0x7632),
+                     __byte_perm(hw[2][w], hw[3][w], 0x5410), __byte_perm(hw[2][w], hw[3][w], 0x7632)}, b0, b1);
+        o[u][w][0] = fmaf(o[u][w][0], alpha, c[0] + c[1]);
+        o[u][w][1] = fmaf(o[u][w][1], alpha, c[2] + c[3]);
       }
     }
+    __syncwarp();
+    load(false, key0 + 2 * NW * 16, slot);
+    slot = slot == 2 ? 0 : slot + 1;
   }
-  // per (warp, sub) partials -> shared memory
-  if (part == 0) {
-    s_m[warp][sub] = m;
-    s_l[warp][sub] = l;
+  // the warps' states -> shared memory: sums over the lanes of a row
+  l += __shfl_xor_sync(0xffffffffu, l, 1);
+  l += __shfl_xor_sync(0xffffffffu, l, 2);
+  if (lane == 0) {
+    s_m[warp] = m;
+    s_l[warp] = l;
   }
 #pragma unroll
-  for (int e = 0; e < 8; ++e) s_o[warp][sub][part * 8 + e] = o[e];
-  __syncthreads();
-  // merge the 4 * KPI partial states in a fixed order
-  float M = -INFINITY;
-  for (int w = 0; w < NW; ++w)
-    for (int k = 0; k < KPI; ++k) M = fmaxf(M, s_m[w][k]);
-  float L = 0.f;
-  for (int w = 0; w < NW; ++w)
-    for (int k = 0; k < KPI; ++k)
-      if (s_m[w][k] != -INFINITY) L += s_l[w][k] * exp2f(s_m[w][k] - M);
-  const size_t bh = static_cast<size_t>(b) * H + head;
-  const size_t out_off = static_cast<size_t>(b) * d + head * HD;
-  uint32_t sat = 0;  // convex combinations of fp16 values: the fp16 split never saturates
-  if (S == 1) {
-    for (int c = threadIdx.x; c < HD; c += blockDim.x) {
-      float acc = 0.f;
-      for (int w = 0; w < NW; ++w)
-        for (int k = 0; k < KPI; ++k)
-          if (s_m[w][k] != -INFINITY) acc += s_o[w][k][c] * exp2f(s_m[w][k] - M);
-      store_split1(out_hi, out_lo, out_off + c, acc / L, fp16, sat);
+  for (int u = 0; u < VT; ++u)
+#pragma unroll
+    for (int w = 0; w < 4; ++w) {
+      const float a = o[u][w][0] + __shfl_xor_sync(0xffffffffu, o[u][w][0], 1);
+      const float c = o[u][w][1] + __shfl_xor_sync(0xffffffffu, o[u][w][1], 1);
+      if (t == 0) *reinterpret_cast<float2*>(&s_o[warp][64 * u + 8 * g + 2 * w]) = make_float2(a, c);
     }
-    return;
+  __syncthreads();
+  // merge the warps' states in order
+  float M = -INFINITY;
+#pragma unroll
+  for (int w = 0; w < NW; ++w) M = fmaxf(M, s_m[w]);
+  float L = 0.f, wt[NW];
+#pragma unroll
+  for (int w = 0; w < NW; ++w) {
+    wt[w] = s_m[w] != -INFINITY ? exp2f(s_m[w] - M) : 0.f;  // -inf: a warp without keys
+    L += s_l[w] * wt[w];
   }
-  const size_t slot = bh * S + split;
-  for (int c = threadIdx.x; c < HD; c += blockDim.x) {
+  const size_t out_off = static_cast<size_t>(b) * d + head * HD;
+  const size_t part0 = static_cast<size_t>(bh - n_whole) * S;  // S > 1: this pair's partials
+  uint32_t sat = 0;  // convex combinations of fp16 values: the fp16 split never saturates
+  for (int c = threadIdx.x; c < HD; c += NT) {
     float acc = 0.f;
-    for (int w = 0; w < NW; ++w)
-      for (int k = 0; k < KPI; ++k)
-        if (s_m[w][k] != -INFINITY) acc += s_o[w][k][c] * exp2f(s_m[w][k] - M);
-    part_o[slot * HD + c] = acc;
+#pragma unroll
+    for (int w = 0; w < NW; ++w) acc += s_o[w][c] * wt[w];
+    if (S == 1)
+      store_split1(out_hi, out_lo, out_off + c, acc / L, fp16, sat);
+    else
+      part_o[(part0 + split) * HD + c] = acc;
   }
-  if (threadIdx.x == 0) part_ml[slot] = make_float2(M, L);
+  if (S == 1) return;
+  if (threadIdx.x == 0) part_ml[part0 + split] = make_float2(M, L);
 
   // ticket: the partial is published (fence) before the counter moves
   __shared__ int s_last;
@@ -746,20 +867,21 @@ __global__ void __launch_bounds__(NW * 32, RES ? 14 : 1) attn_decode_kernel(cons
   if (!s_last) return;
   __threadfence();
   float Mx = -INFINITY;
-  for (int s = 0; s < S; ++s) Mx = fmaxf(Mx, __ldcg(&part_ml[bh * S + s].x));
+#pragma unroll 8
+  for (int s = 0; s < S; ++s) Mx = fmaxf(Mx, __ldcg(&part_ml[part0 + s].x));
   float Lt = 0.f;
   float acc[(HD + NT - 1) / NT];
 #pragma unroll
   for (int i = 0; i < (HD + NT - 1) / NT; ++i) acc[i] = 0.f;
+#pragma unroll 8
   for (int s = 0; s < S; ++s) {
-    const float2 ml = __ldcg(&part_ml[bh * S + s]);
-    if (ml.x == -INFINITY) continue;
-    const float w = exp2f(ml.x - Mx);
+    const float2 ml = __ldcg(&part_ml[part0 + s]);
+    const float w = ml.x != -INFINITY ? exp2f(ml.x - Mx) : 0.f;  // -inf: a range without keys, its partials 0
     Lt += ml.y * w;
 #pragma unroll
     for (int i = 0; i < (HD + NT - 1) / NT; ++i) {
       const int c = threadIdx.x + i * NT;
-      if (c < HD) acc[i] += __ldcg(&part_o[(bh * S + s) * HD + c]) * w;
+      if (c < HD) acc[i] += __ldcg(&part_o[(part0 + s) * HD + c]) * w;
     }
   }
 #pragma unroll
@@ -823,23 +945,32 @@ int attn_rows_launch(const float* q, bf16* out_hi, bf16* out_lo, const AttnTile*
 }
 
 int attn_decode_launch(const float* q, bf16* out_hi, bf16* out_lo, const RowInfo* rows, int B,
-                       int max_ctx, KVLayout kv, int layer, int H, int hd, int chunk,
-                       float* part_o, float2* part_ml, int* counters, cudaStream_t stream, bool fp16) {
+                       int max_ctx, KVLayout kv, int layer, int H, int hd, int n_whole, int S,
+                       float* part_o, float2* part_ml, int* counters, cudaStream_t stream, bool fp16, int num_sms) {
   if (B <= 0) return VLA_OK;
-  // equal key ranges (multiples of 16) no longer than `chunk`
-  const int S = (max_ctx + chunk - 1) / chunk;
-  const int c = ((max_ctx + S - 1) / S + 15) / 16 * 16;
+  if (n_whole < 0 || n_whole > B * H || S < 1) return VLA_ERR_ARG;
+  const int c = ((max_ctx + S - 1) / S + 15) / 16 * 16;  // equal key ranges, multiples of 16
   const float scale_log2 = 1.4426950408889634f / sqrtf(static_cast<float>(hd));
-  dim3 grid(S, H, B);
-  auto go = [&](auto kern) {
-    return launch_pdl(kern, grid, dim3(kDecodeWarps * 32), 0, stream, q, rows, kv, layer, H, c, S, scale_log2, part_o,
-                      part_ml, counters, out_hi, out_lo, fp16);
+  const int64_t grid = n_whole + static_cast<int64_t>(B * H - n_whole) * S;
+  auto go = [&](auto kern, int ring, std::atomic<uint64_t>& attr_done) {
+    int smem = kDecodeWarps * ring;
+    // A grid within one wave is spread evenly: CTAs start as the previous kernel's leave, and the first
+    // SMs to empty would take all they can hold (16 envs x 32 heads: 6 CTAs on some SMs, none on others,
+    // 31 us against 25), so each asks for its share of the shared memory.
+    const int64_t per_sm = (grid + num_sms - 1) / num_sms;
+    if (per_sm < decode_ctas_per_sm(hd)) smem = std::max(smem, static_cast<int>(kSmemPerSm / per_sm - kDecodeStatic) / 128 * 128);
+    if (const cudaError_t e = set_smem_limit(kern, kSmemPerSm - kDecodeStatic, attr_done)) return e;
+    return launch_pdl(kern, dim3(static_cast<unsigned>(grid)), dim3(kDecodeWarps * 32), smem, stream,
+                      q, rows, kv, layer, H, n_whole, c, S, scale_log2, part_o, part_ml, counters, out_hi, out_lo, fp16);
   };
   const bool res = kv.res != nullptr;
+  static std::atomic<uint64_t> done[4];
   if (hd == 128) {
-    VLA_CUDA_TRY(res ? go(attn_decode_kernel<128, true>) : go(attn_decode_kernel<128, false>));
+    VLA_CUDA_TRY(res ? go(attn_decode_kernel<128, true>, DecodeSlot<128, true>::RING, done[0])
+                     : go(attn_decode_kernel<128, false>, DecodeSlot<128, false>::RING, done[1]));
   } else if (hd == 64) {
-    VLA_CUDA_TRY(res ? go(attn_decode_kernel<64, true>) : go(attn_decode_kernel<64, false>));
+    VLA_CUDA_TRY(res ? go(attn_decode_kernel<64, true>, DecodeSlot<64, true>::RING, done[2])
+                     : go(attn_decode_kernel<64, false>, DecodeSlot<64, false>::RING, done[3]));
   } else {
     return VLA_ERR_UNSUPPORTED;
   }

@@ -30,13 +30,16 @@ constexpr int kAttnRowsMax = 16;
 int attn_rows_launch(const float* q, bf16* out_hi, bf16* out_lo, const AttnTile* tiles, int n_tiles, KVLayout kv,
                      int layer, int H, int hd, cudaStream_t stream, bool fp16, bool write_lo);
 
-// One query per env row b (rows[b] gives env and position); key range split into equal ranges
-// of at most `chunk` keys (a multiple of 16 at least 16); partials in part_o [B*H*S*hd] f32 and part_ml [B*H*S]
-// (S = ceil(max_ctx/chunk)); counters [B*H] int must be zero at launch and are zero again
-// when the kernel completes.  The output pair is fp16 if `fp16`, else bf16.
+// One query per env row b (rows[b] gives env and position).  The first n_whole of the B * H (env, head)
+// pairs run on one CTA each, the others on S CTAs with equal key ranges: their partials in part_o
+// [(B * H - n_whole) * S * hd] f32 and part_ml, counters [B * H] int zero at launch and zero again when
+// the kernel completes (none of the three is touched with S == 1).  The output pair is fp16 if `fp16`,
+// else bf16.
 int attn_decode_launch(const float* q, bf16* out_hi, bf16* out_lo, const RowInfo* rows, int B,
-                       int max_ctx, KVLayout kv, int layer, int H, int hd, int chunk,
+                       int max_ctx, KVLayout kv, int layer, int H, int hd, int n_whole, int S,
                        float* part_o, float2* part_ml, int* counters, cudaStream_t stream,
-                       bool fp16);
+                       bool fp16, int num_sms);
+// CTAs of the kernel that an SM holds.
+constexpr int decode_ctas_per_sm(int hd) { return hd == 64 ? 8 : 6; }
 
 }  // namespace vla

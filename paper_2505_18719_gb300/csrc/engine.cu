@@ -166,7 +166,6 @@ struct vla_handle {
   float* part_o = nullptr;
   float2* part_ml = nullptr;
   int* attn_tickets = nullptr;  // [B * H], zero between decode-attention launches
-  int attn_chunk = 320;  // max keys per decode-attention CTA
   int max_tiles = 0;
   // pinned host staging (ring of slots, each guarded by an event)
   static constexpr int kSlots = 4;
@@ -347,27 +346,24 @@ int run_gemm(vla_handle* h, int cls, const bf16* A, size_t a_plane, int lda, con
   return VLA_OK;
 }
 
-// Keys per decode-attention CTA.  A CTA reads 16 keys at a time and pays about 1.3 us per step, so a
-// call with few (env, head) pairs is bound by the length of that chain, not by bandwidth: its ranges
-// are cut until about kDecodeCtas CTAs share the work, down to 32 keys (two steps; shorter ranges pay
-// more for the merge than they save).  One layer of 32 heads at 290 positions, ranges of 320 keys and
-// of this rule: 1 env 36.2 -> 11.5 us, 4 envs 36.0 -> 13.7, 16 envs 39.8 -> 26.5, 32 envs 48.9 ->
-// 44.2; from 64 envs on one range per 320 keys is as fast as any.
-constexpr int kDecodeCtas = 1536;
-constexpr int kDecodeMinKeys = 32;
-int decode_attn_keys(int n_rows, int H, int max_ctx, int max_keys) {
-  const int pairs = n_rows * H;
-  const int by_len = (max_ctx + max_keys - 1) / max_keys;
-  const int by_fill = std::min((kDecodeCtas + pairs / 2) / pairs, (max_ctx + kDecodeMinKeys - 1) / kDecodeMinKeys);
-  const int S = std::max(1, std::max(by_len, by_fill));
-  return std::max(16, ((max_ctx + S - 1) / S + 15) / 16 * 16);
+// How decode attention cuts its n_rows x H (env, head) pairs: full waves of whole pairs, and the pairs
+// left over in ranges that fill one more wave.  No more ranges than that: each one costs its CTA's start
+// and a share of the merge, 4 to 5 us (16 envs x 32 heads, two 7B layers: 1, 2, 3 ranges 1504, 1557,
+// 1599 us a decode; 64 envs uncut, all cut in 2, all in 3: 2294, 2412, 2596).  A range has at least 32 keys, one
+// 16-key step per warp (1 env of 290 positions: 32, 64, 96 keys 1658, 1671, 1694 us a turn), and up to
+// 96 keys stay whole (tiny turn 496 -> 480 us).
+struct DecodeSplit {
+  int n_whole, S;
+};
+DecodeSplit decode_split(int n_rows, int H, int hd, int max_ctx, int num_sms) {
+  const int pairs = n_rows * H, slots = decode_ctas_per_sm(hd) * num_sms;
+  const int rest = pairs % slots;
+  if (!rest || max_ctx <= 96) return {pairs, 1};
+  const int S = std::min(slots / rest, (max_ctx + 31) / 32);
+  return S > 1 ? DecodeSplit{pairs - rest, S} : DecodeSplit{pairs, 1};
 }
-// Partial-output slots (rows x heads x ranges) that decode_attn_keys can ask for.
-size_t decode_attn_slots(int max_rows, int H, int capacity, int max_keys) {
-  const size_t pairs = static_cast<size_t>(max_rows) * H;
-  const size_t by_len = pairs * ((capacity + max_keys - 1) / max_keys);
-  return std::max(by_len, static_cast<size_t>(kDecodeCtas) + pairs);
-}
+// Partial-output slots that decode_split can ask for.
+size_t decode_attn_slots(int hd, int num_sms) { return static_cast<size_t>(decode_ctas_per_sm(hd)) * num_sms; }
 
 // Rows whose last-layer output is needed (a prefill only feeds the head with each env's
 // final row): idx [n] into the chunk's rows, rows [n] their RowInfo, max_ctx = longest context.
@@ -422,15 +418,19 @@ int forward_layers(vla_handle* h, int M, const RowInfo* rows_dev, bool decode, i
         return fail(h, rc, t_err);
       prof_end(h, ev, VLA_KCLASS_OTHER, 0, 16.0 * last->n * d);
       ev = prof_begin(h, VLA_KCLASS_ATTN_DECODE);
+      const DecodeSplit sp = decode_split(last->n, H, hd, last->max_ctx, h->num_sms);
       rc = attn_decode_launch(h->q_last, h->ao, h->ao + pd, last->rows, last->n, last->max_ctx, h->kvl, l, H, hd,
-                              decode_attn_keys(last->n, H, last->max_ctx, h->attn_chunk), h->part_o, h->part_ml, h->attn_tickets, h->stream, h->fp16);
+                              sp.n_whole, sp.S, h->part_o, h->part_ml, h->attn_tickets, h->stream, h->fp16,
+                              h->num_sms);
       prof_end(h, ev, VLA_KCLASS_ATTN_DECODE, 0, 0);
       Mr = last->n;
       resid = h->h_last;
     } else if (decode) {
       ev = prof_begin(h, VLA_KCLASS_ATTN_DECODE);
+      const DecodeSplit sp = decode_split(M, H, hd, max_ctx, h->num_sms);
       rc = attn_decode_launch(h->q, h->ao, h->ao + pd, rows_dev, M, max_ctx, h->kvl, l, H, hd,
-                              decode_attn_keys(M, H, max_ctx, h->attn_chunk), h->part_o, h->part_ml, h->attn_tickets, h->stream, h->fp16);
+                              sp.n_whole, sp.S, h->part_o, h->part_ml, h->attn_tickets, h->stream, h->fp16,
+                              h->num_sms);
       prof_end(h, ev, VLA_KCLASS_ATTN_DECODE, 0, 0);
     } else {
       ev = prof_begin(h, VLA_KCLASS_ATTN_PREFILL);
@@ -602,7 +602,7 @@ int vla_create(const vla_config* cfg, const vla_weights* w, void* cuda_stream, v
     }
   }
   h->ws_bytes = ws;
-  const size_t attn_slots = decode_attn_slots(B, c.n_heads, c.kv_capacity, h->attn_chunk);
+  const size_t attn_slots = decode_attn_slots(c.head_dim, h->num_sms);
   h->max_tiles = h->max_tokens / 64 + B + 1;
   const size_t T = h->max_tokens;
 
@@ -1310,7 +1310,7 @@ static int op_attn_decode(const char* name, const float* q, const void* kv, cons
   L.env_stride = 2 * L.kv_stride;
   L.layer_stride = static_cast<int64_t>(max_env) * L.env_stride;
   const int rc = attn_decode_launch(q, static_cast<bf16*>(out_hi), static_cast<bf16*>(out_lo), rows, B, max_ctx, L,
-                                    0, H, hd, chunk, part_o, part_ml, counters, st, false);
+                                    0, H, hd, 0, static_cast<int>(S), part_o, part_ml, counters, st, false, query_num_sms());
   if (rc != VLA_OK && rc != VLA_ERR_CUDA) return set_err(nullptr, rc, std::string(name) + ": unsupported arguments");
   return rc;
 }

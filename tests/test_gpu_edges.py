@@ -98,3 +98,31 @@ def test_shape_whose_sections_straddle_weight_tiles(monkeypatch):
     ids = I.make_turn_inputs(WL, 0).ids
     rep, _ = _rollout((w, P.weights_to_device(w)), None, ids, [1, 5, 12], 64)
     assert rep.ok(), rep
+
+
+def test_decode_attention_whole_pairs_and_a_split_rest(weights):
+    # 320 envs x 4 heads: more pairs than CTAs resident at once (1216), so the last 64 pairs, envs 304
+    # and up, are cut into key ranges while the others take one CTA each; lengths differ, the shortest
+    # leaves ranges without keys
+    w, wd = weights
+    B, envs = 320, [0, 303, 304, 311, 319]
+    lengths = [130 - 9 * (b % 14) for b in range(B)]
+    ids = I.randint_i32((B, 130), 5, 6, 0, BASE - 1)
+    u = I.uniform_f32((B, SH.action_dim, SH.n_bins), 5, 7)
+    orc = O.Oracle(O.shape_from(SH), w, len(envs))
+    local = list(range(len(envs)))
+    empty = torch.zeros(0, SH.d_model, dtype=torch.bfloat16)
+    orc.prefill(local, [empty for _ in envs], [ids[b, :lengths[b]].tolist() for b in envs])
+    od = orc.decode(local, u[envs], 1.0)
+    feed = torch.full((B, SH.action_dim), BASE, dtype=torch.int32)
+    feed[envs] = torch.as_tensor(od["tokens"], dtype=torch.int32)
+    pol = V.Policy(SH, wd, B, 160, B * 131)
+    try:
+        pol.prefill(None, ids.cuda(), lengths)
+        g = pol.decode(u.cuda(), 1.0, forced=feed.cuda())
+        pol.sync()
+        g = {k: v.cpu().numpy()[envs] for k, v in g.items() if v is not None}
+    finally:
+        pol.close()
+    rep = P.compare_decode(0, local, od, g)
+    assert rep.ok(), rep
