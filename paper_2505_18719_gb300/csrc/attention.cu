@@ -617,6 +617,33 @@ struct DecodeSlot {
   }
 };
 
+// One warp copies the keys (or values) of 16 positions from key0 on, with their codes, into the slot at
+// shared address dst; positions from k_end on read the last one again (their weight is zero).  One commit
+// group, empty when key0 is past the end.
+template <int HD, bool RES, bool VALUE>
+__device__ __forceinline__ void load_slot(uint32_t dst, const f16* base, const uint8_t* res, int key0, int k_end,
+                                          int lane) {
+  using St = DecodeSlot<HD, RES>;
+  if (key0 < k_end) {
+    constexpr int RC = HD / 8;  // chunks of a row
+#pragma unroll
+    for (int n = 0; n < 16 * RC / 32; ++n) {
+      const int i = lane + 32 * n, r = i / RC, c = i % RC;
+      cp_async16(dst + (VALUE ? St::v(r, c) : St::k(r, c)), base + static_cast<int64_t>(min(key0 + r, k_end - 1)) * HD + 8 * c,
+                 true);
+    }
+    if (RES) {
+      constexpr int CC = HD / 32;  // chunks of a row's codes
+#pragma unroll
+      for (int n = 0; n < 16 * CC / 32; ++n) {
+        const int i = lane + 32 * n, r = i / CC, c = i % CC;
+        cp_async16(dst + St::code(r, c), res + static_cast<int64_t>(min(key0 + r, k_end - 1)) * (HD / 2) + 16 * c, true);
+      }
+    }
+  }
+  cp_async_commit();
+}
+
 template <int HD, bool RES, int NW = kDecodeWarps>
 __global__ void __launch_bounds__(NW * 32, decode_ctas_per_sm(HD)) attn_decode_kernel(const float* q, const RowInfo* rows,
                                                           KVLayout kv, int layer, int H,
@@ -661,34 +688,16 @@ __global__ void __launch_bounds__(NW * 32, decode_ctas_per_sm(HD)) attn_decode_k
   const uint8_t* kres = RES ? kv.res + (kbase - kv.base) / 2 : nullptr;
   const uint8_t* vres = RES ? kres + kv.kv_stride / 2 : nullptr;
 
-  // 16 keys (or values) from key0 on into a slot; past the range's end its last one again (weight zero)
-  auto load = [&](bool value, int key0, int slot) {
-    if (key0 < k_end) {
-      const uint32_t dst = smem_u32(ring + slot * St::BYTES);
-      const f16* base = value ? vbase : kbase;
-      constexpr int RC = HD / 8;  // chunks of a row
-#pragma unroll
-      for (int n = 0; n < 16 * RC / 32; ++n) {
-        const int i = lane + 32 * n, r = i / RC, c = i % RC;
-        cp_async16(dst + (value ? St::v(r, c) : St::k(r, c)),
-                   base + static_cast<int64_t>(min(key0 + r, k_end - 1)) * HD + 8 * c, true);
-      }
-      if (RES) {
-        const uint8_t* rbase = value ? vres : kres;
-        constexpr int CC = HD / 32;  // chunks of a row's codes
-#pragma unroll
-        for (int n = 0; n < 16 * CC / 32; ++n) {
-          const int i = lane + 32 * n, r = i / CC, c = i % CC;
-          cp_async16(dst + St::code(r, c), rbase + static_cast<int64_t>(min(key0 + r, k_end - 1)) * (HD / 2) + 16 * c, true);
-        }
-      }
-    }
-    cp_async_commit();
+  auto load_k = [&](int key0, int slot) {
+    load_slot<HD, RES, false>(smem_u32(ring + slot * St::BYTES), kbase, kres, key0, k_end, lane);
+  };
+  auto load_v = [&](int key0, int slot) {
+    load_slot<HD, RES, true>(smem_u32(ring + slot * St::BYTES), vbase, vres, key0, k_end, lane);
   };
   const int key_first = k_begin + warp * 16;
-  load(false, key_first, 0);
-  load(true, key_first, 1);
-  load(false, key_first + NW * 16, 2);
+  load_k(key_first, 0);
+  load_v(key_first, 1);
+  load_k(key_first + NW * 16, 2);
 
   // the query times log2(e) / sqrt(hd), its largest element scaled to [2^9, 2^10): part g of this
   // lane's dims as the B operand
@@ -751,7 +760,7 @@ __global__ void __launch_bounds__(NW * 32, decode_ctas_per_sm(HD)) attn_decode_k
       s1 += c[2] + c[3];
     }
     __syncwarp();  // every lane has read the slot
-    load(true, key0 + NW * 16, slot);
+    load_v(key0 + NW * 16, slot);
     slot = slot == 2 ? 0 : slot + 1;
     // columns 0, 1 are with t = 0 and column 2 with t = 1; then each lane takes keys 2t, 2t + 1,
     // 2t + 8, 2t + 9
@@ -814,7 +823,7 @@ __global__ void __launch_bounds__(NW * 32, decode_ctas_per_sm(HD)) attn_decode_k
       }
     }
     __syncwarp();
-    load(false, key0 + 2 * NW * 16, slot);
+    load_k(key0 + 2 * NW * 16, slot);
     slot = slot == 2 ? 0 : slot + 1;
   }
   // the warps' states -> shared memory: sums over the lanes of a row
@@ -894,6 +903,230 @@ __global__ void __launch_bounds__(NW * 32, decode_ctas_per_sm(HD)) attn_decode_k
   if (threadIdx.x == 0) counters[bh] = 0;  // ready for the next launch
 }
 
+// ------------------------------------------------------------------ up to 8 rows (residual cache)
+// Query tiles of at most 8 rows (the teacher-forced action rows of the score pass) with the decode kernel's
+// layout and ring: the 8 columns of the small operand are the rows, and an fp32 value is an fp16 pair,
+//   S = K_hi Q_hi + K_hi Q_lo + K_lo Q_hi,   O = V_hi P_hi + V_hi P_lo + V_lo P_hi.
+// A lane's S values are keys g, g + 8 of rows 2t, 2t + 1; one 8 x 8 transpose (movmatrix) turns the weights
+// into the operand of the second product.  One CTA of two warps per (tile, head).
+// 64 envs x 32 heads, 6 rows, 296 positions: 71 us against 101 for attn_rows_kernel (one 45 KB stage
+// per CTA: its copies wait for its products).
+__device__ __forceinline__ uint32_t transpose8(uint32_t x) {
+  uint32_t y;
+  asm volatile("movmatrix.sync.aligned.m8n8.trans.b16 %0, %1;" : "=r"(y) : "r"(x));
+  return y;
+}
+
+constexpr int kRows8 = 8;
+template <int HD, int NW = kDecodeWarps>
+__global__ void __launch_bounds__(NW * 32, decode_ctas_per_sm(HD) - 1) attn_rows8_kernel(const float* q, bf16* out_hi, bf16* out_lo,
+                                                             const AttnTile* tiles, KVLayout kv, int layer, int H,
+                                                             float scale_log2, bool fp16, bool write_lo) {
+  constexpr int KT = HD / 32, VT = HD / 64;
+  using St = DecodeSlot<HD, true>;
+  extern __shared__ __align__(128) uint8_t sm_dec[];
+  __shared__ uint4 s_q[2][KT][32];  // the queries as B operands, fp16 hi and lo, per lane
+  __shared__ float s_m[NW][8], s_l[NW][8];
+  static_assert(NW * 8 * HD * 4 <= NW * St::RING, "the warps' outputs reuse the ring");
+
+  pdl_launch_dependents();
+  const int head = blockIdx.y;
+  const int d = H * HD;
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int g = lane >> 2, t = lane & 3;
+  uint8_t* ring = sm_dec + warp * St::RING;
+  const AttnTile tile = tiles[blockIdx.x];  // copied in before the first kernel of this call started
+  pdl_wait();
+  const int k_end = tile.pos0 + tile.nrows;
+  const int64_t e0 = static_cast<int64_t>(layer) * kv.layer_stride + static_cast<int64_t>(tile.env) * kv.env_stride +
+                     static_cast<int64_t>(head) * kv.head_stride;
+  const f16* kbase = kv.base + e0;
+  const f16* vbase = kbase + kv.kv_stride;
+  const uint8_t* kres = kv.res + e0 / 2;
+  const uint8_t* vres = kres + kv.kv_stride / 2;
+  auto load_k = [&](int key0, int slot) {
+    load_slot<HD, true, false>(smem_u32(ring + slot * St::BYTES), kbase, kres, key0, k_end, lane);
+  };
+  auto load_v = [&](int key0, int slot) {
+    load_slot<HD, true, true>(smem_u32(ring + slot * St::BYTES), vbase, vres, key0, k_end, lane);
+  };
+  const int key_first = warp * 16;
+  load_k(key_first, 0);
+  load_v(key_first, 1);
+  load_k(key_first + NW * 16, 2);
+
+  // row g of the tile (past the last: the last again, not written) times log2(e) / sqrt(hd)
+  for (int i = warp; i < KT; i += NW) {
+    const float4* qp = reinterpret_cast<const float4*>(q + static_cast<size_t>(tile.row0 + min(g, tile.nrows - 1)) * d +
+                                                       head * HD + 32 * i + 8 * t);
+    const float4 a = __ldcg(qp), c = __ldcg(qp + 1);
+    uint4 hi, lo;
+    split_h2(a.x * scale_log2, a.y * scale_log2, hi.x, lo.x);
+    split_h2(a.z * scale_log2, a.w * scale_log2, hi.y, lo.y);
+    split_h2(c.x * scale_log2, c.y * scale_log2, hi.z, lo.z);
+    split_h2(c.z * scale_log2, c.w * scale_log2, hi.w, lo.w);
+    s_q[0][i][lane] = hi;
+    s_q[1][i][lane] = lo;
+  }
+  __syncthreads();
+
+  // of rows 2t and 2t + 1: last visible position, running maximum less 10, this lane's share of the sum;
+  // o[u][w]: dims 64 u + 8 g + 2 w (first two) and + 1, rows 2t, 2t + 1
+  int last[2];
+  float m[2], l[2], o[VT][4][4];
+#pragma unroll
+  for (int j = 0; j < 2; ++j) {
+    last[j] = tile.pos0 + min(2 * t + j, tile.nrows - 1);
+    m[j] = -INFINITY;
+    l[j] = 0.f;
+  }
+#pragma unroll
+  for (int u = 0; u < VT; ++u)
+#pragma unroll
+    for (int w = 0; w < 4; ++w) o[u][w][0] = o[u][w][1] = o[u][w][2] = o[u][w][3] = 0.f;
+
+  int slot = 0;  // of this step's keys; its values are in the next one
+  for (int key0 = key_first; key0 < k_end; key0 += NW * 16) {
+    cp_async_wait<2>();
+    __syncwarp();
+    const uint8_t* sb = ring + slot * St::BYTES;
+    float s[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+    for (int i = 0; i < KT; ++i) {
+      const uint4 ka = *reinterpret_cast<const uint4*>(sb + St::k(g, 4 * i + t));
+      const uint4 kb = *reinterpret_cast<const uint4*>(sb + St::k(g + 8, 4 * i + t));
+      const uint4 la = kv_res_lo8(ka, *reinterpret_cast<const uint32_t*>(sb + St::code(g, i) + 4 * t));
+      const uint4 lb = kv_res_lo8(kb, *reinterpret_cast<const uint32_t*>(sb + St::code(g + 8, i) + 4 * t));
+      const uint4 qh = s_q[0][i][lane], ql = s_q[1][i][lane];
+      float c[4] = {0.f, 0.f, 0.f, 0.f};
+      mma16816(c, {la.x, lb.x, la.y, lb.y}, qh.x, qh.y);
+      mma16816(c, {la.z, lb.z, la.w, lb.w}, qh.z, qh.w);
+      mma16816(c, {ka.x, kb.x, ka.y, kb.y}, ql.x, ql.y);
+      mma16816(c, {ka.z, kb.z, ka.w, kb.w}, ql.z, ql.w);
+      mma16816(c, {ka.x, kb.x, ka.y, kb.y}, qh.x, qh.y);
+      mma16816(c, {ka.z, kb.z, ka.w, kb.w}, qh.z, qh.w);
+#pragma unroll
+      for (int e = 0; e < 4; ++e) s[e] += c[e];
+    }
+    __syncwarp();  // every lane has read the slot
+    load_v(key0 + NW * 16, slot);
+    slot = slot == 2 ? 0 : slot + 1;
+    float alpha[2];
+#pragma unroll
+    for (int j = 0; j < 2; ++j) {
+      if (key0 + g > last[j]) s[j] = -INFINITY;
+      if (key0 + g + 8 > last[j]) s[2 + j] = -INFINITY;
+      float mx = fmaxf(s[j], s[2 + j]);
+#pragma unroll
+      for (int x = 4; x <= 16; x <<= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, x));
+      const float m_new = fmaxf(m[j], mx - 10.f);
+      const float ref = m_new != -INFINITY ? m_new : 0.f;  // no key of this row yet
+      alpha[j] = exp2f(m[j] - ref);
+      m[j] = m_new;
+      s[j] = exp2f(s[j] - ref);
+      s[2 + j] = exp2f(s[2 + j] - ref);
+      l[j] = l[j] * alpha[j] + (s[j] + s[2 + j]);
+    }
+    uint32_t ph[2], pl[2];
+    split_h2(s[0], s[1], ph[0], pl[0]);
+    split_h2(s[2], s[3], ph[1], pl[1]);
+#pragma unroll
+    for (int j = 0; j < 2; ++j) {
+      ph[j] = transpose8(ph[j]);
+      pl[j] = transpose8(pl[j]);
+    }
+    cp_async_wait<2>();
+    __syncwarp();
+    sb = ring + slot * St::BYTES;
+#pragma unroll
+    for (int u = 0; u < VT; ++u) {
+      uint32_t hw[4][4], lw[4][4];
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        const int r = 2 * t + (j & 1) + 8 * (j >> 1);
+        const uint4 hv = *reinterpret_cast<const uint4*>(sb + St::v(r, 8 * u + g));
+        const uint4 lv = kv_res_lo8(hv, *reinterpret_cast<const uint32_t*>(sb + St::code(r, 2 * u + (g >> 2)) + 4 * (g & 3)));
+        hw[j][0] = hv.x;
+        hw[j][1] = hv.y;
+        hw[j][2] = hv.z;
+        hw[j][3] = hv.w;
+        lw[j][0] = lv.x;
+        lw[j][1] = lv.y;
+        lw[j][2] = lv.z;
+        lw[j][3] = lv.w;
+      }
+#pragma unroll
+      for (int w = 0; w < 4; ++w) {
+        float c[4] = {0.f, 0.f, 0.f, 0.f};
+        const uint32_t vh[4] = {__byte_perm(hw[0][w], hw[1][w], 0x5410), __byte_perm(hw[0][w], hw[1][w], 0x7632),
+                                __byte_perm(hw[2][w], hw[3][w], 0x5410), __byte_perm(hw[2][w], hw[3][w], 0x7632)};
+        mma16816(c, {__byte_perm(lw[0][w], lw[1][w], 0x5410), __byte_perm(lw[0][w], lw[1][w], 0x7632),
+                     __byte_perm(lw[2][w], lw[3][w], 0x5410), __byte_perm(lw[2][w], lw[3][w], 0x7632)}, ph[0], ph[1]);
+        mma16816(c, vh, pl[0], pl[1]);
+        mma16816(c, vh, ph[0], ph[1]);
+#pragma unroll
+        for (int e = 0; e < 4; ++e) o[u][w][e] = fmaf(o[u][w][e], alpha[e & 1], c[e]);
+      }
+    }
+    __syncwarp();
+    load_k(key0 + 2 * NW * 16, slot);
+    slot = slot == 2 ? 0 : slot + 1;
+  }
+  // the warps' states -> shared memory, the outputs over the rings
+  cp_async_wait<0>();
+#pragma unroll
+  for (int j = 0; j < 2; ++j)
+#pragma unroll
+    for (int x = 4; x <= 16; x <<= 1) l[j] += __shfl_xor_sync(0xffffffffu, l[j], x);
+  if (g == 0) {
+#pragma unroll
+    for (int j = 0; j < 2; ++j) {
+      s_m[warp][2 * t + j] = m[j];
+      s_l[warp][2 * t + j] = l[j];
+    }
+  }
+  __syncthreads();
+  float* mo = reinterpret_cast<float*>(sm_dec);  // [warp][row][HD]
+#pragma unroll
+  for (int u = 0; u < VT; ++u)
+#pragma unroll
+    for (int w = 0; w < 4; ++w) {
+      float* dst = mo + (warp * 8 + 2 * t) * HD + 64 * u + 8 * g + 2 * w;
+      *reinterpret_cast<float2*>(dst) = make_float2(o[u][w][0], o[u][w][2]);
+      *reinterpret_cast<float2*>(dst + HD) = make_float2(o[u][w][1], o[u][w][3]);
+    }
+  __syncthreads();
+  constexpr int CPT = 8;  // output columns of a thread at a time
+  uint32_t sat = 0;       // convex combinations of cached values: the fp16 split never saturates
+  for (int k = tid; k < tile.nrows * (HD / CPT); k += NW * 32) {
+    const int row = k / (HD / CPT), c0 = k % (HD / CPT) * CPT;
+    float mx = -INFINITY, wt[NW], lsum = 0.f;
+#pragma unroll
+    for (int w = 0; w < NW; ++w) mx = fmaxf(mx, s_m[w][row]);  // finite: warp 0 holds key 0
+#pragma unroll
+    for (int w = 0; w < NW; ++w) {
+      wt[w] = exp2f(s_m[w][row] - mx);  // 0 for a warp that saw no visible key of this row
+      lsum += wt[w] * s_l[w][row];
+    }
+    const float inv = 1.f / lsum;
+    uint32_t hi[CPT / 2], lo[CPT / 2];
+#pragma unroll
+    for (int c = 0; c < CPT; c += 2) {
+      float v0 = 0.f, v1 = 0.f;
+#pragma unroll
+      for (int w = 0; w < NW; ++w) {
+        const float2 x = *reinterpret_cast<const float2*>(mo + (w * 8 + row) * HD + c0 + c);
+        v0 += wt[w] * x.x;
+        v1 += wt[w] * x.y;
+      }
+      split_pack2(v0 * inv, v1 * inv, hi[c / 2], lo[c / 2], fp16, sat);
+    }
+    const size_t off = static_cast<size_t>(tile.row0 + row) * d + head * HD + c0;
+    *reinterpret_cast<uint4*>(out_hi + off) = make_uint4(hi[0], hi[1], hi[2], hi[3]);
+    if (write_lo) *reinterpret_cast<uint4*>(out_lo + off) = make_uint4(lo[0], lo[1], lo[2], lo[3]);
+  }
+}
+
 }  // namespace
 
 int attn_chunk_launch(const float* q, bf16* out_hi, bf16* out_lo, const AttnTile* tiles,
@@ -921,13 +1154,28 @@ int attn_chunk_launch(const float* q, bf16* out_hi, bf16* out_lo, const AttnTile
   return VLA_OK;
 }
 
-int attn_rows_launch(const float* q, bf16* out_hi, bf16* out_lo, const AttnTile* tiles, int n_tiles, KVLayout kv,
-                     int layer, int H, int hd, cudaStream_t stream, bool fp16, bool write_lo) {
+int attn_rows_launch(const float* q, bf16* out_hi, bf16* out_lo, const AttnTile* tiles, int n_tiles, int max_rows,
+                     KVLayout kv, int layer, int H, int hd, cudaStream_t stream, bool fp16, bool write_lo) {
   if (n_tiles <= 0) return VLA_OK;
-  if (!kv.res || (hd != 64 && hd != 128)) return VLA_ERR_UNSUPPORTED;
+  if (max_rows > kAttnRowsMax || !kv.res || (hd != 64 && hd != 128)) return VLA_ERR_UNSUPPORTED;
   if ((reinterpret_cast<uintptr_t>(kv.base) & 15) || (reinterpret_cast<uintptr_t>(kv.res) & 15)) return VLA_ERR_ARG;
   const float scale_log2 = 1.4426950408889634f / sqrtf(static_cast<float>(hd));
   const dim3 grid(n_tiles, H);
+  if (max_rows <= kRows8) {
+    auto go = [&](auto kern, int smem, std::atomic<uint64_t>& attr_done) {
+      if (const cudaError_t e = set_smem_limit(kern, smem, attr_done)) return e;
+      return launch_pdl(kern, grid, dim3(kDecodeWarps * 32), smem, stream, q, out_hi, out_lo, tiles, kv, layer, H,
+                        scale_log2, fp16, write_lo);
+    };
+    static std::atomic<uint64_t> done128{0}, done64{0};
+    if (hd == 128)
+      VLA_CUDA_TRY(go(attn_rows8_kernel<128>, kDecodeWarps * DecodeSlot<128, true>::RING, done128));
+    else
+      VLA_CUDA_TRY(go(attn_rows8_kernel<64>, kDecodeWarps * DecodeSlot<64, true>::RING, done64));
+    note_launch();
+    VLA_CUDA_TRY(cudaGetLastError());
+    return VLA_OK;
+  }
   if (hd == 128) {
     static std::atomic<uint64_t> attr_done{0};
     VLA_CUDA_TRY(set_smem_limit(attn_rows_kernel<128>, RowsSmem<128>::SMEM, attr_done));

@@ -437,7 +437,7 @@ int forward_layers(vla_handle* h, int M, const RowInfo* rows_dev, bool decode, i
       // the low plane of the output only where the o projection reads it; tiles of at most 16
       // rows (the score pass) on the few-row kernel
       rc = tile_rows <= kAttnRowsMax
-               ? attn_rows_launch(h->q, h->ao, h->ao + pd, h->tiles, n_tiles, h->kvl, l, H, hd, h->stream, h->fp16,
+               ? attn_rows_launch(h->q, h->ao, h->ao + pd, h->tiles, n_tiles, tile_rows, h->kvl, l, H, hd, h->stream, h->fp16,
                                   gemm_reads_lo(M, kProjO))
                : attn_chunk_tc_launch(h->q, h->ao, h->ao + pd, h->tiles, n_tiles, h->kvl, l, H, hd, h->status,
                                       h->stream, h->fp16, h->num_sms, gemm_reads_lo(M, kProjO));
@@ -1417,8 +1417,10 @@ int vla_op_attn_rows_res(const float* q, const void* kv, const void* kv_res, int
   L.kv_stride = static_cast<int64_t>(H) * L.head_stride;
   L.env_stride = 2 * L.kv_stride;
   L.layer_stride = static_cast<int64_t>(max_env) * L.env_stride;
+  int max_rows = 0;
+  for (int i = 0; i < n_tiles; ++i) max_rows = std::max(max_rows, tiles_host[4 * i + 2]);
   const int rc = attn_rows_launch(q, static_cast<bf16*>(out_hi), static_cast<bf16*>(out_lo),
-                                  reinterpret_cast<const AttnTile*>(tiles_dev), n_tiles, L, 0, H, hd, st, false, true);
+                                  reinterpret_cast<const AttnTile*>(tiles_dev), n_tiles, max_rows, L, 0, H, hd, st, false, true);
   if (rc != VLA_OK && rc != VLA_ERR_CUDA)
     return set_err(nullptr, rc, "vla_op_attn_rows_res: unsupported arguments or misaligned buffers");
   return rc;

@@ -594,3 +594,36 @@ def test_pair_gemm_f16_full_size_sampled():
     bound = (a.abs() @ w.abs().T) * 3e-5 + 1e-6
     assert torch.isfinite(Cs).all()
     assert ((Cs - ref).abs() <= bound).all(), float(((Cs - ref).abs() / bound).max())
+
+
+@pytest.mark.parametrize("hd", [128, 64])
+def test_attn_rows8_matches_fp64(hd):
+    """Tiles of at most 8 rows (the score pass): one to 8 rows after 0 to 300 positions, so that warps and
+    16-key steps without a visible key, contexts shorter than one step and the last cache position occur;
+    NaN past each env's context.  The output pair holds 2^-17 of a value below about 4."""
+    H, cap, max_env = 3, 308, 8
+    chunks = [(0, 0, 1), (1, 0, 8), (2, 7, 5), (3, 300, 8), (4, 100, 6), (5, 13, 6), (6, 15, 2), (7, 31, 3)]
+    rows = sum(n for _, _, n in chunks)
+    x = (I.normal_bf16((max_env, 2, H, cap, hd), 96, hd, 1.0).float()
+         + I.normal_bf16((max_env, 2, H, cap, hd), 96, 7 + hd, 2.0 ** -9).float()).numpy()
+    hi, packed, value = _encode_res4(x)
+    tiles, r = [], 0
+    for env, past, n in chunks:
+        hi[env, :, :, past + n:] = np.float16("nan")
+        tiles.append((env, r, n, past))
+        r += n
+    q = I.normal_bf16((rows, H * hd), 96, 1000 + hd, 1.0).float()
+    tiles_dev = torch.zeros(len(tiles) * 4, dtype=torch.int32, device="cuda")
+    oh = torch.full((rows, H * hd), float("nan"), dtype=torch.bfloat16, device="cuda")
+    ol = torch.full_like(oh, float("nan"))
+    qd, kvd, rsd = q.cuda(), torch.from_numpy(hi).cuda(), torch.from_numpy(packed).cuda()
+    assert V.vla_op_attn_rows_res(qd.data_ptr(), kvd.data_ptr(), rsd.data_ptr(), max_env, H, hd, cap, tiles, rows,
+                                  tiles_dev.data_ptr(), oh.data_ptr(), ol.data_ptr()) == 0, V.vla_last_error(None)
+    out = (oh.cpu().double() + ol.cpu().double()).reshape(rows, H, hd)
+    kv64 = torch.from_numpy(value).double()
+    for env, r0, n, past in tiles:
+        for i in range(n):
+            k, v = kv64[env, 0, :, :past + i + 1], kv64[env, 1, :, :past + i + 1]
+            sc = torch.einsum("hd,hnd->hn", q[r0 + i].reshape(H, hd).double(), k) / math.sqrt(hd)
+            o = torch.einsum("hn,hnd->hd", torch.softmax(sc, -1), v)
+            assert (out[r0 + i] - o).abs().max().item() < 4 * 2.0 ** -17 + 1e-5, (env, i)
