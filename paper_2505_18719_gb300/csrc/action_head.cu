@@ -7,6 +7,8 @@
 // bf16 parts, which hold an fp32 value in full, times the bf16 bin rows: exact products on mma.sync,
 // fp32 sums), the slices' [rows, 256] partial products meet over distributed shared memory, and CTA c
 // then owns rows c (and c + 8): scale by 1 / RMS, logsumexp, argmax (ties to the lowest bin), outputs.
+// Between decode steps the CTA that sampled a row's token also assembles the next step's row from it (its
+// embedding and first RMSNorm), a launch less per step.
 // Bound by the latency of its chain (rows, weights from L2, exchange, block reductions); two kernels,
 // with fp32 FMAs on one CTA per 32 bins x 8 rows before, took 22.5 + 4.3 us
 // at 64 rows x 4096 (cold caches), this one 12.0.
@@ -71,7 +73,7 @@ constexpr size_t head_smem(int d, int rows) {
 }
 
 template <int RPC>  // rows per CTA after the exchange: 8 * RPC rows per cluster
-__global__ void __launch_bounds__(kHeadThreads, 2) head_kernel(const HeadArgs a) {
+__global__ void __launch_bounds__(kHeadThreads) head_kernel(const HeadArgs a) {
   constexpr int ROWS = kHeadCluster * RPC;
   constexpr int DEPTH = RPC == 1 ? 4 : 3;  // 32-wide steps of weights in flight per warp
   extern __shared__ __align__(16) uint8_t head_sm[];
@@ -80,6 +82,7 @@ __global__ void __launch_bounds__(kHeadThreads, 2) head_kernel(const HeadArgs a)
   __shared__ float red_f[8];
   __shared__ ArgMax red_a[8];
   __shared__ float red_m[8];
+  __shared__ int fed_s;
   pdl_launch_dependents();
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int g = lane >> 2, tq = lane & 3;
@@ -273,8 +276,13 @@ __global__ void __launch_bounds__(kHeadThreads, 2) head_kernel(const HeadArgs a)
       if (a.bins_out) a.bins_out[out_i] = ks;
       if (a.act_out) a.act_out[out_i] = static_cast<float>(2 * ks + 1 - 256) * (1.0f / 256.0f);
       if (a.fed_out) a.fed_out[out_i] = fed;
+      fed_s = fed;
     }
     __syncthreads();  // the shared arrays are the next row's
+    // the next step's input row: every CTA of the cluster has read row r of a.h
+    if (a.next_embed)
+      token_row_256(a.next_embed + static_cast<size_t>(fed_s) * d, d, a.next_h + static_cast<size_t>(r) * d, a.next_norm,
+                    static_cast<size_t>(r) * d, red_f, a.status);
   }
   cluster_wait();  // the others are done with this CTA's shared memory
 }

@@ -835,15 +835,15 @@ int vla_decode_actions(vla_handle* h, const float* uniforms, float temperature, 
 
   for (int i = 0; i < A; ++i) {
     if (i > 0) {
+      // the head of the step before assembled this one's rows
       const RowInfo* rows_i = h->rows + static_cast<size_t>(i - 1) * B;
-      int ev = prof_begin(h, VLA_KCLASS_OTHER);
-      rc = assemble_launch(rows_i, B, nullptr, nullptr, h->fed, h->embed, d, c.vocab, h->h, first_norm(h), h->status, h->stream);
-      prof_end(h, ev, VLA_KCLASS_OTHER, 0, 6.0 * B * d);
-      if (rc) return fail(h, rc, t_err);
       if ((rc = forward_layers(h, B, rows_i, true, 0, 0, max_len_p + i))) return rc;
     }
     ha.h = (i == 0) ? h->h_last : h->h;
     ha.step = i;
+    ha.next_embed = i + 1 < A ? h->embed : nullptr;
+    ha.next_h = h->h;
+    ha.next_norm = first_norm(h);
     int ev = prof_begin(h, VLA_KCLASS_HEAD);
     rc = action_head_launch(ha, h->stream);
     prof_end(h, ev, VLA_KCLASS_HEAD, 2.0 * B * 256 * d, 2.0 * 256 * d + 4.0 * B * d);

@@ -35,35 +35,9 @@ __global__ void __launch_bounds__(256) assemble_kernel(const RowInfo* __restrict
     }
     src = embed + static_cast<size_t>(id) * d;
   }
-  float* dst = h + static_cast<size_t>(blockIdx.x) * d;
-  float ss = 0.f;
-  for (int c = threadIdx.x * 4; c < d; c += blockDim.x * 4) {
-    const uint2 x = *reinterpret_cast<const uint2*>(src + c);
-    const float2 a = unpack_bf16x2(x.x), b = unpack_bf16x2(x.y);
-    const float4 v = make_float4(a.x, a.y, b.x, b.y);
-    *reinterpret_cast<float4*>(dst + c) = v;
-    ss += v.x * v.x + v.y * v.y + v.z * v.z + v.w * v.w;
-  }
-  // the first layer's RMSNorm of the row, in rmsnorm_kernel's order (the source row again, from L1)
   __shared__ float red[8];
-  ss = warp_sum(ss);
-  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = ss;
-  __syncthreads();
-  float tot = 0.f;
-  for (int i = 0; i < (blockDim.x >> 5); ++i) tot += red[i];
-  const float r = rsqrtf(tot / static_cast<float>(d) + nm.eps);
   const size_t off = static_cast<size_t>(blockIdx.x) * d;
-  uint32_t sat = 0;
-  for (int c = threadIdx.x * 4; c < d; c += blockDim.x * 4) {
-    const uint2 x = *reinterpret_cast<const uint2*>(src + c), ww = *reinterpret_cast<const uint2*>(nm.w + c);
-    const float2 a = unpack_bf16x2(x.x), b = unpack_bf16x2(x.y), w0 = unpack_bf16x2(ww.x), w1 = unpack_bf16x2(ww.y);
-    uint2 hi, lo;
-    split_pack2(a.x * r * w0.x, a.y * r * w0.y, hi.x, lo.x, nm.fp16, sat);
-    split_pack2(b.x * r * w1.x, b.y * r * w1.y, hi.y, lo.y, nm.fp16, sat);
-    *reinterpret_cast<uint2*>(nm.y_hi + off + c) = hi;
-    *reinterpret_cast<uint2*>(nm.y_lo + off + c) = lo;
-  }
-  report_saturation(status, sat);
+  token_row_256(src, d, h + off, nm, off, red, status);
 }
 
 // y = h * rsqrt(mean square + eps) * w of a row whose sums of squares over 128-column blocks are at hand:

@@ -4,9 +4,7 @@
 
 namespace vla {
 
-// h[r] (f32 [rows, d]) = source row of RowInfo r: visual (bf16 row idx), text (embed[ids[idx]])
-// or token (embed[tokens[idx]]).  Ids outside [0, vocab) -> VLA_STATUS_BAD_TOKEN, row 0.
-// The rows' RMSNorm with weight norm.w goes to norm.y_hi / y_lo [rows, d] as the operand pair.
+// First RMSNorm of assembled rows: weight w, the operand pair y_hi / y_lo [rows, d].
 struct FirstNorm {
   const bf16* w;
   float eps;
@@ -14,6 +12,41 @@ struct FirstNorm {
   bf16* y_lo;
   bool fp16;
 };
+// One 256-thread CTA: the bf16 row src as fp32 to h, and its RMSNorm to the pair at element `off`, summed in
+// rmsnorm_kernel's order (the second read of src comes from L1).  red: 8 floats of shared memory, free on
+// entry; free again once every thread has returned and met at a barrier.
+__device__ __forceinline__ void token_row_256(const bf16* src, int d, float* h, const FirstNorm& nm, size_t off, float* red,
+                                              uint32_t* status) {
+  float ss = 0.f;
+  for (int c = threadIdx.x * 4; c < d; c += 1024) {
+    const uint2 x = *reinterpret_cast<const uint2*>(src + c);
+    const float2 a = unpack_bf16x2(x.x), b = unpack_bf16x2(x.y);
+    const float4 v = make_float4(a.x, a.y, b.x, b.y);
+    *reinterpret_cast<float4*>(h + c) = v;
+    ss += v.x * v.x + v.y * v.y + v.z * v.z + v.w * v.w;
+  }
+  ss = warp_sum(ss);
+  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = ss;
+  __syncthreads();
+  float tot = 0.f;
+  for (int i = 0; i < 8; ++i) tot += red[i];
+  const float r = rsqrtf(tot / static_cast<float>(d) + nm.eps);
+  uint32_t sat = 0;
+  for (int c = threadIdx.x * 4; c < d; c += 1024) {
+    const uint2 x = *reinterpret_cast<const uint2*>(src + c), ww = *reinterpret_cast<const uint2*>(nm.w + c);
+    const float2 a = unpack_bf16x2(x.x), b = unpack_bf16x2(x.y), w0 = unpack_bf16x2(ww.x), w1 = unpack_bf16x2(ww.y);
+    uint2 hi, lo;
+    split_pack2(a.x * r * w0.x, a.y * r * w0.y, hi.x, lo.x, nm.fp16, sat);
+    split_pack2(b.x * r * w1.x, b.y * r * w1.y, hi.y, lo.y, nm.fp16, sat);
+    *reinterpret_cast<uint2*>(nm.y_hi + off + c) = hi;
+    *reinterpret_cast<uint2*>(nm.y_lo + off + c) = lo;
+  }
+  report_saturation(status, sat);
+}
+
+// h[r] (f32 [rows, d]) = source row of RowInfo r: visual (bf16 row idx), text (embed[ids[idx]])
+// or token (embed[tokens[idx]]).  Ids outside [0, vocab) -> VLA_STATUS_BAD_TOKEN, row 0.
+// The rows' RMSNorm with weight norm.w goes to norm.y_hi / y_lo [rows, d] as the operand pair.
 int assemble_launch(const RowInfo* rows, int n_rows, const bf16* visual, const int* ids,
                     const int* tokens, const bf16* embed, int d, int vocab, float* h, const FirstNorm& norm,
                     uint32_t* status, cudaStream_t s);
@@ -64,6 +97,11 @@ struct HeadArgs {
   int* fed_out = nullptr;           // [B, A] token fed to the next step (forced or sampled)
   float* entropy_out = nullptr;     // [B, A] entropy of each token's bin distribution
   uint32_t* status = nullptr;
+  // decode steps with a next one (n_pos == 1): the row of the token fed next, per env, as assemble_launch
+  // would write it (next_embed null: none)
+  const bf16* next_embed = nullptr;
+  float* next_h = nullptr;
+  FirstNorm next_norm{};
 };
 int action_head_launch(const HeadArgs& a, cudaStream_t s);
 
