@@ -318,11 +318,13 @@ int run_gemm(vla_handle* h, int cls, const bf16* A, size_t a_plane, int lda, con
     g.epi.row_d = K;
     g.epi.row_eps = h->cfg.rms_eps;
   }
+  const bool wide = !stream_k && g.splits == 1 && g.block_n == 128 && gemm_wide_ok(g, h->num_sms);
   if (h->ev_used.size() > 8192) prof_harvest(h);
   int ev = prof_begin(h, cls);
   GemmCost cost{0, 0};
   int rc = stream_k ? gemv_launch(g, h->stream, h->num_sms, &cost)
-                    : gemm_launch(g, h->stream, h->num_sms, &cost);
+                    : wide   ? gemm_wide_launch(g, h->stream, &cost)
+                             : gemm_launch(g, h->stream, h->num_sms, &cost);
   prof_end(h, ev, cls, cost.flops, cost.bytes);
   if (rc != VLA_OK) return fail(h, rc, t_err.empty() ? "gemm launch failed" : t_err);
   if (consume) h->y_deferred = false;

@@ -96,6 +96,11 @@ size_t gemv_workspace_bytes(int M, int N, int K, int num_sms);
 bool make_tensor_map_2d(CUtensorMap* m, const void* ptr, int64_t rows, int64_t cols, int64_t ld, int box_rows,
                         bool fp16);
 
+// Residual GEMM of a few hundred rows with K split over clusters, for calls that would run as unsplit
+// 128-column tiles: same arguments and results as gemm_launch there.
+bool gemm_wide_ok(const GemmArgs& a, int num_sms);
+int gemm_wide_launch(const GemmArgs& a, cudaStream_t stream, GemmCost* cost);
+
 // Failure injection (test hook): in the next single-CTA tile GEMM launch, CTA 0 leaves its first
 // pipeline stage unfilled; its bounded wait on that stage runs out (VLA_STATUS_TIMEOUT).
 void gemm_stall_next_launch();

@@ -1747,6 +1747,242 @@ __global__ void __launch_bounds__(kThreads, 2)
   cluster_wait();  // no CTA leaves while its partials are still being sent
 }
 
+// ----------------------------------------------------------------------------- residual GEMM, wide
+// o and down of a few hundred rows (the score pass: 6 rows of each env).  An SM takes in about 85 GB/s from
+// L2, which bounds 128 x 128 tiles (32 KB of operands per 2 MFLOP) at a quarter of the tensor rate, on the
+// 96 of 152 SMs that 384 x 4096 outputs give such tiles.  Here a tile is 128 weight rows by ALL rows of the
+// call (64 KB per 6.3 MFLOP), the weights as the MMA's M like in the decode GEMMs, and a cluster splits K:
+// each CTA stores its fp32 partial rows from TMEM into the shared memory of the CTA that finishes them
+// (over the stages, once every CTA of the cluster is done with its own), which adds them in rank order and
+// applies the residual add and the deferred RMSNorm's outputs.
+// 384 rows, 4096 x 11008: 40 us against 70 of the tile GEMM; 4096 x 4096: 28 against 28 alone with cold
+// caches, but 9 us less in the pass, where its first weights are requested early (score pass of 64 envs, two
+// 7B layers: 645 us, 604 with down here, 586 with both).  A shorter K leaves less than the exchange costs
+// (about 15 us).  Below kWideMin rows the tiles stay: a prefill of one env (289 rows, 1661 against 1621 us a
+// turn of two 7B layers) would gain little, and its rows would round otherwise than in a larger batch's.
+constexpr int kWideMin = 320;
+constexpr int kWideMinK = 4096;
+constexpr int kWideRows = 432;      // the exchange of (rows + 3) x 128 fp32 fits shared memory
+constexpr int kWideC = 4;
+constexpr int kWideThreads = 320;   // producer, MMA issuer, eight warps that move and finish the sums
+constexpr int kWideStages = 3;
+constexpr int kWideFinish = 4;
+struct WideParams {
+  int M, nb, kbt;  // nb: rows per MMA (the call's rows as two halves), a multiple of 16
+  EpiArgs epi;
+  uint64_t wait_limit;
+};
+__device__ __forceinline__ void st_cluster(uint32_t addr, float v) {
+  asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(addr), "f"(v) : "memory");
+}
+
+__global__ void __launch_bounds__(kWideThreads, 1)
+    gemm_wide_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ CUtensorMap tmX, const WideParams p) {
+  constexpr int TR = 128, W_BYTES = TR * BK * 2, C = kWideC, STAGES = kWideStages;
+  const int x_half = p.nb * BK * 2;  // a multiple of 2 KB: swizzle atoms stay aligned
+  const int stage_bytes = W_BYTES + 2 * x_half;
+  constexpr uint32_t TMEM_COLS = 512;
+  const uint32_t IDESC = idesc_for((1u << 4) | (1u << 7) | (1u << 10) | (static_cast<uint32_t>(p.nb >> 3) << 17) |
+                                       (static_cast<uint32_t>(128 >> 4) << 24),
+                                   p.epi.fp16);
+  extern __shared__ uint8_t smem_raw[];
+  uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) &
+                                             ~static_cast<uintptr_t>(1023));
+  uint64_t* bars = reinterpret_cast<uint64_t*>(smem);  // one 1 KB block, then the stages
+  smem += 1024;
+  const uint32_t full0 = smem_u32(bars);
+  const uint32_t empty0 = full0 + 8 * STAGES;
+  const uint32_t done_bar = empty0 + 8 * STAGES;
+  const uint32_t recv_bar = done_bar + 8;
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 2 * STAGES + 2);
+  volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
+
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int rank = static_cast<int>(cluster_ctarank());
+  const int tile = blockIdx.x / C;
+  const int kb0 = p.kbt * rank / C, kb1 = p.kbt * (rank + 1) / C;
+  int ok = 1;
+  if (threadIdx.x == 0) {
+    for (int s = 0; s < STAGES; ++s) {
+      mbar_init(full0 + 8 * s, 1);
+      mbar_init(empty0 + 8 * s, 1);
+    }
+    mbar_init(done_bar, 1);
+    mbar_init(recv_bar, 8 * C);  // each CTA's eight epilogue warps
+    *abort_flag = 0;
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&tmW)) : "memory");
+    asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&tmX)) : "memory");
+  }
+  if (warp == 1) {
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_slot)),
+                 "r"(TMEM_COLS)
+                 : "memory");
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+  }
+  tc_fence_before();
+  __syncthreads();
+  tc_fence_after();
+  pdl_launch_dependents();
+  const uint32_t tmem_base = *tmem_slot;
+  uint32_t* status = p.epi.status;
+  const uint64_t limit = p.wait_limit;
+
+  if (warp == 0) {
+    if (lane == 0) {
+      const int n = kb1 - kb0;
+      const int pre = n < STAGES ? n : STAGES;
+      uint32_t issued = 0, issued_phase = 0;
+      auto load_w = [&](int stage, int kb) {
+        mbar_arrive_expect_tx(full0 + 8 * stage, stage_bytes);
+        tma_load_2d(smem_u32(smem + stage * stage_bytes), &tmW, full0 + 8 * stage, kb * BK, tile * TR);
+      };
+      auto load_x = [&](int stage, int kb) {
+        const uint32_t sx = smem_u32(smem + stage * stage_bytes) + W_BYTES;
+        tma_load_2d(sx, &tmX, full0 + 8 * stage, kb * BK, 0);
+        tma_load_2d(sx + x_half, &tmX, full0 + 8 * stage, kb * BK, p.nb);
+      };
+      for (int i = 0; i < pre; ++i) {  // the weights do not depend on the previous kernel
+        load_w(i, kb0 + i);
+        issued |= 1u << i;
+      }
+      pdl_wait_async();
+      for (int i = 0; i < pre; ++i) load_x(i, kb0 + i);
+      int stage = pre % STAGES;
+      uint32_t phase = (pre == STAGES) ? 1u : 0u;
+      for (int i = pre; i < n; ++i) {
+        if (!wait_bounded(empty0 + 8 * stage, phase ^ 1u, abort_flag, status, limit)) break;
+        load_w(stage, kb0 + i);
+        load_x(stage, kb0 + i);
+        issued_phase = (issued_phase & ~(1u << stage)) | (phase << stage);
+        if (++stage == STAGES) {
+          stage = 0;
+          phase ^= 1u;
+        }
+      }
+      for (int s = 0; s < STAGES; ++s)
+        if (issued & (1u << s)) wait_drain(full0 + 8 * s, (issued_phase >> s) & 1u, limit);
+    }
+  } else if (warp == 1) {
+    if (lane == 0) {
+      int stage = 0;
+      uint32_t phase = 0;
+      for (int kb = kb0; kb < kb1; ++kb) {
+        if (!wait_bounded(full0 + 8 * stage, phase, abort_flag, status, limit)) break;
+        tc_fence_after();
+        const uint32_t sw = smem_u32(smem + stage * stage_bytes);
+        const uint32_t sx = sw + W_BYTES;
+#pragma unroll
+        for (int k = 0; k < BK / 16; ++k) {
+          const uint64_t w = make_sdesc(sw + k * 32);
+          const uint32_t acc = (kb > kb0 || k > 0) ? 1u : 0u;
+          tc_mma(tmem_base, w, make_sdesc(sx + k * 32), IDESC, acc);
+          tc_mma(tmem_base + 256, w, make_sdesc(sx + x_half + k * 32), IDESC, acc);
+        }
+        tc_commit(empty0 + 8 * stage);
+        if (++stage == STAGES) {
+          stage = 0;
+          phase ^= 1u;
+        }
+      }
+      tc_commit(done_bar);
+      wait_drain(done_bar, 0, limit);
+    }
+  } else {
+    if (lane == 0) ok = wait_bounded(done_bar, 0, abort_flag, status, limit) && !*abort_flag ? 1 : 0;
+    ok = __shfl_sync(0xffffffffu, ok, 0);
+  }
+  __syncwarp();
+  cluster_arrive();
+  cluster_wait();  // every CTA is done with its stages: partials may be stored over them
+  const int ml = (p.M + C - 1) / C;  // rows per rank
+  float* recv = reinterpret_cast<float*>(smem);  // [rank][ml][TR]
+  if (warp >= 2) {
+    // for each row the 32 lanes of a warp store 32 consecutive floats (an aborted CTA arrives too)
+    if (ok) {
+      tc_fence_after();
+      const int q = warp & 3, half = (warp - 2) >> 2;  // TMEM lane quarter; half of the rows
+      const uint32_t mine = smem_u32(recv + rank * ml * TR + q * 32 + lane);
+      const uint32_t trow = tmem_base + (static_cast<uint32_t>(q * 32) << 16) + half * 256;
+      const int m0 = half * p.nb, n_m = min(p.nb, p.M - m0);
+      int dst = m0 / ml, i = m0 - dst * ml;
+      uint32_t to = mapa_shared(mine, dst);
+#pragma unroll 1
+      for (int c = 0; c < n_m; c += 16) {
+        float v[16];
+        ld16f(trow + c, v);
+#pragma unroll
+        for (int k = 0; k < 16; ++k) {
+          if (c + k >= n_m) break;
+          st_cluster(to + static_cast<uint32_t>(i * TR * 4), v[k]);
+          if (++i == ml) {
+            i = 0;
+            if (++dst < C) to = mapa_shared(mine, dst);
+          }
+        }
+      }
+      tc_fence_before();
+    }
+    __syncwarp();
+    if (lane < C) mbar_arrive_cluster(mapa_shared(recv_bar, lane));
+  }
+  pdl_wait();  // (long over) the residual is the previous kernels'
+  const EpiArgs& e = p.epi;
+  const int r0 = rank * ml, mn = max(0, min(ml, p.M - r0));
+  uint32_t sat = 0;
+  bool waited = false;
+  for (int k0 = threadIdx.x; k0 < mn * 32; k0 += kWideThreads * kWideFinish) {
+    float4 h[kWideFinish];
+#pragma unroll
+    for (int u = 0; u < kWideFinish; ++u) {
+      const int k = k0 + u * kWideThreads;
+      if (k < mn * 32)
+        h[u] = __ldcg(reinterpret_cast<const float4*>(e.resid + static_cast<size_t>(r0 + (k >> 5)) * e.ldr + tile * TR + (k & 31) * 4));
+    }
+    if (!waited) wait_cluster_data(recv_bar, 0, status, limit);
+    waited = true;
+#pragma unroll
+    for (int u = 0; u < kWideFinish; ++u) {
+      const int k = k0 + u * kWideThreads;
+      if (k >= mn * 32) continue;  // a warp's 32 items are one row's 128 columns
+      const int i = k >> 5, c = (k & 31) * 4, n = tile * TR + c;
+      float4 a = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+      for (int s = 0; s < C; ++s) {
+        const float4 v = *reinterpret_cast<const float4*>(recv + (s * ml + i) * TR + c);
+        a.x += v.x;
+        a.y += v.y;
+        a.z += v.z;
+        a.w += v.w;
+      }
+      const float4 x = make_float4(h[u].x + a.x, h[u].y + a.y, h[u].z + a.z, h[u].w + a.w);
+      *reinterpret_cast<float4*>(e.resid + static_cast<size_t>(r0 + i) * e.ldr + n) = x;
+      if (e.ss_out) {
+        const float ss = warp_sum(x.x * x.x + x.y * x.y + x.z * x.z + x.w * x.w);
+        if (lane == 0) e.ss_out[static_cast<size_t>(tile) * p.M + r0 + i] = ss;
+        const uint2 ww = *reinterpret_cast<const uint2*>(e.norm_w + n);
+        const float2 w0 = unpack_bf16x2(ww.x), w1 = unpack_bf16x2(ww.y);
+        uint2 hi, lo;
+        split_pack2(x.x * w0.x, x.y * w0.y, hi.x, lo.x, e.fp16, sat);
+        split_pack2(x.z * w1.x, x.w * w1.y, hi.y, lo.y, e.fp16, sat);
+        const size_t off = static_cast<size_t>(r0 + i) * e.ldn + n;
+        *reinterpret_cast<uint2*>(e.norm_hi + off) = hi;
+        if (e.norm_lo) *reinterpret_cast<uint2*>(e.norm_lo + off) = lo;
+      }
+    }
+  }
+  if (!waited) wait_cluster_data(recv_bar, 0, status, limit);
+  report_saturation(status, sat);
+  __syncthreads();  // TMEM has been read
+  cluster_arrive();
+  if (warp == 1) {
+    tc_fence_after();
+    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(TMEM_COLS)
+                 : "memory");
+  }
+  cluster_wait();  // no CTA leaves before all have what they were sent (or gave up waiting)
+}
+
 // ----------------------------------------------------------------------------- host side
 typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*,
                                   const cuuint64_t*, const cuuint64_t*, const cuuint32_t*,
@@ -2154,6 +2390,39 @@ int gemm_launch(const GemmArgs& a, cudaStream_t stream, int num_sms, GemmCost* c
 size_t gemv_workspace_bytes(int M, int N, int K, int num_sms) {
   if (M < 1 || M > 128) return 0;
   return stream_plan(M, N, K, num_sms).ws_bytes;
+}
+
+bool gemm_wide_ok(const GemmArgs& a, int num_sms) {
+  return a.epi.kind == EPI_RESID && !a.A_lo && a.M > kWideMin && a.M <= kWideRows && a.N % 128 == 0 &&
+         a.N / 128 * kWideC <= num_sms * 17 / 20 && a.K >= kWideMinK && a.lda % 8 == 0 && a.ldb % 8 == 0 && a.epi.ldr % 4 == 0 &&
+         !((reinterpret_cast<uintptr_t>(a.A) | reinterpret_cast<uintptr_t>(a.B) | reinterpret_cast<uintptr_t>(a.epi.resid)) & 15) &&
+         (!a.epi.norm_w || (a.epi.ss_out && a.epi.norm_hi && a.epi.ldn % 4 == 0 &&
+                            !((reinterpret_cast<uintptr_t>(a.epi.norm_w) | reinterpret_cast<uintptr_t>(a.epi.norm_hi) |
+                               reinterpret_cast<uintptr_t>(a.epi.norm_lo)) & 7)));
+}
+
+int gemm_wide_launch(const GemmArgs& a, cudaStream_t stream, GemmCost* cost) {
+  WideParams p{};
+  p.M = a.M;
+  p.nb = ((a.M + 1) / 2 + 15) / 16 * 16;
+  p.kbt = (a.K + BK - 1) / BK;
+  p.epi = a.epi;
+  p.wait_limit = g_wait_limit_ns.load(std::memory_order_relaxed);
+  CUtensorMap mw, mx;
+  if (!make_map(&mw, a.B, a.N, a.K, a.ldb, 128, a.epi.fp16) || !make_map(&mx, a.A, a.M, a.K, a.lda, p.nb, a.epi.fp16))
+    return cuda_fail(cudaErrorInvalidValue, "tensor maps (wide GEMM)");
+  const int stage = 128 * BK * 2 + 2 * p.nb * BK * 2;
+  const int recv = (a.M + kWideC - 1) / kWideC * kWideC * 128 * 4;
+  const int smem = std::max(kWideStages * stage, recv) + 2048;
+  constexpr int smem_max = 227 * 1024;
+  static std::atomic<uint64_t> attr_done{0};
+  VLA_CUDA_TRY(set_smem_limit(gemm_wide_kernel, smem_max, attr_done));
+  VLA_CUDA_TRY(launch_pdl_cluster(gemm_wide_kernel, dim3(a.N / 128 * kWideC), dim3(kWideThreads), smem, stream, kWideC, mw,
+                                  mx, p));
+  note_launch();
+  VLA_CUDA_TRY(cudaGetLastError());
+  if (cost) *cost = gemm_cost(a);
+  return VLA_OK;
 }
 
 bool gemv_fuses_norm(int M) { return M > kClusterRows; }

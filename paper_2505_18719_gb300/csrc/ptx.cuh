@@ -204,6 +204,26 @@ __device__ __forceinline__ void wait_drain(uint32_t bar, uint32_t parity, uint64
     if (globaltimer() - t0 > limit_ns) return;
   }
 }
+// Wait for what other CTAs of the cluster stored before they arrived on this CTA's barrier; one that
+// runs out reports the timeout.
+__device__ __forceinline__ void wait_cluster_data(uint32_t bar, uint32_t parity, uint32_t* status, uint64_t limit_ns) {
+  const uint64_t t0 = globaltimer();
+  while (true) {
+    uint32_t ok;
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t"
+        "mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n\t"
+        "selp.u32 %0, 1, 0, p;\n\t}"
+        : "=r"(ok)
+        : "r"(bar), "r"(parity)
+        : "memory");
+    if (ok) return;
+    if (globaltimer() - t0 > limit_ns) {
+      if (status) atomicOr(status, VLA_STATUS_TIMEOUT);
+      return;
+    }
+  }
+}
 // The same for data that has to arrive: a wait that runs out reports the timeout.
 __device__ __forceinline__ void wait_drain_reported(uint32_t bar, uint32_t parity, uint32_t* status, uint64_t limit_ns) {
   const uint64_t t0 = globaltimer();

@@ -126,3 +126,25 @@ def test_decode_attention_whole_pairs_and_a_split_rest(weights):
         pol.close()
     rep = P.compare_decode(0, local, od, g)
     assert rep.ok(), rep
+
+
+@pytest.mark.parametrize("B", [53, 54, 64, 71, 72, 73])
+def test_score_matches_decode_around_the_wide_residual_gemm(B):
+    # 6 B score rows: 318 (tile GEMMs), 324 to 432 (o and down on the wide GEMM: an odd split of the rows over
+    # four ranks and padded halves among them), 438 (tile GEMMs again).  The decode runs on activation
+    # pairs throughout, the score pass on fp16 activations past q|k|v: 2^-11 a layer and projection
+    sh = I.ModelShape("tiny", 2, 4096, 32, 128, 4616)
+    w = P.weights_to_device(I.make_weights(sh, 11))
+    ids = I.randint_i32((B, 9), 5, 16, 0, sh.vocab - 257)
+    tokens = I.randint_i32((B, sh.action_dim), 5, 17, sh.vocab - 256, sh.vocab - 1).cuda()
+    u = I.uniform_f32((B, sh.action_dim, 256), 5, 18).cuda()
+    pol = V.Policy(sh, w, B, 32, B * 9)
+    try:
+        pol.prefill(None, ids.cuda(), [1 + b % 9 for b in range(B)])
+        d = pol.decode(u, 1.0, forced=tokens)["logits"].double()
+        s = pol.score(tokens, 1.0)["logits"].double()
+        pol.sync()
+    finally:
+        pol.close()
+    assert ((s - d).norm() / d.norm()).item() < 2e-3
+    assert (s - d).abs().max().item() < 0.02 * d.abs().max().item()
