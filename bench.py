@@ -225,7 +225,7 @@ CASES = {
     "gemm_prefill_down": (4608, 4096, 11008, 256, 1, True),
     "gemm_decode_qkv": (64, 12288, 4096, 128, 2, True),        # one decode step, 64 envs
     "gemm_decode_o": (64, 4096, 4096, 128, 5, True),
-    # weight-streaming decode GEMM (swap-AB, stream-K): block_n / splits unused
+    # weight-streaming decode GEMM (swap-AB): block_n / splits unused
     "gemv_decode_qkv": (64, 12288, 4096, 0, 0, True),
     "gemv_decode_o": (64, 4096, 4096, 0, 0, True),
     "gemv_decode_gate_up": (64, 22016, 4096, 0, 0, True),
@@ -706,7 +706,7 @@ def main():
     roof_dec = None
     if gd["ms"] > 0:
         gbs = gd["bytes"] / (gd["ms"] / 1e3) / 1e9
-        roof_dec = {"bound": "hbm", "kernel": "gemv_tc + stream-K reduction (decode projections)",
+        roof_dec = {"bound": "hbm", "kernel": "gemv_stream + stream-K reduction (decode projections)",
                     "achieved": gbs, "peak": hbm, "unit": "GB/s", "frac": gbs / hbm,
                     "peak_kind": f"{peak_kind} HBM copy",
                     "note": "each launch bracketed by events, which also stops it overlapping its neighbours",

@@ -40,9 +40,10 @@ int vla_op_gemm_pair_bf16(const void* A, const void* A_lo, int lda, const void* 
 
 /* The decode-step projection (§3.1 projections at decode batch sizes, Algorithm 1 rollout):
  * C[M, N] (f32) = (A + A_lo)[M, K] · W[N, K]^T for M <= 128 activation rows, bf16 operands,
- * A_lo required.  Streams W from HBM once: swap-AB tcgen05 MMAs (W rows are the MMA's M),
- * stream-K over the 128-row weight tiles, fp32 partials in `workspace` (at least
- * vla_op_gemm_decode_workspace_bytes(M, N, K) bytes), fixed-order reduction into C.
+ * A_lo required.  Streams W from HBM once: swap-AB tcgen05 MMAs (W rows are the MMA's M).  Up to 32
+ * rows a cluster splits K and sums in shared memory; above, stream-K over the weight tiles with fp32
+ * partials in `workspace` and a fixed-order reduction into C.  `workspace` holds at least
+ * vla_op_gemm_decode_workspace_bytes(M, N, K) bytes at every M.
  * VLA_ERR_ARG for M > 128, NULL pointers or a short workspace. */
 int vla_op_gemm_decode_bf16(const void* A, const void* A_lo, int lda, const void* W, int ldw,
                             float* C, int ldc, int M, int N, int K, float* workspace,
@@ -172,8 +173,8 @@ int vla_op_attn_chunk_res(const float* q, const void* kv, const void* kv_res, in
 /* The same attention for short tiles, the engine's kernel when every tile has at most 16 rows
  * (the PPO ratio pass of Eq. 2: A - 1 teacher-forced rows per env): arguments as
  * vla_op_attn_chunk_res, with 1 <= nrows <= 16 per tile (VLA_ERR_ARG otherwise, nothing runs).
- * mma.sync on one CTA per (tile, head): each cached byte is read once per tile and head, and no
- * MMA row past the 16th is spent; same results to fp32 rounding order. */
+ * mma.sync on one CTA per (tile, head): each cached byte is read once per tile and head (calls whose
+ * tiles have at most 8 rows run on a kernel of their own); same results to fp32 rounding order. */
 int vla_op_attn_rows_res(const float* q, const void* kv, const void* kv_res, int max_env, int H, int hd,
                          int cap, const int32_t* tiles_host, int n_tiles, int rows, int32_t* tiles_dev,
                          void* out_hi, void* out_lo, void* cuda_stream);
