@@ -72,8 +72,11 @@ constexpr size_t head_smem(int d, int rows) {
   return static_cast<size_t>(rows) * head_stride(head_slice(d)) * 3 * 2 + static_cast<size_t>(rows) * kPartStride * 4;
 }
 
-template <int RPC>  // rows per CTA after the exchange: 8 * RPC rows per cluster
-__global__ void __launch_bounds__(kHeadThreads) head_kernel(const HeadArgs a) {
+// RPC: rows per CTA after the exchange, 8 * RPC rows per cluster.  FIRST: the rows come from two places
+// (h_first).  Two CTAs per SM only where the grid needs them (RPC 2: 448 rows are 224 CTAs): the 128 registers
+// that leaves cost a few spills.
+template <int RPC, bool FIRST>
+__global__ void __launch_bounds__(kHeadThreads, RPC) head_kernel(const HeadArgs a) {
   constexpr int ROWS = kHeadCluster * RPC;
   constexpr int DEPTH = RPC == 1 ? 4 : 3;  // 32-wide steps of weights in flight per warp
   extern __shared__ __align__(16) uint8_t head_sm[];
@@ -117,6 +120,11 @@ __global__ void __launch_bounds__(kHeadThreads) head_kernel(const HeadArgs a) {
   for (int j = 0; j < RPC; ++j) {
     const int i = warp * RPC + j, r = r0 + i;
     const float* hrow = a.h + static_cast<size_t>(r) * a.ldh;
+    if (FIRST && r < R) {
+      const int b = r / a.n_pos, pos = r - b * a.n_pos;
+      hrow = pos == 0 ? a.h_first + static_cast<size_t>(b) * a.ldh
+                      : a.h + static_cast<size_t>(b * (a.n_pos - 1) + pos - 1) * a.ldh;
+    }
     float ss = 0.f;
 #pragma unroll 4
     for (int c = lane * 4; c < slice; c += 128) {
@@ -276,6 +284,8 @@ __global__ void __launch_bounds__(kHeadThreads) head_kernel(const HeadArgs a) {
       if (a.bins_out) a.bins_out[out_i] = ks;
       if (a.act_out) a.act_out[out_i] = static_cast<float>(2 * ks + 1 - 256) * (1.0f / 256.0f);
       if (a.fed_out) a.fed_out[out_i] = fed;
+      // the env's last token stays pending (a scored one as given, its range is checked when it is fed)
+      if (a.pending_out && out_i == b * a.A + a.A - 1) a.pending_out[b] = FIRST ? a.forced[out_i] : fed;
       fed_s = fed;
     }
     __syncthreads();  // the shared arrays are the next row's
@@ -292,7 +302,7 @@ __global__ void __launch_bounds__(kHeadThreads) head_kernel(const HeadArgs a) {
 int action_head_launch(const HeadArgs& a, cudaStream_t s) {
   if (a.B <= 0) return VLA_OK;
   if (a.d % 8 || a.ldh % 4 || (reinterpret_cast<uintptr_t>(a.h) & 15) ||
-      (reinterpret_cast<uintptr_t>(a.head_rows) & 15) || (reinterpret_cast<uintptr_t>(a.final_norm) & 7))
+      (reinterpret_cast<uintptr_t>(a.h_first) & 15) || (reinterpret_cast<uintptr_t>(a.head_rows) & 15) || (reinterpret_cast<uintptr_t>(a.final_norm) & 7))
     return VLA_ERR_UNSUPPORTED;
   if (a.d > kHeadMaxD) return VLA_ERR_UNSUPPORTED;
   const int R = a.B * a.n_pos;
@@ -301,11 +311,12 @@ int action_head_launch(const HeadArgs& a, cudaStream_t s) {
     return launch_pdl_cluster(kern, dim3((R + rows - 1) / rows * kHeadCluster), dim3(kHeadThreads), head_smem(a.d, rows),
                               s, kHeadCluster, a);
   };
-  static std::atomic<uint64_t> done1{0}, done2{0};
+  static std::atomic<uint64_t> done[4];
   if (R <= kHeadSmallRows) {
-    VLA_CUDA_TRY(go(head_kernel<1>, kHeadCluster, done1));
+    VLA_CUDA_TRY(a.h_first ? go(head_kernel<1, true>, kHeadCluster, done[0]) : go(head_kernel<1, false>, kHeadCluster, done[1]));
   } else {
-    VLA_CUDA_TRY(go(head_kernel<2>, 2 * kHeadCluster, done2));
+    VLA_CUDA_TRY(a.h_first ? go(head_kernel<2, true>, 2 * kHeadCluster, done[2])
+                           : go(head_kernel<2, false>, 2 * kHeadCluster, done[3]));
   }
   note_launch();
   VLA_CUDA_TRY(cudaGetLastError());

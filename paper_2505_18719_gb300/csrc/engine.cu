@@ -145,7 +145,6 @@ struct vla_handle {
   float* ws = nullptr;
   size_t ws_bytes = 0;
   float* h_last = nullptr;
-  float* head_in = nullptr;
   float* head_entropy = nullptr;  // entropy of each action token's distribution [B, A]
   bool entropy_valid = false;     // set by decode / score, cleared by prefill / reset
   float* q_last = nullptr;  // last layer of a prefill: queries of each env's final row [B, d]
@@ -159,7 +158,6 @@ struct vla_handle {
   RowInfo* rows = nullptr;
   AttnTile* tiles = nullptr;
   int* sidx = nullptr;
-  int* didx = nullptr;
   int* fed = nullptr;
   int* pending = nullptr;
   uint32_t* status = nullptr;
@@ -415,8 +413,7 @@ int forward_layers(vla_handle* h, int M, const RowInfo* rows_dev, bool decode, i
     float* resid = h->h;  // their residual stream
     if (pruned) {
       ev = prof_begin(h, VLA_KCLASS_OTHER);
-      if ((rc = gather_rows_launch(h->q, last->idx, last->n, d, h->q_last, h->stream)) ||
-          (rc = gather_rows_launch(h->h, last->idx, last->n, d, h->h_last, h->stream)))
+      if ((rc = gather_rows2_launch(h->q, h->h, last->idx, last->n, d, h->q_last, h->h_last, h->stream)))
         return fail(h, rc, t_err);
       prof_end(h, ev, VLA_KCLASS_OTHER, 0, 16.0 * last->n * d);
       ev = prof_begin(h, VLA_KCLASS_ATTN_DECODE);
@@ -621,7 +618,6 @@ int vla_create(const vla_config* cfg, const vla_weights* w, void* cuda_stream, v
             alloc(reinterpret_cast<void**>(&h->u), 2 * T * F * sizeof(bf16)) &&
             alloc(reinterpret_cast<void**>(&h->ws), ws) &&
             alloc(reinterpret_cast<void**>(&h->h_last), static_cast<size_t>(B) * d * sizeof(float)) &&
-            alloc(reinterpret_cast<void**>(&h->head_in), static_cast<size_t>(B) * A * d * sizeof(float)) &&
             alloc(reinterpret_cast<void**>(&h->head_entropy), static_cast<size_t>(B) * A * sizeof(float)) &&
             alloc(reinterpret_cast<void**>(&h->q_last), static_cast<size_t>(B) * d * sizeof(float)) &&
             alloc(reinterpret_cast<void**>(&h->ss_part), static_cast<size_t>(d / 128 + 1) * T * sizeof(float)) &&
@@ -629,8 +625,7 @@ int vla_create(const vla_config* cfg, const vla_weights* w, void* cuda_stream, v
             alloc(reinterpret_cast<void**>(&h->rope), static_cast<size_t>(cap) * (c.head_dim / 2) * sizeof(float2)) &&
             alloc(reinterpret_cast<void**>(&h->rows), T * sizeof(RowInfo)) &&
             alloc(reinterpret_cast<void**>(&h->tiles), static_cast<size_t>(h->max_tiles) * sizeof(AttnTile)) &&
-            alloc(reinterpret_cast<void**>(&h->sidx), std::max(T, static_cast<size_t>(B) * A) * sizeof(int)) &&
-            alloc(reinterpret_cast<void**>(&h->didx), std::max(T, static_cast<size_t>(B) * A) * sizeof(int)) &&
+            alloc(reinterpret_cast<void**>(&h->sidx), static_cast<size_t>(B) * sizeof(int)) &&
             alloc(reinterpret_cast<void**>(&h->fed), static_cast<size_t>(B) * A * sizeof(int)) &&
             alloc(reinterpret_cast<void**>(&h->pending), static_cast<size_t>(B) * sizeof(int)) &&
             alloc(reinterpret_cast<void**>(&h->status), sizeof(uint32_t)) &&
@@ -668,8 +663,7 @@ int vla_create(const vla_config* cfg, const vla_weights* w, void* cuda_stream, v
   }
   // pinned staging
   h->stage_bytes = T * sizeof(RowInfo) + static_cast<size_t>(h->max_tiles) * sizeof(AttnTile) +
-                   2 * std::max(T, static_cast<size_t>(B) * A) * sizeof(int) + static_cast<size_t>(B) * sizeof(RowInfo) +
-                   1024;
+                   static_cast<size_t>(B) * (sizeof(int) + sizeof(RowInfo)) + 1024;
   for (int s = 0; s < vla_handle::kSlots; ++s) {
     if (cudaMallocHost(&h->stage_host[s], h->stage_bytes) != cudaSuccess ||
         cudaEventCreateWithFlags(&h->stage_ev[s], cudaEventDisableTiming) != cudaSuccess) {
@@ -833,6 +827,7 @@ int vla_decode_actions(vla_handle* h, const float* uniforms, float temperature, 
   ha.act_out = actions_out;
   ha.logits_out = logits_out;
   ha.fed_out = h->fed;
+  ha.pending_out = h->pending;  // the last token stays pending
   ha.status = h->status;
 
   for (int i = 0; i < A; ++i) {
@@ -851,10 +846,6 @@ int vla_decode_actions(vla_handle* h, const float* uniforms, float temperature, 
     prof_end(h, ev, VLA_KCLASS_HEAD, 2.0 * B * 256 * d, 2.0 * 256 * d + 4.0 * B * d);
     if (rc) return fail(h, rc, t_err);
   }
-  // the last token stays pending
-  if (cudaMemcpy2DAsync(h->pending, sizeof(int), h->fed + (A - 1), A * sizeof(int), sizeof(int), B,
-                        cudaMemcpyDeviceToDevice, h->stream) != cudaSuccess)
-    return fail(h, cuda_fail(cudaGetLastError(), "pending copy"), t_err);
   for (int b = 0; b < B; ++b) {
     h->len[b] = h->len_prefill[b] + (A - 1);
     h->has_pending[b] = 1;
@@ -881,21 +872,13 @@ int vla_score_actions(vla_handle* h, const int32_t* tokens, float temperature, f
   uint8_t* st = static_cast<uint8_t*>(stage_slot(h, &slot));
   RowInfo* rows = reinterpret_cast<RowInfo*>(st);
   AttnTile* tiles = reinterpret_cast<AttnTile*>(rows + M);
-  int* sidx = reinterpret_cast<int*>(tiles + B);
-  int* didx = sidx + M;
   int n_tiles = 0;
   for (int b = 0; b < B; ++b) {
-    for (int j = 0; j < n; ++j) {
-      rows[b * n + j] = RowInfo{b, h->len_prefill[b] + j, ROW_TOKEN, b * A + j};
-      sidx[b * n + j] = b * n + j;
-      didx[b * n + j] = b * A + 1 + j;
-    }
+    for (int j = 0; j < n; ++j) rows[b * n + j] = RowInfo{b, h->len_prefill[b] + j, ROW_TOKEN, b * A + j};
     if (n > 0) tiles[n_tiles++] = AttnTile{b, b * n, n, h->len_prefill[b]};
   }
   if ((rc = upload(h, h->rows, rows, M * sizeof(RowInfo))) ||
-      (rc = upload(h, h->tiles, tiles, n_tiles * sizeof(AttnTile))) ||
-      (rc = upload(h, h->sidx, sidx, M * sizeof(int))) ||
-      (rc = upload(h, h->didx, didx, M * sizeof(int))))
+      (rc = upload(h, h->tiles, tiles, n_tiles * sizeof(AttnTile))))
     return fail(h, rc, t_err);
   cudaEventRecord(h->stage_ev[slot], h->stream);
 
@@ -906,16 +889,11 @@ int vla_score_actions(vla_handle* h, const int32_t* tokens, float temperature, f
     if (rc) return fail(h, rc, t_err);
     if ((rc = forward_layers(h, M, h->rows, false, n_tiles, n, 0))) return rc;
   }
-  // head inputs: row b*A = prefill's last hidden, rows b*A+1+j = chunk rows
-  if (cudaMemcpy2DAsync(h->head_in, static_cast<size_t>(A) * d * sizeof(float), h->h_last, d * sizeof(float),
-                        d * sizeof(float), B, cudaMemcpyDeviceToDevice, h->stream) != cudaSuccess)
-    return fail(h, cuda_fail(cudaGetLastError(), "head input copy"), t_err);
-  if (M > 0 && (rc = scatter_rows_launch(h->h, h->sidx, h->didx, M, d, h->head_in, h->stream)))
-    return fail(h, rc, t_err);
-
   HeadArgs ha;
   ha.entropy_out = h->head_entropy;
-  ha.h = h->head_in;
+  ha.h = h->h;            // the chunk's rows, after each env's
+  ha.h_first = h->h_last;  // final row of the prefill
+  ha.pending_out = h->pending;
   ha.ldh = d;
   ha.B = B;
   ha.n_pos = A;
@@ -937,9 +915,6 @@ int vla_score_actions(vla_handle* h, const int32_t* tokens, float temperature, f
   rc = action_head_launch(ha, h->stream);
   prof_end(h, ev, VLA_KCLASS_HEAD, 2.0 * B * A * 256 * d, 2.0 * 256 * d + 4.0 * B * A * d);
   if (rc) return fail(h, rc, t_err);
-  if (cudaMemcpy2DAsync(h->pending, sizeof(int), tokens + (A - 1), A * sizeof(int), sizeof(int), B,
-                        cudaMemcpyDeviceToDevice, h->stream) != cudaSuccess)
-    return fail(h, cuda_fail(cudaGetLastError(), "pending copy"), t_err);
   for (int b = 0; b < B; ++b) {
     h->len[b] = h->len_prefill[b] + (A - 1);
     h->has_pending[b] = 1;
@@ -1052,8 +1027,8 @@ void vla_destroy(vla_handle* h) {
   if (!h) return;
   DeviceGuard dev_guard(h->dev);  // best effort: the handle is freed whatever happens
   cudaStreamSynchronize(h->stream);
-  void* bufs[] = {h->kv, h->kv_res, h->h, h->y, h->q, h->ao, h->u, h->ws, h->h_last, h->head_in, h->head_entropy, h->q_last, h->ss_part, h->last_rows, h->rope,
-                  h->rows, h->tiles, h->sidx, h->didx, h->fed, h->pending, h->status, h->part_o,
+  void* bufs[] = {h->kv, h->kv_res, h->h, h->y, h->q, h->ao, h->u, h->ws, h->h_last, h->head_entropy, h->q_last, h->ss_part, h->last_rows, h->rope,
+                  h->rows, h->tiles, h->sidx, h->fed, h->pending, h->status, h->part_o,
                   h->part_ml, h->attn_tickets, h->w16, h->w16_range};
   for (void* p : bufs)
     if (p) cudaFree(p);

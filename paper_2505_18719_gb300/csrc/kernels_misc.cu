@@ -106,22 +106,12 @@ __global__ void __launch_bounds__(256) rmsnorm_kernel(const float* h, int ldh,
   report_saturation(status, sat);
 }
 
-__global__ void gather_rows_kernel(const float* src, const int* __restrict__ idx,
-                                   int d, float* __restrict__ dst) {
+__global__ void gather_rows2_kernel(const float* src0, const float* src1, const int* __restrict__ idx, int d,
+                                    float* __restrict__ dst0, float* __restrict__ dst1) {
   pdl_launch_dependents();
   pdl_wait();
-  const float* s = src + static_cast<size_t>(idx[blockIdx.x]) * d;
-  float* o = dst + static_cast<size_t>(blockIdx.x) * d;
-  for (int c = threadIdx.x * 4; c < d; c += blockDim.x * 4)
-    *reinterpret_cast<float4*>(o + c) = *reinterpret_cast<const float4*>(s + c);
-}
-
-__global__ void scatter_rows_kernel(const float* src, const int* __restrict__ sidx,
-                                    const int* __restrict__ didx, int d, float* __restrict__ dst) {
-  pdl_launch_dependents();
-  pdl_wait();
-  const float* s = src + static_cast<size_t>(sidx[blockIdx.x]) * d;
-  float* o = dst + static_cast<size_t>(didx[blockIdx.x]) * d;
+  const float* s = (blockIdx.y ? src1 : src0) + static_cast<size_t>(idx[blockIdx.x]) * d;
+  float* o = (blockIdx.y ? dst1 : dst0) + static_cast<size_t>(blockIdx.x) * d;
   for (int c = threadIdx.x * 4; c < d; c += blockDim.x * 4)
     *reinterpret_cast<float4*>(o + c) = *reinterpret_cast<const float4*>(s + c);
 }
@@ -159,25 +149,15 @@ int norm_scale_launch(const float* h, int ldh, const bf16* w, const float* ss, i
   return VLA_OK;
 }
 
-int gather_rows_launch(const float* src, const int* idx, int n, int d, float* dst, cudaStream_t s) {
-  if (n <= 0) return VLA_OK;
-  VLA_CUDA_TRY(launch_pdl(gather_rows_kernel, dim3(n), dim3(256), 0, s, src, idx, d, dst));
-  note_launch();
-  VLA_CUDA_TRY(cudaGetLastError());
-  return VLA_OK;
-}
-
-}  // namespace vla
-
-namespace vla {
-int scatter_rows_launch(const float* src, const int* sidx, const int* didx, int n, int d, float* dst,
+int gather_rows2_launch(const float* src0, const float* src1, const int* idx, int n, int d, float* dst0, float* dst1,
                         cudaStream_t s) {
   if (n <= 0) return VLA_OK;
-  VLA_CUDA_TRY(launch_pdl(scatter_rows_kernel, dim3(n), dim3(256), 0, s, src, sidx, didx, d, dst));
+  VLA_CUDA_TRY(launch_pdl(gather_rows2_kernel, dim3(n, 2), dim3(256), 0, s, src0, src1, idx, d, dst0, dst1));
   note_launch();
   VLA_CUDA_TRY(cudaGetLastError());
   return VLA_OK;
 }
+
 }  // namespace vla
 
 namespace vla {

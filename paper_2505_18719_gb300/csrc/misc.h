@@ -68,14 +68,14 @@ int rmsnorm_launch(const float* h, int ldh, const bf16* w, int M, int d, float e
 int bf16_to_f16_launch(const bf16* src, f16* dst, size_t n, int* out_of_range, int num_sms,
                        cudaStream_t s);
 
-// dst[i] = src[idx[i]] rows of width d (f32).
-int gather_rows_launch(const float* src, const int* idx, int n, int d, float* dst, cudaStream_t s);
-// dst[didx[i]] = src[sidx[i]] rows of width d (f32), i < n.
-int scatter_rows_launch(const float* src, const int* sidx, const int* didx, int n, int d, float* dst,
+// dst0[i] = src0[idx[i]] and dst1[i] = src1[idx[i]], rows of width d (f32).
+int gather_rows2_launch(const float* src0, const float* src1, const int* idx, int n, int d, float* dst0, float* dst1,
                         cudaStream_t s);
 
 struct HeadArgs {
   const float* h = nullptr;   // input rows, row (b * n_pos + j) has stride ldh
+  // set (score): row j = 0 of env b is h_first's row b, row j > 0 is h's row b * (n_pos - 1) + j - 1
+  const float* h_first = nullptr;
   int ldh = 0;
   int B = 0, n_pos = 1;       // grid: B x n_pos
   int step = 0;               // action index of j = 0 (decode: current step; score: 0)
@@ -96,6 +96,7 @@ struct HeadArgs {
   float* logits_out = nullptr;      // [B, A, 256]
   int* fed_out = nullptr;           // [B, A] token fed to the next step (forced or sampled)
   float* entropy_out = nullptr;     // [B, A] entropy of each token's bin distribution
+  int* pending_out = nullptr;       // [B] each env's token of action A - 1
   uint32_t* status = nullptr;
   // decode steps with a next one (n_pos == 1): the row of the token fed next, per env, as assemble_launch
   // would write it (next_embed null: none)
