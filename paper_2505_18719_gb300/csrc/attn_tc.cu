@@ -190,7 +190,6 @@ __global__ void __launch_bounds__(kAtThreads, 1)
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 38);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
 
-  pdl_launch_dependents();
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int n_my = (p.n_items - static_cast<int>(blockIdx.x) + static_cast<int>(gridDim.x) - 1) /
                    static_cast<int>(gridDim.x);
@@ -230,6 +229,10 @@ __global__ void __launch_bounds__(kAtThreads, 1)
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
+  // With this CTA's TMEM held: 64-wide heads leave 114 KB of the SM's shared memory, room for a CTA of the
+  // cluster GEMM that may follow (prefills of 17 to 32 rows).  Were its TMEM allocated first, this CTA would wait
+  // for it, and it for this kernel.
+  pdl_launch_dependents();
   const uint32_t tmem = *tmem_slot;
 
   auto kslot = [&](int st) { return smem + st * Sm::SLOT; };

@@ -200,6 +200,9 @@ __device__ __forceinline__ float silu_f(float x) { return x / (1.0f + expf(-x));
 // ld.global.cg), never through the non-coherent read-only path (__ldg, const __restrict__):
 // a kernel scheduled early can see stale read-only-cache lines there.  Without the launch
 // attribute both instructions are no-ops.
+// A kernel that allocates tensor memory lets its successor start only once it holds it (after the
+// barrier that follows tcgen05.alloc): a successor's CTA on the same SM could otherwise take the columns
+// first and wait for this kernel, while this kernel's allocation waits for that CTA.
 __device__ __forceinline__ void pdl_launch_dependents() {
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 }

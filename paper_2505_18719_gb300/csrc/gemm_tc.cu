@@ -357,7 +357,6 @@ __global__ void __launch_bounds__(kThreads, 1)
   const uint32_t IDESC = idesc_for(make_idesc<BN>(), p.epi.fp16);
   constexpr bool SWIGLU = (EPI == EPI_SWIGLU);
 
-  pdl_launch_dependents();
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) &
                                              ~static_cast<uintptr_t>(1023));
@@ -401,6 +400,7 @@ __global__ void __launch_bounds__(kThreads, 1)
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
+  pdl_launch_dependents();  // with this CTA's TMEM held
   const uint32_t tmem_base = *tmem_slot;
   const int units = p.tiles_m * p.tiles_n * p.splits;
   uint32_t* status = p.epi.status;
@@ -576,7 +576,6 @@ __global__ void __launch_bounds__(kThreads, 1)
                                    p.epi.fp16);
   constexpr bool SWIGLU = (EPI == EPI_SWIGLU);
 
-  pdl_launch_dependents();
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) &
                                              ~static_cast<uintptr_t>(1023));
@@ -621,6 +620,7 @@ __global__ void __launch_bounds__(kThreads, 1)
   tc_fence_before();
   cluster_sync();  // both CTAs' barriers are initialised before either touches the other's
   tc_fence_after();
+  pdl_launch_dependents();  // with this CTA's TMEM held
   const uint32_t tmem_base = *tmem_slot;
   const int units = p.tiles_m * p.tiles_n;
   const int n_pairs = gridDim.x >> 1;
@@ -1158,7 +1158,6 @@ __global__ void __launch_bounds__(kThreads, 1)
                                    p.fp16);
   static_assert(TMEM_COLS >= 32 && (TMEM_COLS & (TMEM_COLS - 1)) == 0, "TMEM allocation");
 
-  pdl_launch_dependents();
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) &
                                              ~static_cast<uintptr_t>(1023));
@@ -1197,6 +1196,7 @@ __global__ void __launch_bounds__(kThreads, 1)
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
+  pdl_launch_dependents();  // with this CTA's TMEM held
   const uint32_t tmem_base = *tmem_slot;
   const int total = p.tiles * p.kbt;
   const int g_begin = blockIdx.x * p.per_cta;
@@ -1596,7 +1596,7 @@ __global__ void __launch_bounds__(kThreads, 2)
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
-  pdl_launch_dependents();  // this CTA holds its TMEM: the next kernel's CTAs cannot take it first
+  pdl_launch_dependents();  // with this CTA's TMEM held
   const uint32_t tmem_base = *tmem_slot;
   uint32_t* status = p.epi.status;
   const uint64_t limit = p.wait_limit;
@@ -1823,7 +1823,7 @@ __global__ void __launch_bounds__(kWideThreads, 1)
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
-  pdl_launch_dependents();
+  pdl_launch_dependents();  // with this CTA's TMEM held
   const uint32_t tmem_base = *tmem_slot;
   uint32_t* status = p.epi.status;
   const uint64_t limit = p.wait_limit;
