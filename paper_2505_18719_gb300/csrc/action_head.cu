@@ -110,7 +110,8 @@ __global__ void __launch_bounds__(kHeadThreads, RPC) head_kernel(const HeadArgs 
       w[nt] = (step < steps && k < d) ? *reinterpret_cast<const uint4*>(wrow + static_cast<size_t>(nt * 8) * d + k)
                                       : make_uint4(0u, 0u, 0u, 0u);
   };
-  // the bin rows are the caller's weights: requested before the previous kernel is waited for
+  // the bin rows are the caller's weights: requested before the previous kernel is waited for (as a call's
+  // first kernel the head is launched in stream order)
 #pragma unroll
   for (int i = 0; i < DEPTH; ++i) load_w(i, wq[i]);
 
@@ -308,8 +309,8 @@ int action_head_launch(const HeadArgs& a, cudaStream_t s) {
   const int R = a.B * a.n_pos;
   auto go = [&](auto kern, int rows, std::atomic<uint64_t>& attr_done) -> cudaError_t {
     if (const cudaError_t e = set_smem_limit(kern, static_cast<int>(head_smem(kHeadMaxD, rows)), attr_done)) return e;
-    return launch_pdl_cluster(kern, dim3((R + rows - 1) / rows * kHeadCluster), dim3(kHeadThreads), head_smem(a.d, rows),
-                              s, kHeadCluster, a);
+    return launch_cluster_at(a.start, kern, dim3((R + rows - 1) / rows * kHeadCluster), dim3(kHeadThreads),
+                             head_smem(a.d, rows), s, kHeadCluster, a);
   };
   static std::atomic<uint64_t> done[4];
   if (R <= kHeadSmallRows) {

@@ -200,6 +200,10 @@ __device__ __forceinline__ float silu_f(float x) { return x / (1.0f + expf(-x));
 // ld.global.cg), never through the non-coherent read-only path (__ldg, const __restrict__):
 // a kernel scheduled early can see stale read-only-cache lines there.  Without the launch
 // attribute both instructions are no-ops.
+// Weights, which no kernel of the path writes, may be read before the wait: the first kernel of every
+// call that has such a reader is launched in stream order (Start::kInOrder), so whatever the caller
+// queued before the call, an update of those weights among it, has completed before any kernel of the
+// call starts.  (A call's uploads order the stream as well, where it has any.)
 // A kernel that allocates tensor memory lets its successor start only once it holds it (after the
 // barrier that follows tcgen05.alloc): a successor's CTA on the same SM could otherwise take the columns
 // first and wait for this kernel, while this kernel's allocation waits for that CTA.
@@ -224,10 +228,13 @@ inline cudaError_t injected_launch_error() {
 extern std::atomic<uint64_t> g_wait_limit_ns;
 constexpr uint64_t kDefaultWaitLimitNs = 1000000000ull;
 
+// kEarly: programmatic dependent launch.  kInOrder: starts when everything before it on the stream is done.
+enum class Start { kEarly, kInOrder };
+
 // `cluster` > 1: thread-block clusters of that many consecutive CTAs along x.
 template <typename... KArgs, typename... Args>
-inline cudaError_t launch_pdl_cluster(void (*kern)(KArgs...), dim3 grid, dim3 block, size_t smem,
-                                      cudaStream_t stream, int cluster, Args... args) {
+inline cudaError_t launch_cluster_at(Start start, void (*kern)(KArgs...), dim3 grid, dim3 block, size_t smem,
+                                     cudaStream_t stream, int cluster, Args... args) {
   if (const cudaError_t inj = injected_launch_error()) return inj;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = grid;
@@ -235,20 +242,35 @@ inline cudaError_t launch_pdl_cluster(void (*kern)(KArgs...), dim3 grid, dim3 bl
   cfg.dynamicSmemBytes = smem;
   cfg.stream = stream;
   cudaLaunchAttribute attr[2];
-  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr[0].val.programmaticStreamSerializationAllowed = 1;
-  attr[1].id = cudaLaunchAttributeClusterDimension;
-  attr[1].val.clusterDim.x = static_cast<unsigned>(cluster);
-  attr[1].val.clusterDim.y = 1;
-  attr[1].val.clusterDim.z = 1;
+  unsigned n = 0;
+  if (start == Start::kEarly) {
+    attr[n].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[n++].val.programmaticStreamSerializationAllowed = 1;
+  }
+  if (cluster > 1) {
+    attr[n].id = cudaLaunchAttributeClusterDimension;
+    attr[n].val.clusterDim.x = static_cast<unsigned>(cluster);
+    attr[n].val.clusterDim.y = 1;
+    attr[n++].val.clusterDim.z = 1;
+  }
   cfg.attrs = attr;
-  cfg.numAttrs = cluster > 1 ? 2 : 1;
+  cfg.numAttrs = n;
   return cudaLaunchKernelEx(&cfg, kern, static_cast<KArgs>(args)...);
+}
+template <typename... KArgs, typename... Args>
+inline cudaError_t launch_pdl_cluster(void (*kern)(KArgs...), dim3 grid, dim3 block, size_t smem,
+                                      cudaStream_t stream, int cluster, Args... args) {
+  return launch_cluster_at(Start::kEarly, kern, grid, block, smem, stream, cluster, args...);
 }
 template <typename... KArgs, typename... Args>
 inline cudaError_t launch_pdl(void (*kern)(KArgs...), dim3 grid, dim3 block, size_t smem,
                               cudaStream_t stream, Args... args) {
   return launch_pdl_cluster(kern, grid, block, smem, stream, 1, args...);
+}
+template <typename... KArgs, typename... Args>
+inline cudaError_t launch_at(Start start, void (*kern)(KArgs...), dim3 grid, dim3 block, size_t smem,
+                             cudaStream_t stream, Args... args) {
+  return launch_cluster_at(start, kern, grid, block, smem, stream, 1, args...);
 }
 
 // Raises a kernel's dynamic shared-memory limit on the current device.  Function attributes

@@ -838,6 +838,7 @@ int vla_decode_actions(vla_handle* h, const float* uniforms, float temperature, 
     }
     ha.h = (i == 0) ? h->h_last : h->h;
     ha.step = i;
+    ha.start = i == 0 ? Start::kInOrder : Start::kEarly;
     ha.next_embed = i + 1 < A ? h->embed : nullptr;
     ha.next_h = h->h;
     ha.next_norm = first_norm(h);
@@ -893,6 +894,7 @@ int vla_score_actions(vla_handle* h, const int32_t* tokens, float temperature, f
   ha.entropy_out = h->head_entropy;
   ha.h = h->h;            // the chunk's rows, after each env's
   ha.h_first = h->h_last;  // final row of the prefill
+  ha.start = M == 0 ? Start::kInOrder : Start::kEarly;
   ha.pending_out = h->pending;
   ha.ldh = d;
   ha.B = B;
@@ -1151,6 +1153,7 @@ int op_gemm_decode(const std::string& name, bool fp16, const void* A, const void
   g.M = M;
   g.N = N;
   g.K = K;
+  g.start = Start::kInOrder;
   g.workspace = workspace;
   g.workspace_bytes = workspace_bytes;
   g.epi.kind = EPI_F32;
@@ -1215,6 +1218,7 @@ int vla_op_action_head(const float* hs, int ldh, int B, int d, const void* final
       !finite_nonneg(temperature) || (temperature > 0.f && !uniforms))
     return set_err(nullptr, VLA_ERR_ARG, "vla_op_action_head: bad argument");
   HeadArgs ha;
+  ha.start = Start::kInOrder;
   ha.h = hs;
   ha.ldh = ldh;
   ha.B = B;

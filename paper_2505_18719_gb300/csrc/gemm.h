@@ -66,6 +66,9 @@ struct GemmArgs {
   int block_n = 256;        // 128 or 256
   int splits = 1;           // split-K factor (> 1 needs workspace)
   bool pair = false;        // 2-SM tiles (256 x 256 per CTA pair); needs block_n 256, splits 1
+  // kInOrder where the call is the first kernel after the caller's own work (the weight-streaming GEMMs
+  // read B before they wait)
+  Start start = Start::kEarly;
   float* workspace = nullptr;
   size_t workspace_bytes = 0;
   EpiArgs epi;

@@ -2166,14 +2166,14 @@ StreamPlan stream_plan(int M, int N, int K, int num_sms) {
 
 template <int BNX>
 int launch_stream(const CUtensorMap& w, const CUtensorMap& x, const CUtensorMap& x2,
-                const StreamParams& p, int grid, cudaStream_t stream) {
+                const StreamParams& p, int grid, Start start, cudaStream_t stream) {
   constexpr int STAGE = 256 * BK * 2 + 2 * BNX * BK * 2;
   constexpr int STAGES = (196608 / STAGE) < 8 ? (196608 / STAGE) : 8;
   constexpr int smem = STAGES * STAGE + 1024 + 256;
   static std::atomic<uint64_t> attr_done{0};
   auto kern = gemv_stream_kernel<BNX, STAGES>;
   VLA_CUDA_TRY(set_smem_limit(kern, smem, attr_done));
-  VLA_CUDA_TRY(launch_pdl(kern, dim3(grid), dim3(kThreads), smem, stream, w, x, x2, p));
+  VLA_CUDA_TRY(launch_at(start, kern, dim3(grid), dim3(kThreads), smem, stream, w, x, x2, p));
   note_launch();
   VLA_CUDA_TRY(cudaGetLastError());
   return VLA_OK;
@@ -2222,7 +2222,7 @@ ClusterPlan cluster_plan(int M, int N, int K, bool swiglu, int num_sms) {
 
 template <int BNX, int TR>
 int launch_cluster(const CUtensorMap& w, const CUtensorMap& w2, const CUtensorMap& x, const CUtensorMap& x2,
-                const ClusterParams& p, const ClusterPlan& pl, cudaStream_t stream) {
+                   const ClusterParams& p, const ClusterPlan& pl, Start start, cudaStream_t stream) {
   constexpr int STAGE = TR * BK * 2 + 2 * BNX * BK * 2;
   constexpr int STAGES = kClusterData / STAGE;
   // the exchange: the partial tile and the other ranks' rows, (C - 1) * ceil(M / C) < M + C
@@ -2231,7 +2231,7 @@ int launch_cluster(const CUtensorMap& w, const CUtensorMap& w2, const CUtensorMa
   static std::atomic<uint64_t> attr_done{0};
   auto kern = gemv_cluster_kernel<BNX, TR, STAGES>;
   VLA_CUDA_TRY(set_smem_limit(kern, smem, attr_done));
-  VLA_CUDA_TRY(launch_pdl_cluster(kern, dim3(pl.tiles * pl.c), dim3(kThreads), smem, stream, pl.c, w, w2, x, x2, p));
+  VLA_CUDA_TRY(launch_cluster_at(start, kern, dim3(pl.tiles * pl.c), dim3(kThreads), smem, stream, pl.c, w, w2, x, x2, p));
   note_launch();
   VLA_CUDA_TRY(cudaGetLastError());
   return VLA_OK;
@@ -2239,9 +2239,9 @@ int launch_cluster(const CUtensorMap& w, const CUtensorMap& w2, const CUtensorMa
 
 template <int TR>
 int dispatch_cluster(const CUtensorMap& w, const CUtensorMap& w2, const CUtensorMap& x, const CUtensorMap& x2,
-                  const ClusterParams& p, const ClusterPlan& pl, cudaStream_t stream) {
-  return pl.bnx == 16 ? launch_cluster<16, TR>(w, w2, x, x2, p, pl, stream)
-                      : launch_cluster<32, TR>(w, w2, x, x2, p, pl, stream);
+                     const ClusterParams& p, const ClusterPlan& pl, Start start, cudaStream_t stream) {
+  return pl.bnx == 16 ? launch_cluster<16, TR>(w, w2, x, x2, p, pl, start, stream)
+                      : launch_cluster<32, TR>(w, w2, x, x2, p, pl, start, stream);
 }
 
 int cluster_launch_as(const GemmArgs& a, const ClusterPlan& pl, cudaStream_t stream) {
@@ -2260,8 +2260,8 @@ int cluster_launch_as(const GemmArgs& a, const ClusterPlan& pl, cudaStream_t str
   p.kbt = pl.kbt;
   p.epi = a.epi;
   p.wait_limit = g_wait_limit_ns.load(std::memory_order_relaxed);
-  return pl.tr == 256 ? dispatch_cluster<256>(mw, mw2, mx, mx2, p, pl, stream)
-                      : dispatch_cluster<128>(mw, mw2, mx, mx2, p, pl, stream);
+  return pl.tr == 256 ? dispatch_cluster<256>(mw, mw2, mx, mx2, p, pl, a.start, stream)
+                      : dispatch_cluster<128>(mw, mw2, mx, mx2, p, pl, a.start, stream);
 }
 
 }  // namespace
@@ -2487,8 +2487,8 @@ int gemv_launch(const GemmArgs& a, cudaStream_t stream, int num_sms, GemmCost* c
   p.wait_limit = g_wait_limit_ns.load(std::memory_order_relaxed);
   int rc;
   switch (pl.bnx) {
-    case 64: rc = launch_stream<64>(mw, mx, mx2, p, pl.grid, stream); break;
-    default: rc = launch_stream<128>(mw, mx, mx2, p, pl.grid, stream); break;
+    case 64: rc = launch_stream<64>(mw, mx, mx2, p, pl.grid, a.start, stream); break;
+    default: rc = launch_stream<128>(mw, mx, mx2, p, pl.grid, a.start, stream); break;
   }
   if (rc != VLA_OK) return rc;
   const StreamSrc src{a.workspace, pl.bnx, pl.kbt, pl.per_cta, pl.max_seg};

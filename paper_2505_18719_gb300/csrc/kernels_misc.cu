@@ -50,7 +50,7 @@ __global__ void __launch_bounds__(256) norm_scale_kernel(const float* h, int ldh
                                                          uint32_t* status) {
   pdl_launch_dependents();
   const int m = blockIdx.y, c = (blockIdx.x * 256 + threadIdx.x) * 4, lane = threadIdx.x & 31;
-  uint2 ww = make_uint2(0u, 0u);
+  uint2 ww = make_uint2(0u, 0u);  // a weight, and never the call's first kernel: read before the wait
   if (c < d) ww = *reinterpret_cast<const uint2*>(w + c);
   pdl_wait();
   float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
@@ -122,8 +122,8 @@ int assemble_launch(const RowInfo* rows, int n_rows, const bf16* visual, const i
                     const int* tokens, const bf16* embed, int d, int vocab, float* h, const FirstNorm& norm,
                     uint32_t* status, cudaStream_t s) {
   if (n_rows <= 0) return VLA_OK;
-  VLA_CUDA_TRY(launch_pdl(assemble_kernel, dim3(n_rows), dim3(256), 0, s, rows, visual, ids, tokens,
-                          embed, d, vocab, h, norm, status));
+  VLA_CUDA_TRY(launch_at(Start::kInOrder, assemble_kernel, dim3(n_rows), dim3(256), 0, s, rows, visual, ids, tokens,
+                         embed, d, vocab, h, norm, status));
   note_launch();
   VLA_CUDA_TRY(cudaGetLastError());
   return VLA_OK;

@@ -46,7 +46,8 @@ __device__ __forceinline__ void token_row_256(const bf16* src, int d, float* h, 
 
 // h[r] (f32 [rows, d]) = source row of RowInfo r: visual (bf16 row idx), text (embed[ids[idx]])
 // or token (embed[tokens[idx]]).  Ids outside [0, vocab) -> VLA_STATUS_BAD_TOKEN, row 0.
-// The rows' RMSNorm with weight norm.w goes to norm.y_hi / y_lo [rows, d] as the operand pair.
+// The rows' RMSNorm with weight norm.w goes to norm.y_hi / y_lo [rows, d] as the operand pair.  The first kernel
+// of a call: launched in stream order.
 int assemble_launch(const RowInfo* rows, int n_rows, const bf16* visual, const int* ids,
                     const int* tokens, const bf16* embed, int d, int vocab, float* h, const FirstNorm& norm,
                     uint32_t* status, cudaStream_t s);
@@ -73,6 +74,7 @@ int gather_rows2_launch(const float* src0, const float* src1, const int* idx, in
                         cudaStream_t s);
 
 struct HeadArgs {
+  Start start = Start::kEarly;  // kInOrder for the first kernel of a call
   const float* h = nullptr;   // input rows, row (b * n_pos + j) has stride ldh
   // set (score): row j = 0 of env b is h_first's row b, row j > 0 is h's row b * (n_pos - 1) + j - 1
   const float* h_first = nullptr;

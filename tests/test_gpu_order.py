@@ -1,0 +1,154 @@
+"""Weights that a call reads before it waits for the kernel ahead of it are complete when it starts.
+
+The caller's weights are read in place at every call.  A kernel launched with programmatic stream
+serialization may start while the kernel before it is still running, so the first kernel of a call that
+reads weights ahead of its wait has to be launched in stream order.  Captured into a graph, the two kinds
+of launch give edges of different types, which shows the order without running anything.
+"""
+import ctypes
+import dataclasses
+
+import pytest
+import torch
+
+from paper_2505_18719_gb300 import inputs as I
+from paper_2505_18719_gb300 import vla as V
+from tests import parity as P
+
+pytestmark = pytest.mark.gpu
+WL = I.WORKLOADS["tiny_b4"]
+RELAXED = 2
+FULL, PROGRAMMATIC = 0, 1
+
+
+class EdgeData(ctypes.Structure):
+    _fields_ = [("from_port", ctypes.c_ubyte), ("to_port", ctypes.c_ubyte), ("type", ctypes.c_ubyte),
+                ("reserved", ctypes.c_ubyte * 5)]
+
+
+def _edge_types(stream, calls):
+    """The edge types of a captured chain of calls, in the order of the chain."""
+    assert all(c() in (0, None) for c in calls)  # every kernel is loaded before the capture
+    stream.synchronize()
+    cu = ctypes.CDLL("libcuda.so.1")
+    graph = ctypes.c_void_p()
+    st = ctypes.c_void_p(stream.cuda_stream)
+    assert cu.cuStreamBeginCapture_v2(st, RELAXED) == 0
+    rcs = [c() for c in calls]
+    assert cu.cuStreamEndCapture(st, ctypes.byref(graph)) == 0
+    assert all(rc in (0, None) for rc in rcs), rcs
+    n = ctypes.c_size_t(0)
+    assert cu.cuGraphGetEdges_v2(graph, None, None, None, ctypes.byref(n)) == 0
+    src, dst, data = (ctypes.c_void_p * n.value)(), (ctypes.c_void_p * n.value)(), (EdgeData * n.value)()
+    assert cu.cuGraphGetEdges_v2(graph, src, dst, data, ctypes.byref(n)) == 0
+    nxt = {src[i]: (dst[i], data[i].type) for i in range(n.value)}
+    at = (set(nxt) - {d for d, _ in nxt.values()}).pop()
+    types = []
+    while at in nxt:
+        at, t = nxt[at]
+        types.append(t)
+    assert cu.cuGraphDestroy(graph) == 0
+    return types
+
+
+@pytest.fixture(scope="module")
+def bufs():
+    from paper_2505_18719_gb300 import build
+    build.build()
+    V.load()
+    f = lambda *s: torch.zeros(*s, device="cuda")  # noqa: E731
+    b = lambda *s: torch.zeros(*s, dtype=torch.bfloat16, device="cuda")  # noqa: E731
+    return {"x": f(64, 256), "z": f(64, 256), "v": f(64), "act": f(64), "w": b(512, 256), "a": b(64, 256), "lo": b(64, 256),
+            "gain": b(256), "ws": f(1 << 20), "bins": torch.zeros(64, dtype=torch.int32, device="cuda"),
+            "status": torch.zeros(1, dtype=torch.int32, device="cuda")}
+
+
+def _ahead(t, stream):
+    # a kernel that lets its dependents start early
+    return lambda: V.vla_op_rmsnorm(t["x"].data_ptr(), 256, 64, 256, t["gain"].data_ptr(), 1e-6, t["a"].data_ptr(),
+                                    t["lo"].data_ptr(), False, stream.cuda_stream)
+
+
+def test_a_launch_that_waits_first_may_start_early(bufs):
+    s = torch.cuda.Stream()
+    assert _edge_types(s, [_ahead(bufs, s), _ahead(bufs, s)]) == [PROGRAMMATIC]
+
+
+def test_action_head_op_starts_in_stream_order(bufs):
+    t, s = bufs, torch.cuda.Stream()
+    head = lambda: V.vla_op_action_head(t["x"].data_ptr(), 256, 64, 256, t["gain"].data_ptr(),  # noqa: E731
+                                        t["w"].data_ptr(), 1e-6, 0, 0.0, 0, t["bins"].data_ptr(), t["v"].data_ptr(),
+                                        t["act"].data_ptr(), t["z"].data_ptr(), t["status"].data_ptr(), s.cuda_stream)
+    assert _edge_types(s, [_ahead(t, s), head]) == [FULL]
+
+
+@pytest.mark.parametrize("M", [16, 64])
+def test_decode_gemm_ops_start_in_stream_order(bufs, M):
+    t, s = bufs, torch.cuda.Stream()
+    c = torch.zeros(M, 512, device="cuda")
+    for op in (V.vla_op_gemm_decode_bf16, V.vla_op_gemm_decode_f16):
+        gemm = lambda: op(t["a"].data_ptr(), t["lo"].data_ptr(), 256, t["w"].data_ptr(), 256, c.data_ptr(), 512,  # noqa: E731
+                          M, 512, 256, t["ws"].data_ptr(), 4 << 20, s.cuda_stream)
+        assert _edge_types(s, [_ahead(t, s), gemm])[0] == FULL
+
+
+def test_one_token_decode_and_score_start_in_stream_order(bufs):
+    # a handle of one action token uploads nothing in decode and score: the head is their first kernel
+    sh = dataclasses.replace(WL.shape, action_dim=1)
+    s = torch.cuda.Stream()
+    pol = V.Policy(sh, P.weights_to_device(I.make_weights(sh, 3)), 2, 64, 64, stream=s)
+    ids = torch.zeros(2, 4, dtype=torch.int32, device="cuda")
+    u = torch.full((2, 1, 256), 0.5, device="cuda")
+    tok = torch.full((2, 1), sh.vocab - 1, dtype=torch.int32, device="cuda")
+    i32, f32 = torch.zeros(2, 1, dtype=torch.int32, device="cuda"), [torch.zeros(2, 1, device="cuda") for _ in range(2)]
+    torch.cuda.synchronize()
+    pol.prefill(None, ids, [4, 3])
+    pol.sync()
+    decode = lambda: V.vla_decode_actions(pol.h, u.data_ptr(), 1.0, 0, i32.data_ptr(), f32[0].data_ptr(),  # noqa: E731
+                                          f32[1].data_ptr(), 0)
+    score = lambda: V.vla_score_actions(pol.h, tok.data_ptr(), 1.0, f32[0].data_ptr())  # noqa: E731
+    assert _edge_types(s, [_ahead(bufs, s), decode]) == [FULL]
+    assert _edge_types(s, [_ahead(bufs, s), score]) == [FULL]
+    pol.close()
+
+
+@pytest.mark.parametrize("action_dim", [1, 7])
+def test_gains_embeddings_and_lm_head_are_read_at_every_call(action_dim):
+    # changed in place on the stream between calls, without a synchronisation: the results are those of a
+    # handle made after the change, bit for bit
+    sh = dataclasses.replace(WL.shape, action_dim=action_dim)
+    w = P.weights_to_device(I.make_weights(sh, 3))
+    ids = I.randint_i32((2, 9), 5, 6, 0, sh.vocab - 257).cuda()
+    u = I.uniform_f32((2, action_dim, 256), 5, 7).cuda()
+    tok = I.randint_i32((2, action_dim), 5, 8, sh.vocab - 256, sh.vocab - 1).cuda()
+
+    def turn(pol, between=lambda: None):
+        pol.reset()
+        pol.prefill(None, ids, [9, 6])
+        between()
+        d = pol.decode(u, 1.0, forced=tok)
+        between()
+        return [d["logits"], pol.score(tok, 1.0)["logits"]]
+
+    pol = V.Policy(sh, w, 2, 64, 64)
+    before = turn(pol)
+    torch.cuda._sleep(1_000_000)  # keeps the stream busy while the host queues the rest
+    for name in ("embed", "attn_norm", "ffn_norm", "final_norm"):
+        w[name].mul_(1.25)
+    w["lm_head"].neg_()
+    after = turn(pol)
+    w["lm_head"].neg_()
+    # the head alone changed between a prefill and its decode, and back before the score
+    mixed = turn(pol, between=lambda: w["lm_head"].neg_())
+    pol.sync()
+    want = []
+    for _ in range(2):  # as it was for the score of `mixed`, then as it was for its decode and for `after`
+        fresh = V.Policy(sh, w, 2, 64, 64)
+        want.append(turn(fresh))
+        fresh.sync()
+        fresh.close()
+        w["lm_head"].neg_()
+    assert all(torch.equal(a, b) for a, b in zip(after, want[1]))
+    assert not any(torch.equal(a, b) for a, b in zip(after, before))
+    assert torch.equal(mixed[0], want[1][0]) and torch.equal(mixed[1], want[0][1])
+    pol.close()
