@@ -191,11 +191,14 @@ int vla_op_num_sms(void);
  *   launched from now on (0 restores the default, 1 s).  A wait that runs out sets
  *   VLA_STATUS_TIMEOUT, the CTA waits (within the same limit) for its own copies and MMAs,
  *   frees its tensor memory and exits without writing its output tile.
+ * vla_test_set_max_cluster: the clipped objective's cluster has at most this many CTAs (0 restores the
+ *   default), as on a device that cannot place larger ones.
  * vla_test_stall_next_gemm: in the next single-CTA tile GEMM launch, CTA 0 leaves its first
  *   pipeline stage unfilled, so its MMA thread waits on a barrier that nothing completes until
  *   the limit runs out (then as above).  The other CTAs run normally. */
 int vla_test_inject_launch_error(int64_t nth_launch, int cuda_error);
 int vla_test_set_wait_limit_ns(uint64_t limit_ns);
+int vla_test_set_max_cluster(int ctas);
 int vla_test_stall_next_gemm(void);
 
 #ifdef __cplusplus

@@ -298,6 +298,42 @@ inline cudaError_t allow_wide_clusters(Kern kern, std::atomic<uint64_t>& done) {
   return set_attribute_once(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1, done);
 }
 
+// Test hook: no cluster of more CTAs than this is used where the size depends on what the device can place.
+extern std::atomic<int> g_max_cluster;
+constexpr int kDefaultMaxCluster = 16;
+
+// The most CTAs (a power of two, at most `most`) of `kern` that the current device can place as one cluster:
+// a partition of a GPU, or a client with a limit on its SMs, may not hold the non-portable sizes.  Asked once
+// per (kernel, device); `known` holds the answer per device index < 64, 0 = not asked yet.
+template <typename Kern>
+inline cudaError_t max_cluster_size(Kern kern, dim3 block, size_t smem, int most, std::atomic<int> (&known)[64], int* size) {
+  int dev = 0;
+  if (const cudaError_t e = cudaGetDevice(&dev)) return e;
+  int c = dev >= 0 && dev < 64 ? known[dev].load(std::memory_order_acquire) : 0;
+  if (!c) {
+    for (c = most; c > 1; c /= 2) {
+      cudaLaunchConfig_t cfg = {};
+      cfg.gridDim = dim3(static_cast<unsigned>(c));
+      cfg.blockDim = block;
+      cfg.dynamicSmemBytes = smem;
+      cudaLaunchAttribute attr[1];
+      attr[0].id = cudaLaunchAttributeClusterDimension;
+      attr[0].val.clusterDim.x = static_cast<unsigned>(c);
+      attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
+      cfg.attrs = attr;
+      cfg.numAttrs = 1;
+      int n = 0;
+      if (cudaOccupancyMaxActiveClusters(&n, kern, &cfg) == cudaSuccess && n > 0) break;
+      cudaGetLastError();  // a size that the device refuses
+    }
+    if (dev >= 0 && dev < 64) known[dev].store(c, std::memory_order_release);
+  }
+  const int limit = g_max_cluster.load(std::memory_order_relaxed);
+  while (c > 1 && c > limit) c /= 2;
+  *size = c;
+  return cudaSuccess;
+}
+
 // Makes `dev` current for the scope of one API call and gives the caller's device back on exit
 // (the library must not change the current device of the calling thread).
 struct DeviceGuard {

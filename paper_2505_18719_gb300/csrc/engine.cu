@@ -1446,6 +1446,12 @@ int vla_test_set_wait_limit_ns(uint64_t limit_ns) {
   return VLA_OK;
 }
 
+int vla_test_set_max_cluster(int ctas) {
+  if (ctas < 0) return set_err(nullptr, VLA_ERR_ARG, "vla_test_set_max_cluster: bad argument");
+  g_max_cluster.store(ctas ? ctas : kDefaultMaxCluster);
+  return VLA_OK;
+}
+
 int vla_test_stall_next_gemm(void) {
   gemm_stall_next_launch();
   return VLA_OK;

@@ -11,6 +11,7 @@ int64_t g_launch_count = 0;
 std::atomic<int64_t> g_inject_countdown{0};
 std::atomic<int> g_inject_error{0};
 std::atomic<uint64_t> g_wait_limit_ns{kDefaultWaitLimitNs};
+std::atomic<int> g_max_cluster{kDefaultMaxCluster};
 
 namespace {
 

@@ -5,6 +5,8 @@
 //    one lane per env;
 //  * the clipped PPO objective of Eq. 2 with action log-probs as the sum of the 7 token
 //    log-probs (Eq. 1): one cluster, a fixed-order reduction, so the result is deterministic.
+#include <algorithm>
+
 #include "misc.h"
 #include "ptx.cuh"
 
@@ -280,17 +282,22 @@ int gae_launch(const float* r, const float* v, const float* done, int M, int B, 
 int ppo_clip_launch(const float* lp_new, const float* lp_old, const float* adv, int N, int A, float eps,
                     float* objective, float* ratio, float* clip_frac, cudaStream_t s) {
   if (N <= 0) return VLA_ERR_ARG;
-  // one tile per CTA up to 16 CTAs (the non-portable cluster maximum); the staging needs 16-byte
-  // aligned log-probs
+  // one tile per CTA up to 16 CTAs (the non-portable cluster maximum) or what the device can place: the
+  // CTAs take the tiles in turn at any number; the staging needs 16-byte aligned log-probs
   const int tiles = (N + kPpoTile - 1) / kPpoTile;
-  const int n_cta = tiles <= 1 ? 1 : tiles <= 2 ? 2 : tiles <= 4 ? 4 : tiles <= 8 ? 8 : 16;
+  const int want = tiles <= 1 ? 1 : tiles <= 2 ? 2 : tiles <= 4 ? 4 : tiles <= 8 ? 8 : 16;
   const bool staged = A <= kPpoMaxA && !(reinterpret_cast<uintptr_t>(lp_new) & 15) &&
                       !(reinterpret_cast<uintptr_t>(lp_old) & 15);
   static std::atomic<uint64_t> smem_done[2] = {}, cluster_done[2] = {};
+  static std::atomic<int> cluster_size[2][64] = {};
   auto go = [&](auto kern, int stages, int max_a, int which) -> cudaError_t {
     const int smem = staged ? stages * kPpoStageBytes * A : 0;
     if (const cudaError_t e = set_smem_limit(kern, stages * kPpoStageBytes * max_a, smem_done[which])) return e;
     if (const cudaError_t e = allow_wide_clusters(kern, cluster_done[which])) return e;
+    int n_cta = 1;  // asked with the most shared memory that a call takes
+    if (const cudaError_t e = max_cluster_size(kern, dim3(kPpoTile), stages * kPpoStageBytes * max_a, 16, cluster_size[which], &n_cta))
+      return e;
+    n_cta = std::min(n_cta, want);
     return launch_pdl_cluster(kern, dim3(n_cta), dim3(kPpoTile), smem, s, n_cta, lp_new, lp_old, adv, N, A,
                               staged ? 1 : 0, eps, objective, ratio, clip_frac);
   };

@@ -110,6 +110,7 @@ def load(path: str = LIB_PATH):
         "vla_op_read_status": (i32, [vp, ctypes.POINTER(u32)]),
         "vla_test_inject_launch_error": (i32, [i64, i32]),
         "vla_test_set_wait_limit_ns": (i32, [ctypes.c_uint64]),
+        "vla_test_set_max_cluster": (i32, [i32]),
         "vla_test_stall_next_gemm": (i32, []),
     }
     for name, (res, args) in sig.items():
@@ -341,6 +342,10 @@ def vla_test_inject_launch_error(nth_launch: int, cuda_error: int) -> int:
 
 def vla_test_set_wait_limit_ns(limit_ns: int) -> int:
     return load().vla_test_set_wait_limit_ns(int(limit_ns))
+
+
+def vla_test_set_max_cluster(ctas: int) -> int:
+    return load().vla_test_set_max_cluster(ctas)
 
 
 def vla_test_stall_next_gemm() -> int:

@@ -91,6 +91,17 @@ def test_ppo_clip_tile_edges(N, A, offset):
     assert abs(cf.item() - o_cf) <= (near + 0.5) / N
 
 
+# a device (a partition, a client with few SMs) that cannot place clusters of 16 CTAs: fewer CTAs take the tiles
+@pytest.mark.parametrize("most", [8, 4, 2, 1])
+def test_ppo_clip_on_smaller_clusters(most):
+    try:
+        assert V.vla_test_set_max_cluster(most) == 0
+        for N, A in ((4097, 8), (8193, 7), (25000, 12)):
+            test_ppo_clip_tile_edges(N, A, 0)
+    finally:
+        V.vla_test_set_max_cluster(0)
+
+
 def test_learning_entry_points_reject_bad_arguments():
     x = torch.zeros(4, device="cuda")
     p = x.data_ptr()
