@@ -64,6 +64,18 @@ int vla_op_gemm_decode_f16(const void* A, const void* A_lo, int lda, const void*
                            float* C, int ldc, int M, int N, int K, float* workspace,
                            size_t workspace_bytes, void* cuda_stream);
 
+/* The residual projection of a few hundred rows (§3.1 o and down projections of the PPO ratio pass,
+ * Eq. 2: 6 rows of each env): resid[M, N] (f32, row stride ldr) += A[M, K] · W[N, K]^T with fp16 operands
+ * (row strides lda, ldw, multiples of 8), on tiles of 128 weight rows by all rows, K split over
+ * clusters.  With norm_w (bf16 [N]) the RMSNorm that follows is left to the consumer: y_hi / y_lo
+ * (fp16 [M, N], y_lo may be NULL) get the updated row times norm_w, not normalised, and ss_out
+ * (f32 [N / 128, M]) the sums of squares of the updated row over each 128 columns.
+ * VLA_ERR_UNSUPPORTED for calls that the engine gives to the tile GEMMs instead: M outside 321 .. 432,
+ * N no multiple of 128 or with more tiles than clusters of four fit on the GPU at once, K < 4096, or
+ * buffers off their alignment (16 bytes; norm_w and the outputs 8). */
+int vla_op_gemm_resid_f16(const void* A, int lda, const void* W, int ldw, float* resid, int ldr, int M, int N,
+                          int K, const void* norm_w, void* y_hi, void* y_lo, float* ss_out, void* cuda_stream);
+
 /* vla_op_gemm_bf16 without a caller workspace: the paper has no counterpart; this entry
  * point exists for callers that cannot allocate device memory (all device memory owned by
  * another allocator, or a loop that must not pay the synchronisation of cudaMalloc/cudaFree).
@@ -190,12 +202,15 @@ int vla_op_num_sms(void);
  * vla_test_set_wait_limit_ns: limit of each bounded pipeline wait of the tcgen05 GEMMs
  *   launched from now on (0 restores the default, 1 s).  A wait that runs out sets
  *   VLA_STATUS_TIMEOUT, the CTA waits (within the same limit) for its own copies and MMAs,
- *   frees its tensor memory and exits without writing its output tile.
+ *   frees its tensor memory and exits without writing its output tile (nor do the CTAs of its
+ *   cluster, where several share a tile).
  * vla_test_set_max_cluster: the clipped objective's cluster has at most this many CTAs (0 restores the
  *   default), as on a device that cannot place larger ones.
- * vla_test_stall_next_gemm: in the next single-CTA tile GEMM launch, CTA 0 leaves its first
- *   pipeline stage unfilled, so its MMA thread waits on a barrier that nothing completes until
- *   the limit runs out (then as above).  The other CTAs run normally. */
+ * vla_test_stall_next_gemm: in the next launch of the single-CTA tile GEMM, of the cluster GEMM (up to
+ *   32 rows) or of the wide residual GEMM, CTA 0 leaves its first pipeline stage unfilled, so its MMA
+ *   thread waits on a barrier that nothing completes until the limit runs out (then as above).  The
+ *   other CTAs of its cluster leave their share of its output tile unwritten too; all others run
+ *   normally. */
 int vla_test_inject_launch_error(int64_t nth_launch, int cuda_error);
 int vla_test_set_wait_limit_ns(uint64_t limit_ns);
 int vla_test_set_max_cluster(int ctas);

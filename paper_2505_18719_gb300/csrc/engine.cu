@@ -1206,6 +1206,34 @@ int vla_op_gemm_decode_f16(const void* A, const void* A_lo, int lda, const void*
                         workspace_bytes, cuda_stream);
 }
 
+int vla_op_gemm_resid_f16(const void* A, int lda, const void* W, int ldw, float* resid, int ldr, int M, int N, int K,
+                          const void* norm_w, void* y_hi, void* y_lo, float* ss_out, void* cuda_stream) {
+  if (!A || !W || !resid || M < 1 || N < 1 || K < 1 || lda < K || ldw < K || ldr < N || (norm_w && (!y_hi || !ss_out)))
+    return set_err(nullptr, VLA_ERR_ARG, "vla_op_gemm_resid_f16: bad argument");
+  GemmArgs g;
+  g.A = static_cast<const bf16*>(A);
+  g.lda = lda;
+  g.B = static_cast<const bf16*>(W);
+  g.ldb = ldw;
+  g.M = M;
+  g.N = N;
+  g.K = K;
+  g.start = Start::kInOrder;
+  g.epi.kind = EPI_RESID;
+  g.epi.resid = resid;
+  g.epi.ldr = ldr;
+  g.epi.norm_w = static_cast<const bf16*>(norm_w);
+  g.epi.norm_hi = static_cast<bf16*>(y_hi);
+  g.epi.norm_lo = static_cast<bf16*>(y_lo);
+  g.epi.ldn = N;
+  g.epi.ss_out = norm_w ? ss_out : nullptr;
+  g.epi.fp16 = true;
+  if (!gemm_wide_ok(g, query_num_sms()))
+    return set_err(nullptr, VLA_ERR_UNSUPPORTED, "vla_op_gemm_resid_f16: sizes or alignment outside the kernel's range");
+  if (const int rs = op_status_word(&g.epi.status)) return rs;
+  return gemm_wide_launch(g, static_cast<cudaStream_t>(cuda_stream), nullptr);
+}
+
 size_t vla_op_gemm_decode_workspace_bytes(int M, int N, int K) {
   return gemv_workspace_bytes(M, N, K, query_num_sms());
 }

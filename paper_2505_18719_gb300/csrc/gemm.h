@@ -104,8 +104,9 @@ bool make_tensor_map_2d(CUtensorMap* m, const void* ptr, int64_t rows, int64_t c
 bool gemm_wide_ok(const GemmArgs& a, int num_sms);
 int gemm_wide_launch(const GemmArgs& a, cudaStream_t stream, GemmCost* cost);
 
-// Failure injection (test hook): in the next single-CTA tile GEMM launch, CTA 0 leaves its first
-// pipeline stage unfilled; its bounded wait on that stage runs out (VLA_STATUS_TIMEOUT).
+// Failure injection (test hook): in the next launch of the single-CTA tile GEMM, the cluster GEMM or the
+// wide residual GEMM, CTA 0 leaves its first pipeline stage unfilled; its bounded wait on that stage
+// runs out (VLA_STATUS_TIMEOUT).
 void gemm_stall_next_launch();
 int gemv_launch(const GemmArgs& a, cudaStream_t stream, int num_sms, GemmCost* cost);
 

@@ -65,6 +65,8 @@ __device__ __forceinline__ uint32_t idesc_for(uint32_t bf16_desc, bool fp16) {
   return fp16 ? (bf16_desc & ~kIdescBf16Operands) : bf16_desc;
 }
 
+std::atomic<int> g_test_stall{0};  // failure injection: consumed by one launch
+
 struct Params {
   int M, N, K;          // N: columns of B used (SwiGLU: 2F)
   int tiles_m, tiles_n, splits, kb_total, kb_per_split;
@@ -1373,6 +1375,7 @@ struct ClusterParams {
   int M, N, K, kbt;     // kbt: 64-wide k-blocks
   EpiArgs epi;
   uint64_t wait_limit;  // ns per bounded mbarrier wait
+  int stall;            // failure injection (test hook): CTA 0 never fills its first stage
 };
 
 // Copies `bytes` of this CTA's shared memory to the cluster address dst, completing on the mbarrier
@@ -1417,7 +1420,8 @@ __device__ __forceinline__ void store_kv4(f16* dst, uint8_t* res, float4 v) {
 }
 
 // Finishes this CTA's rows of the tile, kFinish items of four columns per thread at a time: what an
-// item reads from global memory is requested before `ready` (the wait for the partial sums).
+// item reads from global memory is requested before `ready` (the wait for the partial sums; false, for
+// a warp as a whole, when they are not there: nothing is stored).
 constexpr int kFinish = 2;
 template <int TR, class Ready>
 __device__ __forceinline__ void gemv_finish(const ClusterParams& p, const TileSums<TR>& t, int tile, Ready ready,
@@ -1427,7 +1431,7 @@ __device__ __forceinline__ void gemv_finish(const ClusterParams& p, const TileSu
   if (e.kind == EPI_SWIGLU) {
     constexpr int V = TR / 8;  // float4s of a row's gate half
     const int F = p.N >> 1;
-    ready();
+    if (!ready()) return;
     for (int k = tid; k < t.mn * V; k += kThreads) {
       const int i = k / V, j = (k - i * V) * 4;
       const float4 g = t.sum4(i, j), u = t.sum4(i, j + TR / 2);
@@ -1464,7 +1468,7 @@ __device__ __forceinline__ void gemv_finish(const ClusterParams& p, const TileSu
         cs[u][0] = c4[0];
         cs[u][1] = c4[1];
       }
-      if (k0 == tid) ready();
+      if (k0 == tid && !ready()) return;
 #pragma unroll
       for (int u = 0; u < kFinish; ++u) {
         const int k = k0 + u * kThreads;
@@ -1511,7 +1515,7 @@ __device__ __forceinline__ void gemv_finish(const ClusterParams& p, const TileSu
         if (resid && vec && k < t.mn * V && n + 4 <= p.N)
           x[u] = __ldcg(reinterpret_cast<const float4*>(out + static_cast<size_t>(t.m0 + k / V) * ld + n));
       }
-      if (k0 == tid) ready();
+      if (k0 == tid && !ready()) return;
 #pragma unroll
       for (int u = 0; u < kFinish; ++u) {
         const int k = k0 + u * kThreads;
@@ -1626,12 +1630,13 @@ __global__ void __launch_bounds__(kThreads, 2)
         tma_load_2d_hint(sx, &tmX, full0 + 8 * stage, kb * BK, 0, pol_x);
         tma_load_2d_hint(sx + X_BYTES, &tmX2, full0 + 8 * stage, kb * BK, 0, pol_x);
       };
-      for (int i = 0; i < pre; ++i) {
+      const int i0 = p.stall && blockIdx.x == 0 ? 1 : 0;
+      for (int i = i0; i < pre; ++i) {
         load_w(i, kb0 + i);
         issued |= 1u << i;
       }
       pdl_wait_async();
-      for (int i = 0; i < pre; ++i) load_x(i, kb0 + i);
+      for (int i = i0; i < pre; ++i) load_x(i, kb0 + i);
       int stage = pre % STAGES;
       uint32_t phase = (pre == STAGES) ? 1u : 0u;
       for (int i = pre; i < n; ++i) {
@@ -1721,6 +1726,9 @@ __global__ void __launch_bounds__(kThreads, 2)
   t.m0 = rank * ml;
   t.mn = max(0, min(ml, p.M - t.m0));
   cluster_wait();
+  // whether a CTA of the cluster gave up (set before it arrived): then nobody stores the tile.  Asked while
+  // the partials are on their way.
+  const uint32_t gave_up = lane < C ? ld_cluster_u32(mapa_shared(smem_u32(tmem_slot + 1), lane)) : 0u;
   if (warp == 0 && lane < C) {
     // lane s sends rank s its rows (an aborted CTA sends too, so that nobody waits for it)
     const int s = lane, n_s = min(ml, p.M - s * ml);
@@ -1734,7 +1742,9 @@ __global__ void __launch_bounds__(kThreads, 2)
   }
   pdl_wait();  // (long over) the residual and the caches of this step are the previous kernels'
   uint32_t sat = 0;
-  gemv_finish<TR>(p, t, tile, [&] { wait_drain_reported(recv_bar, 0, status, limit); }, sat);
+  gemv_finish<TR>(
+      p, t, tile,
+      [&] { return __all_sync(0xffffffffu, wait_drain_reported(recv_bar, 0, status, limit) && !gave_up) != 0; }, sat);
   report_saturation(status, sat);
   __syncwarp();
   cluster_arrive();
@@ -1771,6 +1781,7 @@ struct WideParams {
   int M, nb, kbt;  // nb: rows per MMA (the call's rows as two halves), a multiple of 16
   EpiArgs epi;
   uint64_t wait_limit;
+  int stall;       // as ClusterParams
 };
 __device__ __forceinline__ void st_cluster(uint32_t addr, float v) {
   asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(addr), "f"(v) : "memory");
@@ -1842,12 +1853,13 @@ __global__ void __launch_bounds__(kWideThreads, 1)
         tma_load_2d(sx, &tmX, full0 + 8 * stage, kb * BK, 0);
         tma_load_2d(sx + x_half, &tmX, full0 + 8 * stage, kb * BK, p.nb);
       };
-      for (int i = 0; i < pre; ++i) {  // the weights do not depend on the previous kernel
+      const int i0 = p.stall && blockIdx.x == 0 ? 1 : 0;
+      for (int i = i0; i < pre; ++i) {  // the weights do not depend on the previous kernel
         load_w(i, kb0 + i);
         issued |= 1u << i;
       }
       pdl_wait_async();
-      for (int i = 0; i < pre; ++i) load_x(i, kb0 + i);
+      for (int i = i0; i < pre; ++i) load_x(i, kb0 + i);
       int stage = pre % STAGES;
       uint32_t phase = (pre == STAGES) ? 1u : 0u;
       for (int i = pre; i < n; ++i) {
@@ -1895,6 +1907,8 @@ __global__ void __launch_bounds__(kWideThreads, 1)
   __syncwarp();
   cluster_arrive();
   cluster_wait();  // every CTA is done with its stages: partials may be stored over them
+  // whether a CTA of the cluster gave up (set before it arrived): then nobody stores the tile
+  const uint32_t gave_up = lane < C ? ld_cluster_u32(mapa_shared(smem_u32(tmem_slot + 1), lane)) : 0u;
   const int ml = (p.M + C - 1) / C;  // rows per rank
   float* recv = reinterpret_cast<float*>(smem);  // [rank][ml][TR]
   if (warp >= 2) {
@@ -1939,7 +1953,7 @@ __global__ void __launch_bounds__(kWideThreads, 1)
       if (k < mn * 32)
         h[u] = __ldcg(reinterpret_cast<const float4*>(e.resid + static_cast<size_t>(r0 + (k >> 5)) * e.ldr + tile * TR + (k & 31) * 4));
     }
-    if (!waited) wait_cluster_data(recv_bar, 0, status, limit);
+    if (!waited && !__all_sync(0xffffffffu, wait_cluster_data(recv_bar, 0, status, limit) && !gave_up)) break;
     waited = true;
 #pragma unroll
     for (int u = 0; u < kWideFinish; ++u) {
@@ -2260,6 +2274,7 @@ int cluster_launch_as(const GemmArgs& a, const ClusterPlan& pl, cudaStream_t str
   p.kbt = pl.kbt;
   p.epi = a.epi;
   p.wait_limit = g_wait_limit_ns.load(std::memory_order_relaxed);
+  p.stall = g_test_stall.exchange(0);
   return pl.tr == 256 ? dispatch_cluster<256>(mw, mw2, mx, mx2, p, pl, a.start, stream)
                       : dispatch_cluster<128>(mw, mw2, mx, mx2, p, pl, a.start, stream);
 }
@@ -2271,8 +2286,6 @@ bool make_tensor_map_2d(CUtensorMap* m, const void* ptr, int64_t rows, int64_t c
                         bool fp16) {
   return make_map(m, ptr, rows, cols, ld, box_rows, fp16);
 }
-
-std::atomic<int> g_test_stall{0};
 
 void gemm_stall_next_launch() { g_test_stall.store(1); }
 
@@ -2367,7 +2380,7 @@ int gemm_launch(const GemmArgs& a, cudaStream_t stream, int num_sms, GemmCost* c
     return VLA_OK;
   }
   const int grid = static_cast<int>(units < num_sms ? units : num_sms);
-  p.stall = g_test_stall.exchange(0);  // failure injection: consumed by one tile-GEMM launch
+  p.stall = g_test_stall.exchange(0);
   if (split)
     rc = (BN == 256) ? dispatch_epi<256, true>(run_epi, maps, p, grid, stream)
                      : dispatch_epi<128, true>(run_epi, maps, p, grid, stream);
@@ -2408,6 +2421,7 @@ int gemm_wide_launch(const GemmArgs& a, cudaStream_t stream, GemmCost* cost) {
   p.kbt = (a.K + BK - 1) / BK;
   p.epi = a.epi;
   p.wait_limit = g_wait_limit_ns.load(std::memory_order_relaxed);
+  p.stall = g_test_stall.exchange(0);
   CUtensorMap mw, mx;
   if (!make_map(&mw, a.B, a.N, a.K, a.ldb, 128, a.epi.fp16) || !make_map(&mx, a.A, a.M, a.K, a.lda, p.nb, a.epi.fp16))
     return cuda_fail(cudaErrorInvalidValue, "tensor maps (wide GEMM)");
@@ -2417,8 +2431,8 @@ int gemm_wide_launch(const GemmArgs& a, cudaStream_t stream, GemmCost* cost) {
   constexpr int smem_max = 227 * 1024;
   static std::atomic<uint64_t> attr_done{0};
   VLA_CUDA_TRY(set_smem_limit(gemm_wide_kernel, smem_max, attr_done));
-  VLA_CUDA_TRY(launch_pdl_cluster(gemm_wide_kernel, dim3(a.N / 128 * kWideC), dim3(kWideThreads), smem, stream, kWideC, mw,
-                                  mx, p));
+  VLA_CUDA_TRY(launch_cluster_at(a.start, gemm_wide_kernel, dim3(a.N / 128 * kWideC), dim3(kWideThreads), smem, stream,
+                                 kWideC, mw, mx, p));
   note_launch();
   VLA_CUDA_TRY(cudaGetLastError());
   if (cost) *cost = gemm_cost(a);

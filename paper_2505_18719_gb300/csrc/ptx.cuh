@@ -205,8 +205,8 @@ __device__ __forceinline__ void wait_drain(uint32_t bar, uint32_t parity, uint64
   }
 }
 // Wait for what other CTAs of the cluster stored before they arrived on this CTA's barrier; one that
-// runs out reports the timeout.
-__device__ __forceinline__ void wait_cluster_data(uint32_t bar, uint32_t parity, uint32_t* status, uint64_t limit_ns) {
+// runs out reports the timeout and returns false.
+__device__ __forceinline__ bool wait_cluster_data(uint32_t bar, uint32_t parity, uint32_t* status, uint64_t limit_ns) {
   const uint64_t t0 = globaltimer();
   while (true) {
     uint32_t ok;
@@ -217,22 +217,29 @@ __device__ __forceinline__ void wait_cluster_data(uint32_t bar, uint32_t parity,
         : "=r"(ok)
         : "r"(bar), "r"(parity)
         : "memory");
-    if (ok) return;
+    if (ok) return true;
     if (globaltimer() - t0 > limit_ns) {
       if (status) atomicOr(status, VLA_STATUS_TIMEOUT);
-      return;
+      return false;
     }
   }
 }
-// The same for data that has to arrive: a wait that runs out reports the timeout.
-__device__ __forceinline__ void wait_drain_reported(uint32_t bar, uint32_t parity, uint32_t* status, uint64_t limit_ns) {
+// wait_drain for data that has to arrive: one that runs out reports the timeout and returns false.
+__device__ __forceinline__ bool wait_drain_reported(uint32_t bar, uint32_t parity, uint32_t* status, uint64_t limit_ns) {
   const uint64_t t0 = globaltimer();
   while (!mbar_try_wait(bar, parity)) {
     if (globaltimer() - t0 > limit_ns) {
       if (status) atomicOr(status, VLA_STATUS_TIMEOUT);
-      return;
+      return false;
     }
   }
+  return true;
+}
+// A 32-bit word of shared memory anywhere in the cluster (shared::cluster address).
+__device__ __forceinline__ uint32_t ld_cluster_u32(uint32_t addr) {
+  uint32_t v;
+  asm volatile("ld.shared::cluster.u32 %0, [%1];" : "=r"(v) : "r"(addr) : "memory");
+  return v;
 }
 
 }  // namespace vla

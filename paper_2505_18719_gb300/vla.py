@@ -98,6 +98,7 @@ def load(path: str = LIB_PATH):
         "vla_op_gemm_decode_f16": (i32, [vp, vp, i32, vp, i32, vp, i32, i32, i32, i32, vp, ctypes.c_size_t, vp]),
         "vla_op_gemm_bf16_noalloc": (i32, [vp, vp, i32, vp, i32, vp, i32, i32, i32, i32, i32, i32, vp]),
         "vla_op_action_head": (i32, [vp, i32, i32, i32, vp, vp, f32, vp, f32, vp, vp, vp, vp, vp, vp, vp]),
+        "vla_op_gemm_resid_f16": (i32, [vp, i32, vp, i32, vp, i32, i32, i32, i32, vp, vp, vp, vp, vp]),
         "vla_op_num_sms": (i32, []),
         "vla_op_attn_decode": (i32, [vp, vp, i32, i32, i32, i32, vp, vp, i32, i32, i32, vp, vp, vp, ctypes.c_size_t, vp]),
         "vla_op_attn_decode_workspace_bytes": (ctypes.c_size_t, [i32, i32, i32, i32, i32]),
@@ -256,6 +257,13 @@ def vla_op_gemm_decode_f16(A_ptr, A_lo_ptr, lda, W_ptr, ldw, C_ptr, ldc, M, N, K
                            stream=0) -> int:
     return load().vla_op_gemm_decode_f16(A_ptr, A_lo_ptr, lda, W_ptr, ldw, C_ptr, ldc, M, N, K, ws_ptr,
                                          ws_bytes, stream or None)
+
+
+def vla_op_gemm_resid_f16(A_ptr, lda, W_ptr, ldw, resid_ptr, ldr, M, N, K, norm_w_ptr=0, y_hi_ptr=0, y_lo_ptr=0,
+                          ss_ptr=0, stream=0) -> int:
+    return load().vla_op_gemm_resid_f16(A_ptr or None, lda, W_ptr or None, ldw, resid_ptr or None, ldr, M, N, K,
+                                        norm_w_ptr or None, y_hi_ptr or None, y_lo_ptr or None, ss_ptr or None,
+                                        stream or None)
 
 
 def vla_op_gemm_bf16_noalloc(A_ptr, A_lo_ptr, lda, W_ptr, ldw, C_ptr, ldc, M, N, K, block_n=256,

@@ -5,8 +5,9 @@
   vla_decode_actions, leaves the handle's bookkeeping where it was, and the same calls then
   reproduce a clean run bit for bit.
 * A bounded pipeline wait that nothing completes (vla_test_stall_next_gemm: CTA 0 of the next
-  tile GEMM leaves one stage unfilled) runs out after a short limit: the status word gets
-  VLA_STATUS_TIMEOUT, the other CTAs finish, and the context stays usable.
+  tile, cluster or wide GEMM leaves one stage unfilled) runs out after a short limit: the status word
+  gets VLA_STATUS_TIMEOUT, that output tile stays unwritten, the other CTAs finish, and the context
+  stays usable.
 * An activation beyond the fp16 range is saturated with VLA_STATUS_SATURATED raised, in the
   RMSNorm op and end to end through a handle whose first norm gain is huge.
 """
@@ -108,6 +109,79 @@ def test_gemm_wait_timeout_sets_status_and_recovers():
     rc, st = V.vla_op_read_status()
     assert rc == 0 and st == 0
     assert (C.cpu().double() - ref).abs().max().item() < tol
+
+
+def test_cluster_gemm_wait_timeout_leaves_its_tile_unwritten():
+    # 16 rows, K split over a cluster: the CTAs beside the one that gives up do not store its tile either
+    M, N, K = 16, 512, 1024
+    A, A_lo, W = ((I.normal_bf16(s, 73, i, 1.0).float() * f).half().cuda()
+                  for i, s, f in ((1, (M, K), 1.0), (2, (M, K), 2.0 ** -11), (3, (N, K), 1.0)))
+    ref = (A.double() + A_lo.double()).cpu() @ W.double().cpu().T
+    tol = 2e-5 * math.sqrt(K) * 8
+    ws = torch.zeros(V.vla_op_gemm_decode_workspace_bytes(M, N, K) // 4 + 1, device="cuda")
+    C = torch.empty(M, N, device="cuda")
+
+    def run():
+        C.fill_(float("nan"))
+        assert V.vla_op_gemm_decode_f16(A.data_ptr(), A_lo.data_ptr(), K, W.data_ptr(), K, C.data_ptr(), N, M, N, K,
+                                        ws.data_ptr(), ws.numel() * 4) == 0
+        rc, st = V.vla_op_read_status()
+        assert rc == 0
+        return st, C.cpu().double()
+
+    assert V.vla_op_read_status()[0] == 0
+    assert V.vla_test_set_wait_limit_ns(500_000) == 0
+    assert V.vla_test_stall_next_gemm() == 0
+    st, c = run()
+    assert st & V.VLA_STATUS_TIMEOUT, st
+    lost = int(torch.isnan(c[0]).sum())
+    assert lost in (128, 256)                                   # one tile of weight rows
+    assert torch.isnan(c[:, :lost]).all()
+    assert (c[:, lost:] - ref[:, lost:]).abs().max().item() < tol
+    assert V.vla_test_set_wait_limit_ns(0) == 0
+    st, c = run()
+    assert st == 0 and (c - ref).abs().max().item() < tol
+
+
+def test_wide_residual_gemm_wait_timeout_leaves_its_tile_unwritten():
+    M, N, K = 384, 512, 4096
+    A, W = ((I.normal_bf16(s, 74, i, 1.0).float()).half().cuda() for i, s in ((1, (M, K)), (2, (N, K))))
+    h0 = I.normal_bf16((M, N), 74, 3, 1.0).float().cuda()
+    ref = h0.double().cpu() + A.double().cpu() @ W.double().cpu().T
+    tol = 2e-5 * math.sqrt(K) * 8
+    assert V.vla_op_read_status()[0] == 0
+    assert V.vla_test_set_wait_limit_ns(500_000) == 0
+    assert V.vla_test_stall_next_gemm() == 0
+    h = h0.clone()
+    assert V.vla_op_gemm_resid_f16(A.data_ptr(), K, W.data_ptr(), K, h.data_ptr(), N, M, N, K) == 0
+    rc, st = V.vla_op_read_status()
+    assert rc == 0 and st & V.VLA_STATUS_TIMEOUT, st
+    assert torch.equal(h[:, :128], h0[:, :128])                 # the stalled CTA's cluster stored nothing
+    assert (h.cpu().double() - ref)[:, 128:].abs().max().item() < tol
+    assert V.vla_test_set_wait_limit_ns(0) == 0
+    h = h0.clone()
+    assert V.vla_op_gemm_resid_f16(A.data_ptr(), K, W.data_ptr(), K, h.data_ptr(), N, M, N, K) == 0
+    assert V.vla_op_read_status() == (0, 0)
+    assert (h.cpu().double() - ref).abs().max().item() < tol
+
+
+def test_engine_reports_cluster_gemm_timeout_then_runs_clean(wdev):
+    inp = I.make_turn_inputs(WL, 0)
+    pol = V.Policy(WL.shape, wdev, WL.batch, 128, 512)
+    ref = _turn(pol, inp)
+    pol.reset()
+    pol.prefill(inp.visual.cuda(), inp.ids.cuda(), inp.lengths)
+    pol.sync()
+    assert V.vla_test_set_wait_limit_ns(500_000) == 0
+    assert V.vla_test_stall_next_gemm() == 0
+    pol.decode(inp.uniforms.cuda(), WL.temperature)             # the first decode step's q|k|v
+    assert V.vla_sync(pol.h) == V.VLA_ERR_DEVICE_STATUS
+    assert "timed out" in V.vla_last_error(pol.h)
+    assert V.vla_test_set_wait_limit_ns(0) == 0
+    out = pol.decode(inp.uniforms.cuda(), WL.temperature)       # the same turn again
+    pol.sync()
+    _same({k: v.cpu() for k, v in out.items() if v is not None}, ref)
+    pol.close()
 
 
 def test_engine_reports_gemm_timeout_then_runs_clean(wdev):
