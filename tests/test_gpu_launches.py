@@ -1,9 +1,13 @@
-"""Weights that a call reads before it waits for the kernel ahead of it are complete when it starts.
+"""What captured calls show of their launches: orders and kernels.
+
+Weights that a call reads before it waits for the kernel ahead of it are complete when it starts.
 
 The caller's weights are read in place at every call.  A kernel launched with programmatic stream
 serialization may start while the kernel before it is still running, so the first kernel of a call that
 reads weights ahead of its wait has to be launched in stream order.  Captured into a graph, the two kinds
 of launch give edges of different types, which shows the order without running anything.
+
+The nodes of the graph show which kernels a call of a given size runs on.
 """
 import ctypes
 import dataclasses
@@ -19,6 +23,7 @@ pytestmark = pytest.mark.gpu
 WL = I.WORKLOADS["tiny_b4"]
 RELAXED = 2
 FULL, PROGRAMMATIC = 0, 1
+GEMMS = ("gemm_tc_kernel", "gemm_tc2_kernel", "gemm_wide_kernel", "gemv_cluster_kernel", "gemv_stream_kernel")
 
 
 class EdgeData(ctypes.Structure):
@@ -26,17 +31,50 @@ class EdgeData(ctypes.Structure):
                 ("reserved", ctypes.c_ubyte * 5)]
 
 
-def _edge_types(stream, calls):
-    """The edge types of a captured chain of calls, in the order of the chain."""
+class KernelNode(ctypes.Structure):
+    _fields_ = [("func", ctypes.c_void_p)] + [(n, ctypes.c_uint) for n in ("gx", "gy", "gz", "bx", "by", "bz", "smem")] + \
+               [(n, ctypes.c_void_p) for n in ("params", "extra", "kern", "ctx")]
+
+
+def _capture(cu, stream, calls):
     assert all(c() in (0, None) for c in calls)  # every kernel is loaded before the capture
     stream.synchronize()
-    cu = ctypes.CDLL("libcuda.so.1")
     graph = ctypes.c_void_p()
     st = ctypes.c_void_p(stream.cuda_stream)
     assert cu.cuStreamBeginCapture_v2(st, RELAXED) == 0
     rcs = [c() for c in calls]
     assert cu.cuStreamEndCapture(st, ctypes.byref(graph)) == 0
     assert all(rc in (0, None) for rc in rcs), rcs
+    return graph
+
+
+def _kernel_names(stream, calls):
+    """The (mangled) names of the kernels that the calls launch."""
+    cu = ctypes.CDLL("libcuda.so.1")
+    graph = _capture(cu, stream, calls)
+    n = ctypes.c_size_t(0)
+    assert cu.cuGraphGetNodes(graph, None, ctypes.byref(n)) == 0
+    nodes = (ctypes.c_void_p * n.value)()
+    assert cu.cuGraphGetNodes(graph, nodes, ctypes.byref(n)) == 0
+    names = []
+    for node in nodes:
+        kind, p, name = ctypes.c_int(-1), KernelNode(), ctypes.c_char_p()
+        assert cu.cuGraphNodeGetType(ctypes.c_void_p(node), ctypes.byref(kind)) == 0
+        if kind.value != 0:  # not a kernel
+            continue
+        assert cu.cuGraphKernelNodeGetParams_v2(ctypes.c_void_p(node), ctypes.byref(p)) == 0
+        rc = (cu.cuFuncGetName(ctypes.byref(name), ctypes.c_void_p(p.func)) if p.func
+              else cu.cuKernelGetName(ctypes.byref(name), ctypes.c_void_p(p.kern)))
+        assert rc == 0
+        names.append(name.value.decode())
+    assert cu.cuGraphDestroy(graph) == 0
+    return names
+
+
+def _edge_types(stream, calls):
+    """The edge types of a captured chain of calls, in the order of the chain."""
+    cu = ctypes.CDLL("libcuda.so.1")
+    graph = _capture(cu, stream, calls)
     n = ctypes.c_size_t(0)
     assert cu.cuGraphGetEdges_v2(graph, None, None, None, ctypes.byref(n)) == 0
     src, dst, data = (ctypes.c_void_p * n.value)(), (ctypes.c_void_p * n.value)(), (EdgeData * n.value)()
@@ -151,4 +189,40 @@ def test_gains_embeddings_and_lm_head_are_read_at_every_call(action_dim):
     assert all(torch.equal(a, b) for a, b in zip(after, want[1]))
     assert not any(torch.equal(a, b) for a, b in zip(after, before))
     assert torch.equal(mixed[0], want[1][0]) and torch.equal(mixed[1], want[0][1])
+    pol.close()
+
+
+@pytest.mark.parametrize("B", [53, 54, 72, 73])
+def test_score_pass_runs_o_and_down_on_the_wide_gemm(B):
+    # 324 to 432 score rows; 318 and 438 stay on the tile GEMMs
+    sh = I.ModelShape("tiny", 2, 4096, 32, 128, 4616)
+    s = torch.cuda.Stream()
+    pol = V.Policy(sh, P.weights_to_device(I.make_weights(sh, 11)), B, 32, B * 2, stream=s)
+    ids = torch.zeros(B, 2, dtype=torch.int32, device="cuda")
+    tok = torch.full((B, sh.action_dim), sh.vocab - 1, dtype=torch.int32, device="cuda")
+    lp = torch.zeros(B, sh.action_dim, device="cuda")
+    torch.cuda.synchronize()
+    pol.prefill(None, ids, [2] * B)
+    names = _kernel_names(s, [lambda: V.vla_score_actions(pol.h, tok.data_ptr(), 1.0, lp.data_ptr())])
+    gemms = [k for n in names for k in GEMMS if k in n]  # q|k|v, o, gate|up, down of each layer
+    o_down = "gemm_wide_kernel" if 54 <= B <= 72 else "gemm_tc_kernel"
+    assert gemms == ["gemm_tc_kernel", o_down] * (2 * sh.n_layers)
+    pol.close()
+
+
+@pytest.mark.parametrize("B,kernel", [(1, "gemv_cluster_kernel"), (32, "gemv_cluster_kernel"), (33, "gemv_stream_kernel"),
+                                      (128, "gemv_stream_kernel"), (129, "gemm_tc_kernel")])
+def test_decode_projections_kernel_by_rows(B, kernel):
+    s = torch.cuda.Stream()
+    pol = V.Policy(WL.shape, P.weights_to_device(I.make_weights(WL.shape, 3)), B, 32, B * 2, stream=s)
+    ids = torch.zeros(B, 2, dtype=torch.int32, device="cuda")
+    u = torch.full((B, WL.shape.action_dim, 256), 0.5, device="cuda")
+    i32 = torch.zeros(B, WL.shape.action_dim, dtype=torch.int32, device="cuda")
+    f32 = [torch.zeros(B, WL.shape.action_dim, device="cuda") for _ in range(2)]
+    torch.cuda.synchronize()
+    pol.prefill(None, ids, [2] * B)
+    names = _kernel_names(s, [lambda: V.vla_decode_actions(pol.h, u.data_ptr(), 1.0, 0, i32.data_ptr(),
+                                                           f32[0].data_ptr(), f32[1].data_ptr(), 0)])
+    gemms = [k for n in names for k in GEMMS if k in n]
+    assert gemms == [kernel] * (6 * 4 * WL.shape.n_layers)
     pol.close()

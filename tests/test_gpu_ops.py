@@ -627,3 +627,54 @@ def test_attn_rows8_matches_fp64(hd):
             sc = torch.einsum("hd,hnd->hn", q[r0 + i].reshape(H, hd).double(), k) / math.sqrt(hd)
             o = torch.einsum("hn,hnd->hd", torch.softmax(sc, -1), v)
             assert (out[r0 + i] - o).abs().max().item() < 4 * 2.0 ** -17 + 1e-5, (env, i)
+
+
+@pytest.mark.parametrize("M,N,K", [
+    (321, 128, 4096),      # the fewest rows: an odd split over four ranks, 31 rows of padding
+    (322, 640, 4104),      # a K tail
+    (384, 4096, 4096),     # o of the 7B shape, 64 envs
+    (384, 4096, 11008),    # down
+    (431, 256, 4160),
+    (432, 512, 8200),      # the most rows
+])
+def test_wide_residual_gemm_matches_fp64(M, N, K):
+    """resid += A W^T, and with a gain the unnormalised operand pair and the sums of squares of the RMSNorm
+    that follows.  fp16 operands are exact, so the sum's error is that of fp32 accumulation."""
+    A = I.normal_bf16((M, K), 97, 1, 1.0).float().half().cuda()
+    W = I.normal_bf16((N, K), 97, 2, 1.0).float().half().cuda()
+    h0 = I.normal_bf16((M, N), 97, 3, 30.0).float().cuda()
+    gain = I.normal_bf16((N,), 97, 4, 1.0).cuda()
+    ref = (h0.double() + A.double() @ W.double().T)
+    outs = []
+    for norm in (False, True, True):
+        h = h0.clone()
+        yh, yl = (torch.full((M, N), float("nan"), dtype=torch.float16, device="cuda") for _ in range(2))
+        ss = torch.full((N // 128, M), float("nan"), device="cuda")
+        assert V.vla_op_gemm_resid_f16(A.data_ptr(), K, W.data_ptr(), K, h.data_ptr(), N, M, N, K,
+                                       *((gain.data_ptr(), yh.data_ptr(), yl.data_ptr(), ss.data_ptr()) if norm else ())) == 0
+        assert V.vla_op_read_status() == (0, 0)
+        assert (h.double() - ref).abs().max().item() < 2e-5 * math.sqrt(K) * 8
+        outs.append((h, yh, yl, ss))
+    h, yh, yl, ss = outs[1]
+    assert torch.equal(h, outs[0][0])
+    assert all(torch.equal(a, b) for a, b in zip(outs[1], outs[2]))  # a fixed order of summation
+    # 128 squares in fp32; the pair holds 2^-21 of a value (2^-24 absolute among fp16's subnormals)
+    sq = h.double().square().view(M, N // 128, 128).sum(-1).T
+    assert ((ss.double() - sq).abs() <= 128 * 2.0 ** -24 * sq).all()
+    y = h.double() * gain.double()
+    assert ((yh.double() + yl.double() - y).abs() <= y.abs() * 2.0 ** -21 + 2.0 ** -24).all()
+
+
+def test_wide_residual_gemm_range():
+    # the sizes that the engine leaves to the tile GEMMs are refused, nothing runs
+    A = torch.zeros(433, 4096, dtype=torch.float16, device="cuda")
+    W = torch.zeros(4352, 4096, dtype=torch.float16, device="cuda")
+    h = torch.full((433, 4352), 2.0, device="cuda")
+    call = lambda M, N, K, off=0: V.vla_op_gemm_resid_f16(A.data_ptr() + off, 4096, W.data_ptr(), 4096,  # noqa: E731
+                                                          h.data_ptr(), 4352, M, N, K)
+    for M, N, K in ((320, 256, 4096), (433, 256, 4096), (384, 192, 4096), (384, 4224, 4096), (384, 256, 4088)):
+        assert call(M, N, K) == V.VLA_ERR_UNSUPPORTED, (M, N, K)
+    assert call(384, 256, 4096, off=8) == V.VLA_ERR_UNSUPPORTED
+    assert call(0, 256, 4096) == V.VLA_ERR_ARG
+    assert call(384, 4096, 4096) == 0
+    assert (h == 2.0).all() and V.vla_op_read_status() == (0, 0)
