@@ -202,8 +202,8 @@ int vla_op_num_sms(void);
  * vla_test_set_wait_limit_ns: limit of each bounded pipeline wait of the tcgen05 GEMMs
  *   launched from now on (0 restores the default, 1 s).  A wait that runs out sets
  *   VLA_STATUS_TIMEOUT, the CTA waits (within the same limit) for its own copies and MMAs,
- *   frees its tensor memory and exits without writing its output tile (nor do the CTAs of its
- *   cluster, where several share a tile).
+ *   frees its tensor memory and exits without writing its output tile.  Where several CTAs share a
+ *   tile, the others' wait for its share runs out as well and nobody writes it.
  * vla_test_set_max_cluster: the clipped objective's cluster has at most this many CTAs (0 restores the
  *   default), as on a device that cannot place larger ones.
  * vla_test_stall_next_gemm: in the next launch of the single-CTA tile GEMM, of the cluster GEMM (up to

@@ -1726,15 +1726,14 @@ __global__ void __launch_bounds__(kThreads, 2)
   t.m0 = rank * ml;
   t.mn = max(0, min(ml, p.M - t.m0));
   cluster_wait();
-  // whether a CTA of the cluster gave up (set before it arrived): then nobody stores the tile.  Asked while
-  // the partials are on their way.
-  const uint32_t gave_up = lane < C ? ld_cluster_u32(mapa_shared(smem_u32(tmem_slot + 1), lane)) : 0u;
+  const bool gave_up = *abort_flag != 0;
   if (warp == 0 && lane < C) {
-    // lane s sends rank s its rows (an aborted CTA sends too, so that nobody waits for it)
+    // lane s sends rank s its rows.  A CTA that gave up sends nothing: the others' wait for its rows runs out
+    // too, and none of them stores the tile.
     const int s = lane, n_s = min(ml, p.M - s * ml);
     if (s == rank) {
       mbar_arrive_expect_tx(recv_bar, static_cast<uint32_t>((C - 1) * t.mn * TR * 4));
-    } else if (n_s > 0) {
+    } else if (n_s > 0 && !gave_up) {
       const int slot = rank - (rank > s ? 1 : 0);
       bulk_copy_cluster(mapa_shared(smem_u32(t.recv + slot * ml * TR), s), smem_u32(t.part + s * ml * TR),
                         static_cast<uint32_t>(n_s * TR * 4), mapa_shared(recv_bar, s));
@@ -1744,7 +1743,7 @@ __global__ void __launch_bounds__(kThreads, 2)
   uint32_t sat = 0;
   gemv_finish<TR>(
       p, t, tile,
-      [&] { return __all_sync(0xffffffffu, wait_drain_reported(recv_bar, 0, status, limit) && !gave_up) != 0; }, sat);
+      [&] { return __all_sync(0xffffffffu, wait_drain_reported(recv_bar, 0, status, limit)) != 0 && !gave_up; }, sat);
   report_saturation(status, sat);
   __syncwarp();
   cluster_arrive();
@@ -1907,12 +1906,11 @@ __global__ void __launch_bounds__(kWideThreads, 1)
   __syncwarp();
   cluster_arrive();
   cluster_wait();  // every CTA is done with its stages: partials may be stored over them
-  // whether a CTA of the cluster gave up (set before it arrived): then nobody stores the tile
-  const uint32_t gave_up = lane < C ? ld_cluster_u32(mapa_shared(smem_u32(tmem_slot + 1), lane)) : 0u;
   const int ml = (p.M + C - 1) / C;  // rows per rank
   float* recv = reinterpret_cast<float*>(smem);  // [rank][ml][TR]
   if (warp >= 2) {
-    // for each row the 32 lanes of a warp store 32 consecutive floats (an aborted CTA arrives too)
+    // for each row the 32 lanes of a warp store 32 consecutive floats.  A CTA that gave up neither stores nor
+    // arrives: the others' wait for its rows runs out too, and none of them stores the tile.
     if (ok) {
       tc_fence_after();
       const int q = warp & 3, half = (warp - 2) >> 2;  // TMEM lane quarter; half of the rows
@@ -1936,9 +1934,9 @@ __global__ void __launch_bounds__(kWideThreads, 1)
         }
       }
       tc_fence_before();
+      __syncwarp();
+      if (lane < C) mbar_arrive_cluster(mapa_shared(recv_bar, lane));
     }
-    __syncwarp();
-    if (lane < C) mbar_arrive_cluster(mapa_shared(recv_bar, lane));
   }
   pdl_wait();  // (long over) the residual is the previous kernels'
   const EpiArgs& e = p.epi;
@@ -1953,7 +1951,7 @@ __global__ void __launch_bounds__(kWideThreads, 1)
       if (k < mn * 32)
         h[u] = __ldcg(reinterpret_cast<const float4*>(e.resid + static_cast<size_t>(r0 + (k >> 5)) * e.ldr + tile * TR + (k & 31) * 4));
     }
-    if (!waited && !__all_sync(0xffffffffu, wait_cluster_data(recv_bar, 0, status, limit) && !gave_up)) break;
+    if (!waited && !__all_sync(0xffffffffu, wait_cluster_data(recv_bar, 0, status, limit))) break;
     waited = true;
 #pragma unroll
     for (int u = 0; u < kWideFinish; ++u) {
@@ -1985,7 +1983,6 @@ __global__ void __launch_bounds__(kWideThreads, 1)
       }
     }
   }
-  if (!waited) wait_cluster_data(recv_bar, 0, status, limit);
   report_saturation(status, sat);
   __syncthreads();  // TMEM has been read
   cluster_arrive();
@@ -1994,7 +1991,7 @@ __global__ void __launch_bounds__(kWideThreads, 1)
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(TMEM_COLS)
                  : "memory");
   }
-  cluster_wait();  // no CTA leaves before all have what they were sent (or gave up waiting)
+  cluster_wait();  // no CTA leaves while another may still store into it
 }
 
 // ----------------------------------------------------------------------------- host side

@@ -235,11 +235,5 @@ __device__ __forceinline__ bool wait_drain_reported(uint32_t bar, uint32_t parit
   }
   return true;
 }
-// A 32-bit word of shared memory anywhere in the cluster (shared::cluster address).
-__device__ __forceinline__ uint32_t ld_cluster_u32(uint32_t addr) {
-  uint32_t v;
-  asm volatile("ld.shared::cluster.u32 %0, [%1];" : "=r"(v) : "r"(addr) : "memory");
-  return v;
-}
 
 }  // namespace vla
