@@ -206,7 +206,8 @@ __device__ __forceinline__ float silu_f(float x) { return x / (1.0f + expf(-x));
 // call starts.  (A call's uploads order the stream as well, where it has any.)
 // A kernel that allocates tensor memory lets its successor start only once it holds it (after the
 // barrier that follows tcgen05.alloc): a successor's CTA on the same SM could otherwise take the columns
-// first and wait for this kernel, while this kernel's allocation waits for that CTA.
+// first and wait for this kernel, while this kernel's allocation waits for that CTA.  (gemv_stream_kernel,
+// beside which no such CTA fits, lets it start at once.)
 __device__ __forceinline__ void pdl_launch_dependents() {
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 }
