@@ -903,6 +903,133 @@ __global__ void __launch_bounds__(NW * 32, decode_ctas_per_sm(HD)) attn_decode_k
   if (threadIdx.x == 0) counters[bh] = 0;  // ready for the next launch
 }
 
+// One query per (env, head) over a short context, when there are many pairs: a CTA lives for one or two steps
+// of 16 keys per warp, so its time is latency and what counts is how many are resident.  fp32 FMAs on 72
+// registers let 14 CTAs share an SM (the kernel above: 6 or 8; decode_short has both sides).  LPK lanes read one key row, 16 bytes
+// (and 4 bytes of codes) each; a lane group has 4 keys and values in flight; its dot products meet by
+// shuffles; the groups' online softmax states merge through shared memory in a fixed order.
+template <int HD, bool RES, int NW = kDecodeWarps>
+__global__ void __launch_bounds__(NW * 32, RES ? 14 : 1) attn_decode_short_kernel(
+    const float* q, const RowInfo* rows, KVLayout kv, int layer, int H, float scale_log2, bf16* __restrict__ out_hi,
+    bf16* __restrict__ out_lo, bool fp16) {
+  constexpr int LPK = HD / 8;    // lanes per key row
+  constexpr int KPI = 32 / LPK;  // key rows per warp instruction
+  constexpr int U = 4;           // key rows per lane group loaded ahead
+  __shared__ float s_m[NW][KPI], s_l[NW][KPI];
+  __shared__ float s_o[NW][KPI][HD];
+
+  pdl_launch_dependents();
+  pdl_wait();
+  const int b = blockIdx.x / H, head = blockIdx.x - b * H;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int sub = lane / LPK, part = lane - sub * LPK;
+  const int env = __ldcg(&rows[b].env), k_end = __ldcg(&rows[b].pos) + 1;
+  const size_t off = static_cast<size_t>(b) * H * HD + head * HD;
+
+  float qv[8];
+  {
+    const float4* qp = reinterpret_cast<const float4*>(q + off + part * 8);
+    const float4 a = __ldcg(qp), c = __ldcg(qp + 1);
+    const float v[8] = {a.x, a.y, a.z, a.w, c.x, c.y, c.z, c.w};
+#pragma unroll
+    for (int e = 0; e < 8; ++e) qv[e] = v[e] * scale_log2;
+  }
+  const f16* kbase = kv.base + static_cast<int64_t>(layer) * kv.layer_stride + static_cast<int64_t>(env) * kv.env_stride +
+                     static_cast<int64_t>(head) * kv.head_stride;
+  const f16* vbase = kbase + kv.kv_stride;
+  const uint8_t* kres = RES ? kv.res + (kbase - kv.base) / 2 : nullptr;
+  const uint8_t* vres = RES ? kres + kv.kv_stride / 2 : nullptr;
+
+  float m = -INFINITY, l = 0.f, o[8];
+#pragma unroll
+  for (int e = 0; e < 8; ++e) o[e] = 0.f;
+  for (int key0 = warp * KPI * U; key0 < k_end; key0 += NW * KPI * U) {
+    uint4 kk[U], vv[U];
+    uint32_t kc[U], vc[U];
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      const int key = key0 + u * KPI + sub;
+      kk[u] = vv[u] = make_uint4(0u, 0u, 0u, 0u);
+      kc[u] = vc[u] = 0u;
+      if (key < k_end) {
+        kk[u] = *reinterpret_cast<const uint4*>(kbase + static_cast<int64_t>(key) * HD + part * 8);
+        vv[u] = *reinterpret_cast<const uint4*>(vbase + static_cast<int64_t>(key) * HD + part * 8);
+        if (RES) {
+          kc[u] = *reinterpret_cast<const uint32_t*>(kres + static_cast<int64_t>(key) * (HD / 2) + part * 4);
+          vc[u] = *reinterpret_cast<const uint32_t*>(vres + static_cast<int64_t>(key) * (HD / 2) + part * 4);
+        }
+      }
+    }
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      const uint32_t w[4] = {kk[u].x, kk[u].y, kk[u].z, kk[u].w};
+      float acc = 0.f;
+#pragma unroll
+      for (int e = 0; e < 4; ++e) {
+        const float2 f = unpack_f16x2(w[e]);
+        acc = fmaf(qv[2 * e], f.x, acc);
+        acc = fmaf(qv[2 * e + 1], f.y, acc);
+      }
+      if (RES) {
+        const uint4 kl = kv_res_lo8(kk[u], kc[u]);
+        const uint32_t wl[4] = {kl.x, kl.y, kl.z, kl.w};
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+          const float2 f = unpack_f16x2(wl[e]);
+          acc = fmaf(qv[2 * e], f.x, acc);
+          acc = fmaf(qv[2 * e + 1], f.y, acc);
+        }
+      }
+#pragma unroll
+      for (int x = LPK / 2; x > 0; x >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, x);
+      if (key0 + u * KPI + sub < k_end) {  // the same for all lanes of a key row
+        const float m_new = fmaxf(m, acc);
+        const float alpha = exp2f(m - m_new), p = exp2f(acc - m_new);
+        m = m_new;
+        l = l * alpha + p;
+        const uint32_t v4[4] = {vv[u].x, vv[u].y, vv[u].z, vv[u].w};
+        uint32_t vl4[4] = {0u, 0u, 0u, 0u};
+        if (RES) {
+          const uint4 vl = kv_res_lo8(vv[u], vc[u]);
+          vl4[0] = vl.x;
+          vl4[1] = vl.y;
+          vl4[2] = vl.z;
+          vl4[3] = vl.w;
+        }
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+          const float2 f = unpack_f16x2(v4[e]), fl = unpack_f16x2(vl4[e]);
+          o[2 * e] = fmaf(p, f.x + fl.x, o[2 * e] * alpha);
+          o[2 * e + 1] = fmaf(p, f.y + fl.y, o[2 * e + 1] * alpha);
+        }
+      }
+    }
+  }
+  if (part == 0) {
+    s_m[warp][sub] = m;
+    s_l[warp][sub] = l;
+  }
+#pragma unroll
+  for (int e = 0; e < 8; ++e) s_o[warp][sub][part * 8 + e] = o[e];
+  __syncthreads();
+  // merge the groups' states in order (-inf: a group without keys)
+  float M = -INFINITY;
+  for (int w = 0; w < NW; ++w)
+    for (int k = 0; k < KPI; ++k) M = fmaxf(M, s_m[w][k]);
+  float L = 0.f;
+  for (int w = 0; w < NW; ++w)
+    for (int k = 0; k < KPI; ++k)
+      if (s_m[w][k] != -INFINITY) L += s_l[w][k] * exp2f(s_m[w][k] - M);
+  uint32_t sat = 0;  // convex combinations of cached values: the fp16 split never saturates
+  for (int c = threadIdx.x; c < HD; c += NW * 32) {
+    float acc = 0.f;
+    for (int w = 0; w < NW; ++w)
+      for (int k = 0; k < KPI; ++k)
+        if (s_m[w][k] != -INFINITY) acc += s_o[w][k][c] * exp2f(s_m[w][k] - M);
+    store_split1(out_hi, out_lo, off + c, acc / L, fp16, sat);
+  }
+}
+
 // ------------------------------------------------------------------ up to 8 rows (residual cache)
 // Query tiles of at most 8 rows (the teacher-forced action rows of the score pass) with the decode kernel's
 // layout and ring: the 8 columns of the small operand are the rows, and an fp32 value is an fp16 pair,
@@ -1186,6 +1313,27 @@ int attn_rows_launch(const float* q, bf16* out_hi, bf16* out_lo, const AttnTile*
     VLA_CUDA_TRY(set_smem_limit(attn_rows_kernel<64>, RowsSmem<64>::SMEM, attr_done));
     VLA_CUDA_TRY(launch_pdl(attn_rows_kernel<64>, grid, dim3(128), RowsSmem<64>::SMEM, stream, q, out_hi, out_lo,
                             tiles, kv, layer, H, scale_log2, fp16, write_lo));
+  }
+  note_launch();
+  VLA_CUDA_TRY(cudaGetLastError());
+  return VLA_OK;
+}
+
+int attn_decode_short_launch(const float* q, bf16* out_hi, bf16* out_lo, const RowInfo* rows, int B, KVLayout kv,
+                             int layer, int H, int hd, cudaStream_t stream, bool fp16) {
+  if (B <= 0) return VLA_OK;
+  const float scale_log2 = 1.4426950408889634f / sqrtf(static_cast<float>(hd));
+  auto go = [&](auto kern) {
+    return launch_pdl(kern, dim3(static_cast<unsigned>(B) * H), dim3(kDecodeWarps * 32), 0, stream, q, rows, kv, layer, H,
+                      scale_log2, out_hi, out_lo, fp16);
+  };
+  const bool res = kv.res != nullptr;
+  if (hd == 128) {
+    VLA_CUDA_TRY(res ? go(attn_decode_short_kernel<128, true>) : go(attn_decode_short_kernel<128, false>));
+  } else if (hd == 64) {
+    VLA_CUDA_TRY(res ? go(attn_decode_short_kernel<64, true>) : go(attn_decode_short_kernel<64, false>));
+  } else {
+    return VLA_ERR_UNSUPPORTED;
   }
   note_launch();
   VLA_CUDA_TRY(cudaGetLastError());

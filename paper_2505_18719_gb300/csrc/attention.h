@@ -42,4 +42,20 @@ int attn_decode_launch(const float* q, bf16* out_hi, bf16* out_lo, const RowInfo
 // CTAs of the kernel that an SM holds.
 constexpr int decode_ctas_per_sm(int hd) { return hd == 64 ? 8 : 6; }
 
+// The same on the kernel for many (env, head) pairs over short contexts, one CTA per pair.
+int attn_decode_short_launch(const float* q, bf16* out_hi, bf16* out_lo, const RowInfo* rows, int B, KVLayout kv,
+                             int layer, int H, int hd, cudaStream_t stream, bool fp16);
+// Where it is the faster one when the cache comes from HBM.  A decode's time on attn_decode_launch's kernel
+// over that on this one, in 8 layers of 8 64-wide heads (envs x 8 pairs) and two 7B layers (envs x 32 pairs), at
+// 24 / 100 / 130 / 200 positions, 152 SMs:
+//   64-wide   512 pairs .97 / .93 / .91 / .87   640 1.04 / 1.02 / 1.00 / .97   768 1.05 / 1.06 / 1.04 / 1.01
+//             1024 1.06 / 1.05 / 1.03 / 1.00    1536 1.08 / 1.04 / 1.02 / .99  2048 1.12 / 1.09 / 1.08
+//   128-wide  992 at 60 to 100 .99               1056 1.03 / 1.02 / .99 / .98   1824 1.04 / 1.02 / 1.00 / .98
+//             3072 1.08 / 1.02 / 1.00 / .98     4096 1.10 / 1.06 / 1.05 / 1.02 8192 1.14 / 1.08 / 1.05
+// (256 envs x 8 positions: 3738 against 3271 us, and 3348 against 2807 in the 7B layers.)
+constexpr bool decode_short(int pairs, int max_ctx, int hd, int num_sms) {
+  const int few = (hd == 64 ? 4 : 7) * num_sms, many = (hd == 64 ? 5 : 24) * num_sms;
+  return pairs > few && max_ctx <= (hd == 64 ? (pairs > many ? 160 : 112) : (pairs > many ? 192 : 128));
+}
+
 }  // namespace vla

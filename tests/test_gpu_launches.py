@@ -226,3 +226,54 @@ def test_decode_projections_kernel_by_rows(B, kernel):
     gemms = [k for n in names for k in GEMMS if k in n]
     assert gemms == [kernel] * (6 * 4 * WL.shape.n_layers)
     pol.close()
+
+
+def test_decode_of_many_envs_over_short_contexts():
+    # 120 envs x 8 heads, and a model larger than L2: decode attention on the kernel for many pairs.  The logits are those of a small batch, on the other kernel: both run on
+    # operand pairs (2^-21) through 24 layers
+    sh = I.ModelShape("tiny", 24, 512, 8, 64, 1368)
+    B, n = 120, 8
+    w = P.weights_to_device(I.make_weights(sh, 3))
+    ids = I.randint_i32((B, 1), 5, 6, 0, sh.vocab - 257).cuda()
+    u = I.uniform_f32((B, sh.action_dim, 256), 5, 7).cuda()
+    tok = I.randint_i32((B, sh.action_dim), 5, 8, sh.vocab - 256, sh.vocab - 1).cuda()
+    s = torch.cuda.Stream()
+    torch.cuda.synchronize()
+    z, names = [], []
+    for envs in (B, n):
+        pol = V.Policy(sh, w, envs, 160, 1024, stream=s)
+        with torch.cuda.stream(s):
+            pol.prefill(None, ids, [1] * envs)
+            out = pol.decode(u, 1.0, forced=tok)
+            pol.sync()
+            z.append(out["logits"][:n].double())
+            names.append(_kernel_names(s, [lambda: V.vla_decode_actions(
+                pol.h, u.data_ptr(), 1.0, tok.data_ptr(), out["tokens"].data_ptr(), out["logprobs"].data_ptr(),
+                out["actions"].data_ptr(), 0)]))
+        pol.close()
+    assert ((z[0] - z[1]).norm() / z[1].norm()).item() < 1e-4
+    short = [sum("attn_decode_short_kernel" in x for x in k) for k in names]
+    assert short == [6 * sh.n_layers, 0]
+    assert [sum("attn_decode" in x for x in k) for k in names] == [6 * sh.n_layers] * 2
+
+
+@pytest.mark.parametrize("hd,per_sm,over,ctx,short", [
+    (64, 4, 1, 112, True), (64, 4, 0, 112, False), (64, 4, 1, 113, False), (64, 5, 1, 160, True), (64, 5, 1, 161, False),
+    (128, 7, 1, 128, True), (128, 7, 0, 128, False), (128, 7, 1, 129, False), (128, 24, 1, 192, True),
+    (128, 24, 1, 193, False)])
+def test_decode_attention_kernel_by_pairs_and_positions(hd, per_sm, over, ctx, short):
+    H, s = 8, torch.cuda.Stream()
+    B = (per_sm * V.vla_op_num_sms() + H - 1) // H + over
+    cap = (ctx + 15) // 16 * 16
+    q = torch.zeros(B, H, hd, device="cuda")
+    kv = torch.zeros(1, 2, H, cap, hd, dtype=torch.float16, device="cuda")
+    env, pos = (torch.full((B,), v, dtype=torch.int32, device="cuda") for v in (0, ctx - 1))
+    out = torch.zeros(2, B, H * hd, dtype=torch.bfloat16, device="cuda")
+    nbytes = V.vla_op_attn_decode_workspace_bytes(B, H, hd, ctx)
+    ws = torch.zeros(nbytes // 4 + 1, device="cuda")
+    torch.cuda.synchronize()
+    names = _kernel_names(s, [lambda: V.vla_op_attn_decode(
+        q.data_ptr(), kv.data_ptr(), 1, H, hd, cap, env.data_ptr(), pos.data_ptr(), B, ctx, out[0].data_ptr(),
+        out[1].data_ptr(), ws.data_ptr(), nbytes, s.cuda_stream)])
+    names = [n for n in names if "attn_decode" in n]
+    assert len(names) == 1 and ("attn_decode_short_kernel" in names[0]) == short, names

@@ -678,3 +678,16 @@ def test_wide_residual_gemm_range():
     assert call(0, 256, 4096) == V.VLA_ERR_ARG
     assert call(384, 4096, 4096) == 0
     assert (h == 2.0).all() and V.vla_op_read_status() == (0, 0)
+
+
+@pytest.mark.parametrize("hd,per_sm,over,longest", [(64, 4, 1, 112), (64, 4, 0, 112), (64, 4, 1, 113), (64, 5, 1, 160),
+                                                    (128, 7, 1, 128), (128, 7, 0, 128), (128, 7, 1, 9)])
+def test_decode_attention_of_many_pairs_over_short_contexts(hd, per_sm, over, longest):
+    # around the sizes from which a kernel of its own takes such calls
+    H = 8
+    B = (per_sm * V.vla_op_num_sms() + H - 1) // H + over
+    ctx = [longest] + [min(longest, (1, 2, 3, 5, 8, 9, 16, 17, 31, 32, 33, 64, 65, 100, 127, 160)[b % 16])
+                       for b in range(B - 1)]
+    cap = (longest + 15) // 16 * 16
+    test_decode_attention_matches_fp64(B, H, hd, cap, ctx)
+    test_decode_attention_res_matches_fp64(B, H, hd, cap, ctx)
