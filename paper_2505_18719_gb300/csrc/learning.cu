@@ -55,6 +55,11 @@ __global__ void __launch_bounds__(256) value_head_kernel(const float* h, int ldh
 // one-thread-per-env loop over global memory paid a load's latency every step: 128 steps x 256 envs
 // took 75.5 us with cold caches (23.8 us a call back to back), now 5.2 (about 9, the caller's share
 // included); 1024 x 4096 took 552 us, now 23.1.
+// Blocks of `size` that hold n >= 1 items (no sum that overflows at the largest n).
+__host__ __device__ constexpr int blocks_of(int n, int size) { return (n - 1) / size + 1; }
+static_assert(blocks_of(1, 64) == 1 && blocks_of(64, 64) == 1 && blocks_of(65, 64) == 2 && blocks_of(0x7fffffff, 64) == 1 << 25,
+              "blocks");
+
 constexpr int kGaeT = 64;                 // steps per chunk
 constexpr int kGaeWarps = 8;
 constexpr int kGaeRows = kGaeT / kGaeWarps;  // steps of a chunk per warp
@@ -69,7 +74,7 @@ __global__ void __launch_bounds__(32 * kGaeWarps) gae_kernel(const float* r, con
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int b = blockIdx.x * 32 + lane;
   const bool ok = b < B;
-  const int n_chunks = (M + kGaeT - 1) / kGaeT;
+  const int n_chunks = blocks_of(M, kGaeT);
   float xr[kGaeRows], xv[kGaeRows], xn[kGaeRows], xd[kGaeRows];
   // steps of chunk k: t0 + 0 .. kGaeT-1; this warp's are t0 + warp * kGaeRows + i
   auto load = [&](int k) {
@@ -156,7 +161,7 @@ __global__ void __launch_bounds__(kPpoTile) ppo_clip_kernel(const float* lp_new,
   pdl_wait();
   const int n_cta = static_cast<int>(gridDim.x), rank = static_cast<int>(blockIdx.x);
   const int tid = threadIdx.x;
-  const int tiles = (N + kPpoTile - 1) / kPpoTile;
+  const int tiles = blocks_of(N, kPpoTile);
   const int plane = kPpoTile * A;
   auto stage_load = [&](int tile, int st) {
     if (tile < tiles) {
@@ -178,8 +183,7 @@ __global__ void __launch_bounds__(kPpoTile) ppo_clip_kernel(const float* lp_new,
   };
   float acc = 0.f, clipped = 0.f;
   auto adv_of = [&](int tile) {
-    const int n = tile * kPpoTile + tid;
-    return tile < tiles && n < N ? adv[n] : 0.f;
+    return tile < tiles && tile * kPpoTile + tid < N ? adv[tile * kPpoTile + tid] : 0.f;
   };
   float a = adv_of(rank);
   if (staged)
@@ -283,10 +287,13 @@ int ppo_clip_launch(const float* lp_new, const float* lp_old, const float* adv, 
                     float* objective, float* ratio, float* clip_frac, cudaStream_t s) {
   if (N <= 0) return VLA_ERR_ARG;
   // one tile per CTA up to 16 CTAs (the non-portable cluster maximum) or what the device can place: the
-  // CTAs take the tiles in turn at any number; the staging needs 16-byte aligned log-probs
-  const int tiles = (N + kPpoTile - 1) / kPpoTile;
-  const int want = tiles <= 1 ? 1 : tiles <= 2 ? 2 : tiles <= 4 ? 4 : tiles <= 8 ? 8 : 16;
-  const bool staged = A <= kPpoMaxA && !(reinterpret_cast<uintptr_t>(lp_new) & 15) &&
+  // CTAs take the tiles in turn at any number; the staging needs 16-byte aligned log-probs.  Two tiles of
+  // few tokens are read in place by one CTA: 1024 x 7 takes 2.7 us back to back and 12.4 alone, on two CTAs
+  // 3.1 to 3.4 and 13.2 (1024 x 8: 4.0 and 14.0, on two CTAs 3.3 and 13.5).
+  const int tiles = blocks_of(N, kPpoTile);
+  const bool small = tiles <= 2 && A < 8;
+  const int want = tiles <= 1 || small ? 1 : tiles <= 2 ? 2 : tiles <= 4 ? 4 : tiles <= 8 ? 8 : 16;
+  const bool staged = !small && A <= kPpoMaxA && !(reinterpret_cast<uintptr_t>(lp_new) & 15) &&
                       !(reinterpret_cast<uintptr_t>(lp_old) & 15);
   static std::atomic<uint64_t> smem_done[2] = {}, cluster_done[2] = {};
   static std::atomic<int> cluster_size[2][64] = {};

@@ -91,6 +91,12 @@ def test_ppo_clip_tile_edges(N, A, offset):
     assert abs(cf.item() - o_cf) <= (near + 0.5) / N
 
 
+# the objective's step from one CTA that reads in place to clusters that stage
+@pytest.mark.parametrize("N,A", [(1, 1), (512, 7), (512, 8), (1024, 7), (1024, 1), (1024, 8), (1025, 7)])
+def test_ppo_clip_small_calls(N, A):
+    test_ppo_clip_tile_edges(N, A, 0)
+
+
 # a device (a partition, a client with few SMs) that cannot place clusters of 16 CTAs: fewer CTAs take the tiles
 @pytest.mark.parametrize("most", [8, 4, 2, 1])
 def test_ppo_clip_on_smaller_clusters(most):
