@@ -112,7 +112,7 @@ int vla_op_read_status(void* cuda_stream, uint32_t* status_out);
  * sampler of vla_decode_actions with uniforms (f32 [B, 256]) at `temperature`.
  * forced (int32 [B] bin indices 0..255, or NULL) selects whose log-prob is returned.
  * Outputs (device, [B]): bins_out int32 (sampled bin k), logprobs_out f32, actions_out f32,
- * logits_out f32 [B, 256] (required: the logits are formed there before sampling).  status:
+ * logits_out f32 [B, 256] (required).  status:
  * device uint32 word, OR-ed with VLA_STATUS_* bits.  h must be 16-byte aligned with ldh a
  * multiple of 4, head_rows 16-byte aligned, final_norm 8-byte aligned, d a multiple of 8 and
  * at most 6400 (else VLA_ERR_UNSUPPORTED). */

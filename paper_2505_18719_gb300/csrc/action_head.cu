@@ -284,7 +284,6 @@ __global__ void __launch_bounds__(kHeadThreads, RPC) head_kernel(const HeadArgs 
       if (a.tokens_out) a.tokens_out[out_i] = a.token_base + ks;
       if (a.bins_out) a.bins_out[out_i] = ks;
       if (a.act_out) a.act_out[out_i] = static_cast<float>(2 * ks + 1 - 256) * (1.0f / 256.0f);
-      if (a.fed_out) a.fed_out[out_i] = fed;
       // the env's last token stays pending (a scored one as given, its range is checked when it is fed)
       if (a.pending_out && out_i == b * a.A + a.A - 1) a.pending_out[b] = FIRST ? a.forced[out_i] : fed;
       fed_s = fed;
@@ -303,7 +302,8 @@ __global__ void __launch_bounds__(kHeadThreads, RPC) head_kernel(const HeadArgs 
 int action_head_launch(const HeadArgs& a, cudaStream_t s) {
   if (a.B <= 0) return VLA_OK;
   if (a.d % 8 || a.ldh % 4 || (reinterpret_cast<uintptr_t>(a.h) & 15) ||
-      (reinterpret_cast<uintptr_t>(a.h_first) & 15) || (reinterpret_cast<uintptr_t>(a.head_rows) & 15) || (reinterpret_cast<uintptr_t>(a.final_norm) & 7))
+      (reinterpret_cast<uintptr_t>(a.h_first) & 15) || (reinterpret_cast<uintptr_t>(a.head_rows) & 15) ||
+      (reinterpret_cast<uintptr_t>(a.final_norm) & 7))
     return VLA_ERR_UNSUPPORTED;
   if (a.d > kHeadMaxD) return VLA_ERR_UNSUPPORTED;
   const int R = a.B * a.n_pos;

@@ -159,7 +159,6 @@ struct vla_handle {
   RowInfo* rows = nullptr;
   AttnTile* tiles = nullptr;
   int* sidx = nullptr;
-  int* fed = nullptr;
   int* pending = nullptr;
   uint32_t* status = nullptr;
   float* part_o = nullptr;
@@ -640,7 +639,6 @@ int vla_create(const vla_config* cfg, const vla_weights* w, void* cuda_stream, v
             alloc(reinterpret_cast<void**>(&h->rows), T * sizeof(RowInfo)) &&
             alloc(reinterpret_cast<void**>(&h->tiles), static_cast<size_t>(h->max_tiles) * sizeof(AttnTile)) &&
             alloc(reinterpret_cast<void**>(&h->sidx), static_cast<size_t>(B) * sizeof(int)) &&
-            alloc(reinterpret_cast<void**>(&h->fed), static_cast<size_t>(B) * A * sizeof(int)) &&
             alloc(reinterpret_cast<void**>(&h->pending), static_cast<size_t>(B) * sizeof(int)) &&
             alloc(reinterpret_cast<void**>(&h->status), sizeof(uint32_t)) &&
             alloc(reinterpret_cast<void**>(&h->part_o), attn_slots * c.head_dim * sizeof(float)) &&
@@ -810,7 +808,8 @@ int vla_decode_actions(vla_handle* h, const float* uniforms, float temperature, 
   const vla_config& c = h->cfg;
   const int B = h->active_batch, A = c.action_dim, d = c.d_model;
 
-  // decode rows of steps 1..A-1: env b at position len_prefill[b] + i - 1, fed token of step i-1
+  // decode rows of steps 1..A-1: env b at position len_prefill[b] + i - 1 (its row is written by the head of the
+  // step before: only env and position are read)
   int slot;
   RowInfo* rows = static_cast<RowInfo*>(stage_slot(h, &slot));
   for (int i = 1; i < A; ++i)
@@ -840,7 +839,6 @@ int vla_decode_actions(vla_handle* h, const float* uniforms, float temperature, 
   ha.lp_out = logprobs_out;
   ha.act_out = actions_out;
   ha.logits_out = logits_out;
-  ha.fed_out = h->fed;
   ha.pending_out = h->pending;  // the last token stays pending
   ha.status = h->status;
 
@@ -1044,7 +1042,7 @@ void vla_destroy(vla_handle* h) {
   DeviceGuard dev_guard(h->dev);  // best effort: the handle is freed whatever happens
   cudaStreamSynchronize(h->stream);
   void* bufs[] = {h->kv, h->kv_res, h->h, h->y, h->q, h->ao, h->u, h->ws, h->h_last, h->head_entropy, h->q_last, h->ss_part, h->last_rows, h->rope,
-                  h->rows, h->tiles, h->sidx, h->fed, h->pending, h->status, h->part_o,
+                  h->rows, h->tiles, h->sidx, h->pending, h->status, h->part_o,
                   h->part_ml, h->attn_tickets, h->w16, h->w16_range};
   for (void* p : bufs)
     if (p) cudaFree(p);

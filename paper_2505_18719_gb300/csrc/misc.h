@@ -96,7 +96,6 @@ struct HeadArgs {
   float* lp_out = nullptr;          // [B, A]
   float* act_out = nullptr;         // [B, A]
   float* logits_out = nullptr;      // [B, A, 256]
-  int* fed_out = nullptr;           // [B, A] token fed to the next step (forced or sampled)
   float* entropy_out = nullptr;     // [B, A] entropy of each token's bin distribution
   int* pending_out = nullptr;       // [B] each env's token of action A - 1
   uint32_t* status = nullptr;
