@@ -70,8 +70,8 @@ int vla_op_gemm_decode_f16(const void* A, const void* A_lo, int lda, const void*
  * clusters.  With norm_w (bf16 [N]) the RMSNorm that follows is left to the consumer: y_hi / y_lo
  * (fp16 [M, N], y_lo may be NULL) get the updated row times norm_w, not normalised, and ss_out
  * (f32 [N / 128, M]) the sums of squares of the updated row over each 128 columns.
- * VLA_ERR_UNSUPPORTED for calls that the engine gives to the tile GEMMs instead: M outside 321 .. 432,
- * N no multiple of 128 or with more tiles than clusters of four fit on the GPU at once, K < 4096, or
+ * VLA_ERR_UNSUPPORTED for calls that the engine gives to the tile GEMMs instead: M outside 257 .. 432,
+ * N no multiple of 128 or with more tiles than clusters of four fit on the GPU at once, K < 3072, or
  * buffers off their alignment (16 bytes; norm_w and the outputs 8). */
 int vla_op_gemm_resid_f16(const void* A, int lda, const void* W, int ldw, float* resid, int ldr, int M, int N,
                           int K, const void* norm_w, void* y_hi, void* y_lo, float* ss_out, void* cuda_stream);

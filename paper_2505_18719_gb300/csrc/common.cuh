@@ -303,6 +303,25 @@ inline cudaError_t allow_wide_clusters(Kern kern, std::atomic<uint64_t>& done) {
 extern std::atomic<int> g_max_cluster;
 constexpr int kDefaultMaxCluster = 16;
 
+// Clusters of c CTAs of `kern` that the current device holds at once; 0 where it refuses the size.
+template <typename Kern>
+inline int max_active_clusters(Kern kern, dim3 block, size_t smem, int c) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(static_cast<unsigned>(c));
+  cfg.blockDim = block;
+  cfg.dynamicSmemBytes = smem;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeClusterDimension;
+  attr[0].val.clusterDim.x = static_cast<unsigned>(c);
+  attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  int n = 0;
+  if (cudaOccupancyMaxActiveClusters(&n, kern, &cfg) == cudaSuccess && n > 0) return n;
+  cudaGetLastError();
+  return 0;
+}
+
 // The most CTAs (a power of two, at most `most`) of `kern` that the current device can place as one cluster:
 // a partition of a GPU, or a client with a limit on its SMs, may not hold the non-portable sizes.  Asked once
 // per (kernel, device); `known` holds the answer per device index < 64, 0 = not asked yet.
@@ -312,21 +331,8 @@ inline cudaError_t max_cluster_size(Kern kern, dim3 block, size_t smem, int most
   if (const cudaError_t e = cudaGetDevice(&dev)) return e;
   int c = dev >= 0 && dev < 64 ? known[dev].load(std::memory_order_acquire) : 0;
   if (!c) {
-    for (c = most; c > 1; c /= 2) {
-      cudaLaunchConfig_t cfg = {};
-      cfg.gridDim = dim3(static_cast<unsigned>(c));
-      cfg.blockDim = block;
-      cfg.dynamicSmemBytes = smem;
-      cudaLaunchAttribute attr[1];
-      attr[0].id = cudaLaunchAttributeClusterDimension;
-      attr[0].val.clusterDim.x = static_cast<unsigned>(c);
-      attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
-      cfg.attrs = attr;
-      cfg.numAttrs = 1;
-      int n = 0;
-      if (cudaOccupancyMaxActiveClusters(&n, kern, &cfg) == cudaSuccess && n > 0) break;
-      cudaGetLastError();  // a size that the device refuses
-    }
+    for (c = most; c > 1; c /= 2)
+      if (max_active_clusters(kern, block, smem, c) > 0) break;
     if (dev >= 0 && dev < 64) known[dev].store(c, std::memory_order_release);
   }
   const int limit = g_max_cluster.load(std::memory_order_relaxed);

@@ -316,7 +316,7 @@ int run_gemm(vla_handle* h, int cls, const bf16* A, size_t a_plane, int lda, con
     g.epi.row_d = K;
     g.epi.row_eps = h->cfg.rms_eps;
   }
-  const bool wide = !stream_k && g.splits == 1 && g.block_n == 128 && gemm_wide_ok(g, h->num_sms);
+  const bool wide = !stream_k && g.splits == 1 && g.block_n == 128 && gemm_wide_ok(g);
   if (h->ev_used.size() > 8192) prof_harvest(h);
   int ev = prof_begin(h, cls);
   GemmCost cost{0, 0};
@@ -1240,7 +1240,7 @@ int vla_op_gemm_resid_f16(const void* A, int lda, const void* W, int ldw, float*
   g.epi.ldn = N;
   g.epi.ss_out = norm_w ? ss_out : nullptr;
   g.epi.fp16 = true;
-  if (!gemm_wide_ok(g, query_num_sms()))
+  if (!gemm_wide_ok(g))
     return set_err(nullptr, VLA_ERR_UNSUPPORTED, "vla_op_gemm_resid_f16: sizes or alignment outside the kernel's range");
   if (const int rs = op_status_word(&g.epi.status)) return rs;
   return gemm_wide_launch(g, static_cast<cudaStream_t>(cuda_stream), nullptr);

@@ -101,7 +101,7 @@ bool make_tensor_map_2d(CUtensorMap* m, const void* ptr, int64_t rows, int64_t c
 
 // Residual GEMM of a few hundred rows with K split over clusters, for calls that would run as unsplit
 // 128-column tiles: same arguments and results as gemm_launch there.
-bool gemm_wide_ok(const GemmArgs& a, int num_sms);
+bool gemm_wide_ok(const GemmArgs& a);
 int gemm_wide_launch(const GemmArgs& a, cudaStream_t stream, GemmCost* cost);
 
 // Failure injection (test hook): in the next launch of the single-CTA tile GEMM, the cluster GEMM or the

@@ -1766,13 +1766,17 @@ __global__ void __launch_bounds__(kThreads, 2)
 // each CTA stores its fp32 partial rows from TMEM into the shared memory of the CTA that finishes them
 // (over the stages, once every CTA of the cluster is done with its own), which adds them in rank order and
 // applies the residual add and the deferred RMSNorm's outputs.
-// 384 rows, 4096 x 11008: 40 us against 70 of the tile GEMM; 4096 x 4096: 28 against 28 alone with cold
-// caches, but 9 us less in the pass, where its first weights are requested early (score pass of 64 envs, two
-// 7B layers: 645 us, 604 with down here, 586 with both).  A shorter K leaves less than the exchange costs
-// (about 15 us).  Below kWideMin rows the tiles stay: a prefill of one env (289 rows, 1661 against 1621 us a
-// turn of two 7B layers) would gain little, and its rows would round otherwise than in a larger batch's.
-constexpr int kWideMin = 320;
-constexpr int kWideMinK = 4096;
+// It takes the calls that would run as unsplit 128-column tiles from 257 rows on (up to 256 two row tiles are
+// few enough for the tile GEMM to split K), as long as all its clusters fit at once.  Score pass of two
+// layers over 40 positions, us, o and down on the tile GEMM against this one:
+//   7B, 258 / 318 / 324 / 384 / 432 rows         518 / 524 / 525 / 533 / 636   442 / 453 / 460 / 477 / 586
+//   d 4608 (36 clusters), 324 / 384 / 432 rows   630 / 641 / 704               560 / 575 / 645
+//   d 3584, 258 / 432 rows                       494 / 567                     410 / 510
+//   d 3072 / 2048, 432 rows                      451 / 306                     399 / 308 (K = 2048: 310)
+// and a prefill of one env, 289 rows: 423 against 384.  Error against 64 bits at 4096 x 11008: 3.0e-6 against
+// 1.2e-5 (K in four sums).
+constexpr int kWideMin = 256;
+constexpr int kWideMinK = 3072;
 constexpr int kWideRows = 432;      // the exchange of (rows + 3) x 128 fp32 fits shared memory
 constexpr int kWideC = 4;
 constexpr int kWideThreads = 320;   // producer, MMA issuer, eight warps that move and finish the sums
@@ -2406,9 +2410,22 @@ size_t gemv_workspace_bytes(int M, int N, int K, int num_sms) {
   return stream_plan(M, N, K, num_sms).ws_bytes;
 }
 
-bool gemm_wide_ok(const GemmArgs& a, int num_sms) {
+constexpr int kWideSmemMax = 227 * 1024;
+// Clusters of gemm_wide_kernel that the current device holds at once (36 on 152 SMs), asked once per device.
+static int wide_clusters() {
+  static std::atomic<uint64_t> attr_done{0};
+  static std::atomic<int> known[64] = {};  // the answer + 1
+  int dev = 0, n = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess || set_smem_limit(gemm_wide_kernel, kWideSmemMax, attr_done) != cudaSuccess) return 0;
+  if (dev >= 0 && dev < 64 && (n = known[dev].load(std::memory_order_acquire))) return n - 1;
+  n = max_active_clusters(gemm_wide_kernel, dim3(kWideThreads), kWideSmemMax, kWideC);
+  if (dev >= 0 && dev < 64) known[dev].store(n + 1, std::memory_order_release);
+  return n;
+}
+
+bool gemm_wide_ok(const GemmArgs& a) {
   return a.epi.kind == EPI_RESID && !a.A_lo && a.M > kWideMin && a.M <= kWideRows && a.N % 128 == 0 &&
-         a.N / 128 * kWideC <= num_sms * 17 / 20 && a.K >= kWideMinK && a.lda % 8 == 0 && a.ldb % 8 == 0 && a.epi.ldr % 4 == 0 &&
+         a.K >= kWideMinK && a.N / 128 <= wide_clusters() && a.lda % 8 == 0 && a.ldb % 8 == 0 && a.epi.ldr % 4 == 0 &&
          !((reinterpret_cast<uintptr_t>(a.A) | reinterpret_cast<uintptr_t>(a.B) | reinterpret_cast<uintptr_t>(a.epi.resid)) & 15) &&
          (!a.epi.norm_w || (a.epi.ss_out && a.epi.norm_hi && a.epi.ldn % 4 == 0 &&
                             !((reinterpret_cast<uintptr_t>(a.epi.norm_w) | reinterpret_cast<uintptr_t>(a.epi.norm_hi) |
@@ -2429,9 +2446,8 @@ int gemm_wide_launch(const GemmArgs& a, cudaStream_t stream, GemmCost* cost) {
   const int stage = 128 * BK * 2 + 2 * p.nb * BK * 2;
   const int recv = (a.M + kWideC - 1) / kWideC * kWideC * 128 * 4;
   const int smem = std::max(kWideStages * stage, recv) + 2048;
-  constexpr int smem_max = 227 * 1024;
   static std::atomic<uint64_t> attr_done{0};
-  VLA_CUDA_TRY(set_smem_limit(gemm_wide_kernel, smem_max, attr_done));
+  VLA_CUDA_TRY(set_smem_limit(gemm_wide_kernel, kWideSmemMax, attr_done));
   VLA_CUDA_TRY(launch_cluster_at(a.start, gemm_wide_kernel, dim3(a.N / 128 * kWideC), dim3(kWideThreads), smem, stream,
                                  kWideC, mw, mx, p));
   note_launch();

@@ -192,9 +192,9 @@ def test_gains_embeddings_and_lm_head_are_read_at_every_call(action_dim):
     pol.close()
 
 
-@pytest.mark.parametrize("B", [53, 54, 72, 73])
+@pytest.mark.parametrize("B", [42, 43, 72, 73])
 def test_score_pass_runs_o_and_down_on_the_wide_gemm(B):
-    # 324 to 432 score rows; 318 and 438 stay on the tile GEMMs
+    # 258 to 432 score rows; 252 and 438 stay on the tile GEMMs
     sh = I.ModelShape("tiny", 2, 4096, 32, 128, 4616)
     s = torch.cuda.Stream()
     pol = V.Policy(sh, P.weights_to_device(I.make_weights(sh, 11)), B, 32, B * 2, stream=s)
@@ -205,7 +205,7 @@ def test_score_pass_runs_o_and_down_on_the_wide_gemm(B):
     pol.prefill(None, ids, [2] * B)
     names = _kernel_names(s, [lambda: V.vla_score_actions(pol.h, tok.data_ptr(), 1.0, lp.data_ptr())])
     gemms = [k for n in names for k in GEMMS if k in n]  # q|k|v, o, gate|up, down of each layer
-    o_down = "gemm_wide_kernel" if 54 <= B <= 72 else "gemm_tc_kernel"
+    o_down = "gemm_wide_kernel" if 43 <= B <= 72 else "gemm_tc_kernel"
     assert gemms == ["gemm_tc_kernel", o_down] * (2 * sh.n_layers)
     pol.close()
 

@@ -630,7 +630,9 @@ def test_attn_rows8_matches_fp64(hd):
 
 
 @pytest.mark.parametrize("M,N,K", [
-    (321, 128, 4096),      # the fewest rows: an odd split over four ranks, 31 rows of padding
+    (257, 128, 4096),      # the fewest rows: an odd split over four ranks, 31 rows of padding
+    (289, 4608, 4608),     # the most weight tiles that fit at once on 152 SMs
+    (321, 384, 3072),      # the shortest K
     (322, 640, 4104),      # a K tail
     (384, 4096, 4096),     # o of the 7B shape, 64 envs
     (384, 4096, 11008),    # down
@@ -668,11 +670,11 @@ def test_wide_residual_gemm_matches_fp64(M, N, K):
 def test_wide_residual_gemm_range():
     # the sizes that the engine leaves to the tile GEMMs are refused, nothing runs
     A = torch.zeros(433, 4096, dtype=torch.float16, device="cuda")
-    W = torch.zeros(4352, 4096, dtype=torch.float16, device="cuda")
-    h = torch.full((433, 4352), 2.0, device="cuda")
+    W = torch.zeros(4864, 4096, dtype=torch.float16, device="cuda")
+    h = torch.full((433, 4864), 2.0, device="cuda")
     call = lambda M, N, K, off=0: V.vla_op_gemm_resid_f16(A.data_ptr() + off, 4096, W.data_ptr(), 4096,  # noqa: E731
-                                                          h.data_ptr(), 4352, M, N, K)
-    for M, N, K in ((320, 256, 4096), (433, 256, 4096), (384, 192, 4096), (384, 4224, 4096), (384, 256, 4088)):
+                                                          h.data_ptr(), 4864, M, N, K)
+    for M, N, K in ((256, 256, 4096), (433, 256, 4096), (384, 192, 4096), (384, 4864, 4096), (384, 256, 3064)):
         assert call(M, N, K) == V.VLA_ERR_UNSUPPORTED, (M, N, K)
     assert call(384, 256, 4096, off=8) == V.VLA_ERR_UNSUPPORTED
     assert call(0, 256, 4096) == V.VLA_ERR_ARG
