@@ -230,8 +230,15 @@ CASES = {
     "gemv_decode_o": (64, 4096, 4096, 0, 0, True),
     "gemv_decode_gate_up": (64, 22016, 4096, 0, 0, True),
     "gemv_decode_down": (64, 4096, 11008, 0, 0, True),
+    "gemv_decode_qkv_b16": (16, 12288, 4096, 0, 0, True),      # up to 32 rows: the cluster kernel
+    "gemv_decode_o_b16": (16, 4096, 4096, 0, 0, True),
     "attn_decode": None,                                       # see run_attn_case
     "attn_decode_res": None,
+    "attn_decode_short_res": None,                             # 256 envs x 32 heads over 8 to 24 positions
+    "action_head": None,                                       # see run_head_case
+    # residual GEMM of the score pass (64 envs x 6 rows) with K split over clusters, fp16
+    "wide_score_o": (384, 4096, 4096, 0, 0, False),
+    "wide_score_down": (384, 4096, 11008, 0, 0, False),
     "learning": None,                                          # see run_learning_case
     "attn_chunk": None,                                        # see run_attn_chunk_case
     "attn_score": None,                                        # 6 rows per env after the prefix
@@ -282,7 +289,8 @@ CASES.update({k + "_f16": v for k, v in list(CASES.items()) if v is not None})
 
 def run_attn_case(args):
     """Decode attention for 64 envs x 32 heads at ~290 cached positions (one layer); attn_decode_res
-    reads the fp16 parts and their 4-bit residual codes (the engine's form)."""
+    reads the fp16 parts and their 4-bit residual codes (the engine's form); attn_decode_short_res
+    the same for 256 envs over 8 to 24 positions."""
     import torch
     import __graft_entry__
     __graft_entry__.build()
@@ -291,11 +299,14 @@ def run_attn_case(args):
     B, H, hd = 64, 32, 128
     scale = max(1, args.attn_ctx_scale)
     cap = 320 * scale
+    short = args.case == "attn_decode_short_res"
+    if short:
+        B, cap = 256, 32
     kv = I.normal_bf16((B, 2, H, cap, hd), 5, 1, 1.0).cuda().half()
     res = args.case.endswith("_res")
     codes = I.randint_i32((B * 2 * H * cap * hd // 2,), 5, 4, 0, 256).to(torch.uint8).cuda() if res else None
     q = I.normal_bf16((B, H, hd), 5, 2, 1.0).cuda().float()
-    ctx = I.randint_i32((B,), 5, 3, 273, 311) * scale
+    ctx = I.randint_i32((B,), 5, 3, 8, 25) if short else I.randint_i32((B,), 5, 3, 273, 311) * scale
     env = torch.arange(B, dtype=torch.int32, device="cuda")
     pos = (ctx - 1).cuda()
     max_ctx = int(ctx.max())
@@ -436,6 +447,34 @@ def run_learning_case(args):
     return 0
 
 
+def run_head_case(args):
+    """The action head on 64 rows of the 7B width."""
+    import torch
+    import __graft_entry__
+    __graft_entry__.build()
+    from paper_2505_18719_gb300 import inputs as I
+    from paper_2505_18719_gb300 import vla as V
+    B, d = 64, 4096
+    h = I.normal_bf16((B, d), 6, 1, 1.0).float().cuda()
+    gain = torch.ones(d, dtype=torch.bfloat16, device="cuda")
+    rows = I.normal_bf16((256, d), 6, 2, 0.02).cuda()
+    u = I.uniform_f32((B, 256), 6, 3).cuda()
+    bins, status = (torch.zeros(n, dtype=torch.int32, device="cuda") for n in (B, 1))
+    lp, act = (torch.empty(B, device="cuda") for _ in range(2))
+    z = torch.empty(B, 256, device="cuda")
+    e0, e1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+    for i in range(args.warmup + args.steps):
+        if i == args.warmup:
+            e0.record()
+        assert V.vla_op_action_head(h.data_ptr(), d, B, d, gain.data_ptr(), rows.data_ptr(), 1e-6, u.data_ptr(), 1.0, 0,
+                                    bins.data_ptr(), lp.data_ptr(), act.data_ptr(), z.data_ptr(), status.data_ptr()) == 0
+    e1.record()
+    torch.cuda.synchronize()
+    print(json.dumps({"case": args.case, "rows": B, "d": d, "us": e0.elapsed_time(e1) / args.steps * 1e3,
+                      "bytes": 2.0 * 256 * d + B * (4.0 * d + 2048)}))
+    return 0
+
+
 def run_case(args):
     """Time one GEMM shape through the GEMM op entry points (CUDA events, device-resident
     operands); bf16 operands, or fp16 for the NAME_f16 cases."""
@@ -444,14 +483,16 @@ def run_case(args):
     __graft_entry__.build()
     from paper_2505_18719_gb300 import inputs as I
     from paper_2505_18719_gb300 import vla as V
-    if args.case in ("attn_decode", "attn_decode_res"):
+    if args.case.startswith("attn_decode"):
         return run_attn_case(args)
+    if args.case == "action_head":
+        return run_head_case(args)
     if args.case == "learning":
         return run_learning_case(args)
     if args.case.startswith(("attn_chunk", "attn_score")):
         return run_attn_chunk_case(args)
     M, N, K, bn, splits, split_a = CASES[args.case]
-    fp16 = args.case.endswith("_f16")
+    fp16 = args.case.endswith("_f16") or args.case.startswith("wide")
     A = I.normal_bf16((M, K), 1, 1, 1.0).cuda()
     A_lo = I.normal_bf16((M, K), 1, 2, 2.0 ** -9).cuda()
     W = I.normal_bf16((N, K), 1, 3, 0.02).cuda()
@@ -475,6 +516,13 @@ def run_case(args):
         def launch():
             rc = op_decode(A.data_ptr(), A_lo.data_ptr(), K, W.data_ptr(), K, C.data_ptr(), N,
                            M, N, K, ws.data_ptr(), nbytes, stream.cuda_stream)
+            assert rc == 0, V.vla_last_error()
+    elif args.case.startswith("wide"):
+        C.zero_()
+
+        def launch():
+            rc = V.vla_op_gemm_resid_f16(A.data_ptr(), K, W.data_ptr(), K, C.data_ptr(), N, M, N, K,
+                                         stream=stream.cuda_stream)
             assert rc == 0, V.vla_last_error()
     else:
         ws = torch.empty(max(1, splits * M * N), dtype=torch.float32, device="cuda")
