@@ -1422,8 +1422,8 @@ __device__ __forceinline__ void store_kv4(f16* dst, uint8_t* res, float4 v) {
 }
 
 // Finishes this CTA's rows of the tile, kFinish items of four columns per thread at a time: what an
-// item reads from global memory is requested before `ready` (the wait for the partial sums; false, for
-// a warp as a whole, when they are not there: nothing is stored).
+// item reads from global memory is requested before `ready` (the wait for the partial sums; false when they
+// are not there: nothing is stored).
 constexpr int kFinish = 2;
 template <int TR, class Ready>
 __device__ __forceinline__ void gemv_finish(const ClusterParams& p, const TileSums<TR>& t, int tile, Ready ready,
@@ -1433,12 +1433,12 @@ __device__ __forceinline__ void gemv_finish(const ClusterParams& p, const TileSu
   if (e.kind == EPI_SWIGLU) {
     constexpr int V = TR / 8;  // float4s of a row's gate half
     const int F = p.N >> 1;
-    if (!ready()) return;
+    const bool there = ready();
     for (int k = tid; k < t.mn * V; k += kThreads) {
       const int i = k / V, j = (k - i * V) * 4;
       const float4 g = t.sum4(i, j), u = t.sum4(i, j + TR / 2);
       const int f = tile * (TR / 2) + j;
-      if (f >= F) continue;  // F % 4 == 0: four features are in or out together
+      if (f >= F || !there) continue;  // F % 4 == 0: four features are in or out together
       uint2 hi, lo;
       split_pack2(silu_f(g.x) * u.x, silu_f(g.y) * u.y, hi.x, lo.x, e.fp16, sat);
       split_pack2(silu_f(g.z) * u.z, silu_f(g.w) * u.w, hi.y, lo.y, e.fp16, sat);
@@ -1451,6 +1451,7 @@ __device__ __forceinline__ void gemv_finish(const ClusterParams& p, const TileSu
     // index i and of its partner i + hd / 2
     constexpr int V = TR / 8;
     const int d = e.d, hd = e.hd, half = hd >> 1;
+    bool there = false;
     for (int k0 = tid; k0 < t.mn * V || k0 == tid; k0 += kThreads * kFinish) {
       int env[kFinish], pos[kFinish];
       float4 cs[kFinish][2];  // (cos, sin) of i .. i + 3
@@ -1470,7 +1471,7 @@ __device__ __forceinline__ void gemv_finish(const ClusterParams& p, const TileSu
         cs[u][0] = c4[0];
         cs[u][1] = c4[1];
       }
-      if (k0 == tid && !ready()) return;
+      if (k0 == tid) there = ready();
 #pragma unroll
       for (int u = 0; u < kFinish; ++u) {
         const int k = k0 + u * kThreads;
@@ -1479,7 +1480,7 @@ __device__ __forceinline__ void gemv_finish(const ClusterParams& p, const TileSu
         const int lh = j / half, i = j - lh * half;
         float4 a = t.sum4(row, lh * hd + i), b = t.sum4(row, lh * hd + i + half);
         const int n = tile * TR + lh * hd;
-        if (n >= p.N) continue;
+        if (n >= p.N || !there) continue;
         const int sec = n / d, head = (n - sec * d) / hd;
         if (sec < 2) {
           const float4 c0 = cs[u][0], c1 = cs[u][1], x = a, y = b;
@@ -1508,6 +1509,7 @@ __device__ __forceinline__ void gemv_finish(const ClusterParams& p, const TileSu
     float* out = resid ? e.resid : e.out_f32;
     const int ld = resid ? e.ldr : e.ldo;
     const bool vec = !(ld & 3) && !(reinterpret_cast<uintptr_t>(out) & 15);
+    bool there = false;
     for (int k0 = tid; k0 < t.mn * V || k0 == tid; k0 += kThreads * kFinish) {
       float4 x[kFinish];
 #pragma unroll
@@ -1517,7 +1519,7 @@ __device__ __forceinline__ void gemv_finish(const ClusterParams& p, const TileSu
         if (resid && vec && k < t.mn * V && n + 4 <= p.N)
           x[u] = __ldcg(reinterpret_cast<const float4*>(out + static_cast<size_t>(t.m0 + k / V) * ld + n));
       }
-      if (k0 == tid && !ready()) return;
+      if (k0 == tid) there = ready();
 #pragma unroll
       for (int u = 0; u < kFinish; ++u) {
         const int k = k0 + u * kThreads;
@@ -1528,16 +1530,16 @@ __device__ __forceinline__ void gemv_finish(const ClusterParams& p, const TileSu
         float* o = out + static_cast<size_t>(t.m0 + i) * ld + n;
         if (vec && n + 4 <= p.N) {
           const float4 h = make_float4(x[u].x + a.x, x[u].y + a.y, x[u].z + a.z, x[u].w + a.w);
-          *reinterpret_cast<float4*>(o) = h;
+          if (there) *reinterpret_cast<float4*>(o) = h;
           if (e.ss_out) {  // a warp holds 128 columns of one row (N % 128 == 0): in or out together
             const float ss = warp_sum(h.x * h.x + h.y * h.y + h.z * h.z + h.w * h.w);
-            if ((tid & 31) == 0) e.ss_out[static_cast<size_t>(n / 128) * p.M + t.m0 + i] = ss;
+            if ((tid & 31) == 0 && there) e.ss_out[static_cast<size_t>(n / 128) * p.M + t.m0 + i] = ss;
           }
         } else {
           const float v[4] = {a.x, a.y, a.z, a.w};
 #pragma unroll
           for (int q = 0; q < 4; ++q)
-            if (n + q < p.N) o[q] = resid ? __ldcg(o + q) + v[q] : v[q];
+            if (there && n + q < p.N) o[q] = resid ? __ldcg(o + q) + v[q] : v[q];
         }
       }
     }
@@ -1745,7 +1747,7 @@ __global__ void __launch_bounds__(kThreads, 2)
   uint32_t sat = 0;
   gemv_finish<TR>(
       p, t, tile,
-      [&] { return __all_sync(0xffffffffu, wait_drain_reported(recv_bar, 0, status, limit)) != 0 && !gave_up; }, sat);
+      [&] { return wait_drain_reported(recv_bar, 0, status, limit) && !gave_up; }, sat);
   report_saturation(status, sat);
   __syncwarp();
   cluster_arrive();
