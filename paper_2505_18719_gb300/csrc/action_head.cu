@@ -10,8 +10,8 @@
 // Between decode steps the CTA that sampled a row's token also assembles the next step's row from it (its
 // embedding and first RMSNorm), a launch less per step.
 // Bound by the latency of its chain (rows, weights from L2, exchange, block reductions); two kernels,
-// with fp32 FMAs on one CTA per 32 bins x 8 rows before, took 22.5 + 4.3 us
-// at 64 rows x 4096 (cold caches), this one 12.0.
+// with fp32 FMAs on one CTA per 32 bins x 8 rows before, took 22.2 + 4.3 us at 64 rows x 4096 in a
+// decode's launch list (cold caches), this one 15.0 with the next step's rows; alone 12.4.
 #include "misc.h"
 #include "ptx.cuh"
 

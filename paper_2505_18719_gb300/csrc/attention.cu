@@ -2,15 +2,18 @@
 // self-attention; §3.3: the whole trajectory is one context, so every chunk attends to all
 // earlier turns).
 //
-//  * attn_chunk: query rows of one env at consecutive positions (a prefill chunk, or the
-//    6 teacher-forced action rows of the score pass) against keys 0..pos of that env.
-//    One CTA per (64-row tile, head); mma.sync tensor-core flash attention with fp32
-//    accumulation on fp16 K/V, the fp32 queries and the softmax weights each taken as an
-//    fp16 hi/lo pair; the output is written as the operand hi/lo pair the O-projection GEMM
-//    reads (fp16 for the engine, bf16 for the op entry points).
-//  * attn_decode: one query per env (the decode step) with the key range split across CTAs
-//    (flash-decoding); each CTA writes its partial (reference exponent, sum, unnormalised output)
-//    and the last CTA of the (env, head) to finish merges the splits in a fixed order.
+//  * attn_rows8 / attn_rows: chunks whose tiles all have at most 8 / 16 rows at consecutive positions of
+//    one env (the score pass's teacher-forced action rows) over the fp16 + residual cache, one CTA per
+//    (tile, head), mma.sync.  (Longer tiles, a prefill's, run on attn_tc.cu.)
+//  * attn_decode: one query per env (the decode step, and each env's last row in a prefill's last
+//    layer): full waves of whole (env, head) pairs on one CTA each, the pairs left over with their key
+//    range split across CTAs (flash-decoding), whose partials (reference exponent, sum, unnormalised
+//    output) the last one to finish merges in a fixed order.  attn_decode_short: many pairs over short
+//    contexts.
+//  * attn_chunk: tiles of 64 rows over a cache of fp16 alone, for the op entry point.
+//
+// The fp32 queries and the softmax weights are taken as two or three 16-bit parts; the output is the
+// operand hi/lo pair that the O-projection GEMM reads (fp16 for the engine, bf16 for the op entry points).
 //
 // Keys visible to a query at position p are positions 0..p (all of them are in the cache:
 // chunk rows write their K/V in the QKV epilogue before attention runs).
@@ -1352,7 +1355,9 @@ int attn_decode_launch(const float* q, bf16* out_hi, bf16* out_lo, const RowInfo
     int smem = kDecodeWarps * ring;
     // A grid within one wave is spread evenly: CTAs start as the previous kernel's leave, and the first
     // SMs to empty would take all they can hold (16 envs x 32 heads: 6 CTAs on some SMs, none on others,
-    // 31 us against 25), so each asks for its share of the shared memory.
+    // 31 us against 25), so each asks for its share of the shared memory.  The price is that nothing else
+    // fits beside them, the next projection's early CTAs among it: decode of 64 envs of 8 small layers takes
+    // 3294 us so and 3364 without.
     const int64_t per_sm = (grid + num_sms - 1) / num_sms;
     if (per_sm < decode_ctas_per_sm(hd)) smem = std::max(smem, static_cast<int>(kSmemPerSm / per_sm - kDecodeStatic) / 128 * 128);
     if (const cudaError_t e = set_smem_limit(kern, kSmemPerSm - kDecodeStatic, attr_done)) return e;

@@ -1762,7 +1762,7 @@ __global__ void __launch_bounds__(kThreads, 2)
 
 // ----------------------------------------------------------------------------- residual GEMM, wide
 // o and down of a few hundred rows (the score pass: 6 rows of each env).  An SM takes in about 85 GB/s from
-// L2, which bounds 128 x 128 tiles (32 KB of operands per 2 MFLOP) at a quarter of the tensor rate, on the
+// L2 (5.6 MB of down's operands in 66 us), which bounds 128 x 128 tiles (32 KB of operands per 2 MFLOP) at a quarter of the tensor rate, on the
 // 96 of 152 SMs that 384 x 4096 outputs give such tiles.  Here a tile is 128 weight rows by ALL rows of the
 // call (64 KB per 6.3 MFLOP), the weights as the MMA's M like in the decode GEMMs, and a cluster splits K:
 // each CTA stores its fp32 partial rows from TMEM into the shared memory of the CTA that finishes them
@@ -2164,7 +2164,8 @@ GemmCost gemm_cost(const GemmArgs& a) {
   return c;
 }
 
-// Stream-K plan of the weight-streaming GEMM.
+// Stream-K plan of the weight-streaming GEMM (up to 32 rows, where the cluster kernel runs, only the workspace
+// size that the op asks its callers for).
 struct StreamPlan {
   int bnx, grid, tiles, kbt, per_cta, max_seg;
   size_t ws_bytes;
@@ -2203,6 +2204,9 @@ int launch_stream(const CUtensorMap& w, const CUtensorMap& x, const CUtensorMap&
 // Shared memory of a cluster-kernel CTA for stages, then partial tiles: two CTAs per SM (at most 113 KB
 // each with the 2 KB of alignment and barriers and the runtime's 1 KB).
 constexpr int kClusterData = 112640;
+// Both forms in decodes of 17 / 24 / 32 envs, us, stream-K (64-row tiles) against this one: two 7B layers
+// 1619 / 1719 / 1877 against 1517 / 1606 / 1769; 8 small layers 2723 / 2846 / 2835 against 2128 / 2234 / 2346.  At 64
+// rows 2302 against 2319; this form was not built for sizes between.
 constexpr int kClusterRows = 32;
 
 // Tile rows, cluster size and grid of the cluster kernel.

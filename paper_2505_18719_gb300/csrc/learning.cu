@@ -47,19 +47,19 @@ __global__ void __launch_bounds__(256) value_head_kernel(const float* h, int ldh
   }
 }
 
+// Blocks of `size` that hold n >= 1 items (no sum that overflows at the largest n).
+__host__ __device__ constexpr int blocks_of(int n, int size) { return (n - 1) / size + 1; }
+static_assert(blocks_of(1, 64) == 1 && blocks_of(64, 64) == 1 && blocks_of(65, 64) == 2 && blocks_of(0x7fffffff, 64) == 1 << 25,
+              "blocks");
+
 // GAE: A_t = delta_t + c_t A_{t+1} with c_t = gamma lam (1 - done_t), t = M-1 .. 0, for 32 envs per
 // CTA (lane = env).  The recurrence is a chain of M dependent FMAs per env, so everything else is
 // taken off it: all 8 warps load a chunk of 64 steps ahead (coalesced over the envs) and put (delta_t,
 // c_t) into shared memory, warp 0 walks the chunk (one FMA a step, same order and rounding as a plain
 // loop), and all warps write A and A + V out while the next chunk's loads are in flight.  The
 // one-thread-per-env loop over global memory paid a load's latency every step: 128 steps x 256 envs
-// took 75.5 us with cold caches (23.8 us a call back to back), now 5.2 (about 9, the caller's share
-// included); 1024 x 4096 took 552 us, now 23.1.
-// Blocks of `size` that hold n >= 1 items (no sum that overflows at the largest n).
-__host__ __device__ constexpr int blocks_of(int n, int size) { return (n - 1) / size + 1; }
-static_assert(blocks_of(1, 64) == 1 && blocks_of(64, 64) == 1 && blocks_of(65, 64) == 2 && blocks_of(0x7fffffff, 64) == 1 << 25,
-              "blocks");
-
+// took 75.5 us with cold caches (23.7 us a call back to back, 34 alone), now 5.2 (3.5 back to back, 13
+// alone; 8 to 11 through the caller's tensors); 1024 x 4096 took 552 us, now 23.1.
 constexpr int kGaeT = 64;                 // steps per chunk
 constexpr int kGaeWarps = 8;
 constexpr int kGaeRows = kGaeT / kGaeWarps;  // steps of a chunk per warp
@@ -136,9 +136,9 @@ __global__ void __launch_bounds__(32 * kGaeWarps) gae_kernel(const float* r, con
 // flight; A floats per sample are then read at stride A), one sample per thread; the CTAs' sums meet in CTA
 // 0 over distributed shared memory in a fixed order, so no scratch memory is shared between
 // calls and repeated calls give identical results.  One CTA of 1024 threads walked all samples
-// before: 32768 x 7 took 41.3 us with cold caches (21.9 us a call back to back; one SM's share of bandwidth
-// and latency), now 7.6 (about 12, the caller's share included) on 16 CTAs; 1M samples x 7 took 1215 us,
-// now 111, the bandwidth of those 16 SMs.
+// before: 32768 x 7 took 41.3 us with cold caches (21.8 us a call back to back, 32 alone; one SM's share of
+// bandwidth and latency), now 7.6 (5.8 back to back, 16 alone; 11 to 14 through the caller's tensors) on 16
+// CTAs; 1M samples x 7 took 1215 us, now 111, the bandwidth of those 16 SMs.
 constexpr int kPpoTile = 512;   // samples per tile = threads
 constexpr int kPpoMaxA = 16;    // more tokens per sample are read in place (no staging)
 
