@@ -1729,14 +1729,15 @@ __global__ void __launch_bounds__(kThreads, 2)
   t.ml = ml;
   t.m0 = rank * ml;
   t.mn = max(0, min(ml, p.M - t.m0));
+  uint32_t gave_up;  // this CTA (final since the barrier above)
+  asm volatile("ld.shared.u32 %0, [%1];" : "=r"(gave_up) : "r"(smem_u32(tmem_slot + 1)) : "memory");
   cluster_wait();
-  const bool gave_up = *abort_flag != 0;
   if (warp == 0 && lane < C) {
-    // lane s sends rank s its rows.  A CTA that gave up sends nothing: the others' wait for its rows runs out
-    // too, and none of them stores the tile.
+    // lane s sends rank s its rows.  A CTA that gave up sends nothing and expects bytes that nobody sends: all
+    // waits for the sums run out, and no CTA of the cluster stores the tile.
     const int s = lane, n_s = min(ml, p.M - s * ml);
     if (s == rank) {
-      mbar_arrive_expect_tx(recv_bar, static_cast<uint32_t>((C - 1) * t.mn * TR * 4));
+      mbar_arrive_expect_tx(recv_bar, static_cast<uint32_t>((C - 1) * t.mn * TR * 4) + (gave_up ? 16u : 0u));
     } else if (n_s > 0 && !gave_up) {
       const int slot = rank - (rank > s ? 1 : 0);
       bulk_copy_cluster(mapa_shared(smem_u32(t.recv + slot * ml * TR), s), smem_u32(t.part + s * ml * TR),
@@ -1745,9 +1746,7 @@ __global__ void __launch_bounds__(kThreads, 2)
   }
   pdl_wait();  // (long over) the residual and the caches of this step are the previous kernels'
   uint32_t sat = 0;
-  gemv_finish<TR>(
-      p, t, tile,
-      [&] { return wait_drain_reported(recv_bar, 0, status, limit) && !gave_up; }, sat);
+  gemv_finish<TR>(p, t, tile, [&] { return wait_drain_reported(recv_bar, 0, status, limit); }, sat);
   report_saturation(status, sat);
   __syncwarp();
   cluster_arrive();
