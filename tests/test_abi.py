@@ -83,3 +83,13 @@ def test_host_argument_errors_without_gpu(lib):
     assert lib.vla_test_inject_launch_error(3, 0) == V.VLA_ERR_ARG
     assert lib.vla_test_inject_launch_error(0, 0) == V.VLA_OK
     assert lib.vla_test_set_wait_limit_ns(0) == V.VLA_OK
+
+
+def test_residual_gemm_and_cluster_hook_argument_errors(lib):
+    assert V.vla_op_gemm_resid_f16(0, 0, 0, 0, 0, 0, 384, 128, 4096) == V.VLA_ERR_ARG
+    assert "vla_op_gemm_resid_f16" in V.vla_last_error(None)
+    assert V.vla_op_gemm_resid_f16(16, 4096, 16, 4096, 16, 64, 384, 128, 4096) == V.VLA_ERR_ARG       # ldr < N
+    assert V.vla_op_gemm_resid_f16(16, 4096, 16, 4096, 16, 128, 384, 128, 4096, 16) == V.VLA_ERR_ARG  # norm without outputs
+    assert V.vla_op_gemm_resid_f16(16, 4096, 16, 4096, 16, 128, 256, 128, 4096) == V.VLA_ERR_UNSUPPORTED
+    assert V.vla_test_set_max_cluster(-1) == V.VLA_ERR_ARG
+    assert V.vla_test_set_max_cluster(0) == V.VLA_OK
